@@ -182,8 +182,9 @@ int pf_set_stencil(pf_grid_t g, int stencil);
  * k_steps (temporal-blocking depth, 2D only). 0 for any value = library default.
  * Unsupported combinations are rejected with PF_ERR_INVALID_ARG.
  * Supported: 2D tiles 64x16, 128x16, 32x32, 128x32; k in {1, 2, 4} (CH, C: {1, 2});
- * 3D tiles 32x16, 64x8 (general kernel, every model and size) and 64x16, 128x8, 128x16
- * (TMA-staged kernel: AC and GS with nx % tile_x == 0 and ny % tile_y == 0); k = 1;
+ * 3D tiles 32x16, 64x8 (general kernels, every model and size; with the 7-point stencil
+ * Allen-Cahn and Gray-Scott run two steps a launch, and a grid whose tuning was never set runs
+ * these too, whatever tile the default names) and 64x16, 128x8, 128x16 (TMA-staged kernel: AC and GS with nx % tile_x == 0 and ny % tile_y == 0); k = 1;
  * 3D k = 2 with tile nx x 8 (nx = 128 or 256; AC and GS).
  * 3D tile 32x8 selects the box kernel (Models B and C, k = 1 or 2, nx % 4 == 0, any ny and
  * nz): a CTA stages a whole 32 x 8 x 8 box with a halo of 2 k and runs k steps on regions that

@@ -227,6 +227,25 @@ int k1_tile(pf_grid_s* g, int tile) {
   return 0;
 }
 
+// Steps a launch of (tile, k) advances where the plan has that many left: k, except that the
+// general 3D tiles run Allen-Cahn and Gray-Scott with the 7-point stencil two steps at a time
+// (pf_fe3d_two.cu; the same bits as two single steps).
+int launch_depth(const pf_grid_s* g, int tile, int k) {
+  const bool pairs = g->dim == 3 && g->stencil == PF_ST_STD && tile < kFirstTmaTile3D && k == 1 &&
+                     (g->model == PF_MODEL_AC || g->model == PF_MODEL_GS);
+  return pairs ? 2 : k;
+}
+
+// The tile pf_step runs. Where a 3D grid's tuning is the library's own choice (nothing asked
+// for), the general tile's kernel takes the place of the depth-1 TMA tile that pf_get_tuning
+// names: it passes the TMA tiles wherever both run (256^3 GS 510 against 369 GLUPS, AC 816/716,
+// Model B 419/393, Model C 279/165; 64^3 GS 90/60, Model B 58/38), with the same bits.
+int run_tile(const pf_grid_s* g) {
+  const bool untuned = g->dim == 3 && g->stencil == PF_ST_STD && g->model != PF_MODEL_RD &&
+                       g->req_tile < 0 && g->req_k == 0;
+  return untuned ? 0 : g->tile;
+}
+
 // A kernel that gave up on a bounded wait leaves a flag; report it (and clear it).
 int check_device_error(pf_grid_s* g) {
   int flag = 0;
@@ -262,12 +281,15 @@ cudaError_t launch_step(pf_grid_s* g, int tile, int k, int src, int dst, cudaStr
   if (g->dim == 2) return launch_fe2d_stencil(g->stencil, g->model, tile, k, q, in, out, g->params, st);
   if (g->stencil != PF_ST_STD) return launch_fe3d(g->model, tile, q, in, out, g->params, st, g->stencil);
   if (tile == kTileBox3D) return launch_fe3d_box(g->model, k, q, in, out, g->params, st);
-  if (k == 2) {
+  if (k == 2 && tile >= kFirstTmaTile3D) {
     int tx, ty;
     tile3d_shape(tile, &tx, &ty);
     return launch_fe3d_tb2(g, tx, src, dst, st);
   }
   tile = k1_tile(g, tile);
+  const bool r2 = g->model == PF_MODEL_CH || g->model == PF_MODEL_C;
+  if (tile < kFirstTmaTile3D && (k == 2 || r2))
+    return launch_fe3d_two(g, src, dst, st);
   if (tile >= kFirstTmaTile3D) return launch_fe3d_tma(g, tile - kFirstTmaTile3D, src, dst, st);
   return launch_fe3d(g->model, tile, q, in, out, g->params, st);
 }
@@ -296,7 +318,8 @@ static int count_launches(int64_t n, int kmax) {
 }
 
 // Record the launches of pf_step(n) from buffer g->cur into a graph on the private stream.
-static int record_step_graph(pf_grid_s* g, int64_t n, cudaGraphExec_t* exec, int* flip) {
+static int record_step_graph(pf_grid_s* g, int tile, int depth, int64_t n,
+                             cudaGraphExec_t* exec, int* flip) {
   if (g->capture == nullptr)
     PF_CUDA_TRY(cudaStreamCreateWithFlags(&g->capture, cudaStreamNonBlocking));
   PF_CUDA_TRY(cudaStreamBeginCapture(g->capture, cudaStreamCaptureModeRelaxed));
@@ -304,9 +327,9 @@ static int record_step_graph(pf_grid_s* g, int64_t n, cudaGraphExec_t* exec, int
   int src = g->cur, launches = 0;
   int64_t left = n;
   while (left > 0 && e == cudaSuccess) {
-    int k = g->k;
+    int k = depth;
     while (k > left) k >>= 1;
-    e = launch_step(g, g->tile, k, src, 1 - src, g->capture);
+    e = launch_step(g, tile, k, src, 1 - src, g->capture);
     src = 1 - src;
     left -= k;
     ++launches;
@@ -577,12 +600,14 @@ int pf_step(pf_grid_t g, int64_t n_steps) {
     g->cur = 1 - g->cur;
     return PF_OK;
   }
-  if (count_launches(n_steps, g->k) >= kGraphMinLaunches) {
+  const int tile = run_tile(g);
+  const int depth = launch_depth(g, tile, g->k);
+  if (count_launches(n_steps, depth) >= kGraphMinLaunches) {
     // replay a recorded graph of the whole launch sequence (one host call)
     pf_grid_s::StepGraph* hit = nullptr;
     pf_grid_s::StepGraph* victim = &g->step_graphs[0];
     for (auto& sg : g->step_graphs) {
-      if (sg.exec && sg.steps == n_steps && sg.tile == g->tile && sg.k == g->k &&
+      if (sg.exec && sg.steps == n_steps && sg.tile == tile && sg.k == g->k &&
           sg.start == g->cur)
         hit = &sg;
       if (sg.used < victim->used) victim = &sg;
@@ -590,9 +615,9 @@ int pf_step(pf_grid_t g, int64_t n_steps) {
     if (hit == nullptr) {
       if (victim->exec) cudaGraphExecDestroy(victim->exec);
       *victim = pf_grid_s::StepGraph();
-      if (int rc = record_step_graph(g, n_steps, &victim->exec, &victim->flip)) return rc;
+      if (int rc = record_step_graph(g, tile, depth, n_steps, &victim->exec, &victim->flip)) return rc;
       victim->steps = n_steps;
-      victim->tile = g->tile;
+      victim->tile = tile;
       victim->k = g->k;
       victim->start = g->cur;
       hit = victim;
@@ -604,9 +629,9 @@ int pf_step(pf_grid_t g, int64_t n_steps) {
   }
   int64_t left = n_steps;
   while (left > 0) {
-    int k = g->k;
+    int k = depth;
     while (k > left) k >>= 1;  // k in {4, 2, 1}
-    PF_CUDA_TRY(launch_step(g, g->tile, k, g->cur, 1 - g->cur, g->stream));
+    PF_CUDA_TRY(launch_step(g, tile, k, g->cur, 1 - g->cur, g->stream));
     g->cur = 1 - g->cur;
     left -= k;
   }
@@ -803,6 +828,9 @@ int pf_autotune(pf_grid_t g, int probe_launches, int* tile_x, int* tile_y, int* 
     for (int ki = 0; ki < 4 && rc == PF_OK; ++ki) {
       const int k = ks[ki];
       if (!tile_supported(g, t, k)) continue;
+      // the two general 3D tiles run the same kernel with the 7-point stencil
+      if (g->dim == 3 && t == 1 && g->stencil == PF_ST_STD) continue;
+      const int depth = launch_depth(g, t, k);
       // the cluster and band kernels run a whole pf_step in one launch: probe them that way
       const bool cluster = g->dim == 2 && (t == kTileCluster2D || t == kTileBands2D);
       const int64_t probe_steps = cluster ? (int64_t)probe_launches * k * 16 : 0;
@@ -810,7 +838,7 @@ int pf_autotune(pf_grid_t g, int probe_launches, int* tile_x, int* tile_y, int* 
       // Tiled candidates run as a replayed graph of n_l launches, as pf_step runs them.
       const int n_l = probe_launches > 8 ? probe_launches : 8;
       cudaGraphExec_t probe = nullptr;
-      cudaError_t e = launch_step(g, t, k, g->cur, 1 - g->cur, g->stream);  // warm-up
+      cudaError_t e = launch_step(g, t, depth, g->cur, 1 - g->cur, g->stream);  // warm-up
       if (cluster && (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources)) {
         // the on-chip kernels need all their CTAs resident at once; where the device cannot
         // host them now (other work, a restricted context), they are not candidates
@@ -824,7 +852,7 @@ int pf_autotune(pf_grid_t g, int probe_launches, int* tile_x, int* tile_y, int* 
         if (e == cudaSuccess) {
           cudaError_t el = cudaSuccess;
           for (int i = 0; i < n_l && el == cudaSuccess; ++i)
-            el = launch_step(g, t, k, g->cur, 1 - g->cur, g->capture);
+            el = launch_step(g, t, depth, g->cur, 1 - g->cur, g->capture);
           cudaGraph_t graph = nullptr;
           e = cudaStreamEndCapture(g->capture, &graph);
           if (e == cudaSuccess) e = el;
@@ -856,7 +884,7 @@ int pf_autotune(pf_grid_t g, int probe_launches, int* tile_x, int* tile_y, int* 
         rc = cuda_fail(e, "pf_autotune probe");
         break;
       }
-      const float per_step = cluster ? ms / probe_steps : ms / ((float)n_l * k);
+      const float per_step = cluster ? ms / probe_steps : ms / ((float)n_l * depth);
       if (per_step < best) {
         best = per_step;
         best_tile = t;

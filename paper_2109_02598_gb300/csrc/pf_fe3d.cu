@@ -410,9 +410,13 @@ cudaError_t launch3_tile(int tile_id, const Geom& g, FieldPtrs in, FieldOut out,
     if (tile_id == 0) return launch3<MODEL, 32, 16, PF_ST_ISO27>(g, in, out, m, s);
     return launch3<MODEL, 64, 8, PF_ST_ISO27>(g, in, out, m, s);
   }
-  if (stencil != PF_ST_STD) return cudaErrorInvalidValue;
-  if (tile_id == 0) return launch3<MODEL, 32, 16, PF_ST_STD>(g, in, out, m, s);
-  return launch3<MODEL, 64, 8, PF_ST_STD>(g, in, out, m, s);
+  // 7-point: a single step of Allen-Cahn and Gray-Scott (pairs of steps, and Models B and C,
+  // run in pf_fe3d_two.cu)
+  if constexpr (ModelTraits<MODEL>::R == 1) {
+    if (stencil == PF_ST_STD && tile_id == 0) return launch3<MODEL, 32, 16, PF_ST_STD>(g, in, out, m, s);
+    if (stencil == PF_ST_STD) return launch3<MODEL, 64, 8, PF_ST_STD>(g, in, out, m, s);
+  }
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace

@@ -14,13 +14,13 @@
 // bitwise identical to two depth-1 steps.
 //
 // Requires nx == W, ny % TY == 0 and ny >= 2.
+#include "pf_fe3d_tb.cuh"
 #include "pf_grid.h"
 #include "pf_internal.h"
 #include "pf_tma.cuh"
 
 #include <cudaTypedefs.h>
 
-#include <algorithm>
 #include <type_traits>
 
 namespace pf {
@@ -76,56 +76,6 @@ __device__ __forceinline__ void x_edges_c(const float* row, int x4, const float4
   xm = lane == 0 ? em : wm;
   xp = lane == 31 ? ep : wp;
 }
-
-template <int MODEL>
-__device__ __forceinline__ void update4(const float4* c, const float4* lap, float4* res,
-                                        const ModelParams& m) {
-  if constexpr (MODEL == PF_MODEL_AC) {
-    res[0].x = ac_update(c[0].x, lap[0].x, m);
-    res[0].y = ac_update(c[0].y, lap[0].y, m);
-    res[0].z = ac_update(c[0].z, lap[0].z, m);
-    res[0].w = ac_update(c[0].w, lap[0].w, m);
-  } else {
-    gs_update(c[0].x, c[1].x, lap[0].x, lap[1].x, m, res[0].x, res[1].x);
-    gs_update(c[0].y, c[1].y, lap[0].y, lap[1].y, m, res[0].y, res[1].y);
-    gs_update(c[0].z, c[1].z, lap[0].z, lap[1].z, m, res[0].z, res[1].z);
-    gs_update(c[0].w, c[1].w, lap[0].w, lap[1].w, m, res[0].w, res[1].w);
-  }
-}
-
-// 7-point Laplacians of four sites: centre c, z-neighbours zm/zp, rows above/below and the
-// two x-edge scalars of the centre row. Gray-Scott's stencil factor is carried in D_u and D_v
-// (its lap_scale is 1), so its final multiply is left out, as lap_scaled does: the same bits,
-// eight instructions fewer per float4 and level (GS 256^3: 503 -> 521 GLUPS). The sums run as
-// packed FP32 pairs (lap3d_sum4: lap3d_sum's operations in its order, each lane's bits
-// unchanged) while the update stays scalar, which splits the arithmetic between the heavy FMA
-// pipe (the pairs) and both pipes (the scalars): GS 256^3 558 -> 596 GLUPS. Packing the
-// update too loads the heavy pipe alone (measured slower before this change).
-template <int MODEL>
-__device__ __forceinline__ float4 lap3d_x4(const float4& c, const float4& ym, const float4& yp,
-                                           const float4& zm, const float4& zp, float xm,
-                                           float xp, float lap_scale) {
-  float4 l = lap3d_sum4(c, xm, xp, ym, yp, zm, zp);
-  if constexpr (MODEL != PF_MODEL_GS) l = mul4(lap_scale, l);  // lap_scaled
-  return l;
-}
-
-// How the (row tile, plane) work is split over the CTAs (chosen on the host, tb2_schedule).
-//   ITEMS:    item = (tile, chunk of chunk_len planes), items dealt round-robin over the CTAs,
-//             chunks alternating up and down in z.
-//   BALANCED: the (tile, plane) units in tile-major order cut into gridDim.x equal ranges,
-//             one per CTA (a range crossing a tile boundary makes two segments), direction
-//             alternating by CTA.
-//   ROWS:     full_rows rows of one CTA per tile, row c streaming planes [c L, (c+1) L) in
-//             the direction of chunk c; the remaining CTAs split the top row [full_rows L, nz)
-//             of every tile in tile-major order. CTAs of neighbouring tiles in a full row work
-//             on the same plane at the same time, so the halo rows they share come from L2.
-struct Tb2Sched {
-  int mode;
-  int nchunks, chunk_len;    // ITEMS
-  int full_rows, L, pdir;    // ROWS: rows of ncols CTAs, their chunk length, partial direction
-};
-constexpr int kTb2Items = 0, kTb2Balanced = 1, kTb2Rows = 2;
 
 // Per-thread state of one z-stream: z-windows of the input planes (level 1's z-neighbours and
 // centre) and of the first-level planes (level 2's), three slots each, slot = plane mod 3, so
@@ -397,61 +347,6 @@ __global__ void __launch_bounds__(CfgB<MODEL, W, TY, NS, V_>::NT, 1)
         (void)mbar_wait_bounded(&bars[q % NS], (q / NS) & 1u, kWaitBudgetCycles);
     }
   }
-}
-
-// The work split with the shortest longest-CTA plane count (each segment streams 4 halo
-// planes besides its own), ROWS preferred when it is within one plane of the best, since it
-// keeps neighbouring tiles in step over z.
-Tb2Sched tb2_schedule(int ncols, int nz, long long slots, long long* grid_out) {
-  Tb2Sched s{};
-  // ITEMS
-  long long nchunks = slots / ncols;
-  if (nchunks > nz / 4) nchunks = nz / 4;
-  if (nchunks < 1) nchunks = 1;
-  const int chunk_len = (int)((nz + nchunks - 1) / nchunks);
-  nchunks = (nz + chunk_len - 1) / chunk_len;
-  const long long items = (long long)ncols * nchunks;
-  const long long item_grid = items < slots ? items : slots;
-  const long long item_span = (items + item_grid - 1) / item_grid * (chunk_len + 4);
-  // BALANCED: about units / slots + 8 planes (two segments at most when a range is under nz)
-  const long long units = (long long)ncols * nz;
-  const long long per = (units + slots - 1) / slots;
-  const long long bal_span = per + (per < nz ? 8 : 4 * ((per + nz - 1) / nz + 1));
-  const long long bal_grid = slots < units ? slots : units;
-  // ROWS
-  long long rows_span = -1, rows_L = 0;
-  const long long F = slots / ncols, R = slots - F * ncols;
-  for (long long L = 4; F >= 1 && L * F <= nz; ++L) {
-    const long long Lp = nz - F * L;  // planes of the top row
-    long long span = L + 4;
-    if (Lp > 0) {
-      if (R == 0) continue;
-      const long long pu = ((long long)ncols * Lp + R - 1) / R;
-      const long long segs = (pu + Lp - 1) / Lp + 1;
-      span = std::max(span, pu + 4 * segs);
-    }
-    if (rows_span < 0 || span < rows_span) {
-      rows_span = span;
-      rows_L = L;
-    }
-  }
-  const long long best = std::min(item_span, slots > item_grid ? bal_span : item_span);
-  if (rows_span > 0 && rows_span <= best + 1) {
-    s.mode = kTb2Rows;
-    s.full_rows = (int)F;
-    s.L = (int)rows_L;
-    s.pdir = ((F - 1) & 1) ? 1 : -1;  // meet the last full row's chunk at its end
-    *grid_out = (nz - F * rows_L) > 0 ? slots : F * ncols;
-  } else if (bal_span < item_span && slots > item_grid) {
-    s.mode = kTb2Balanced;
-    *grid_out = bal_grid;
-  } else {
-    s.mode = kTb2Items;
-    *grid_out = item_grid;
-  }
-  s.nchunks = (int)nchunks;
-  s.chunk_len = chunk_len;
-  return s;
 }
 
 template <int MODEL, int W, int TY, int NS, int V = 1>

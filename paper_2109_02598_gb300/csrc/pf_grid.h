@@ -51,6 +51,39 @@ struct Tb2Cache {
   Tb2Maps maps[2];
 };
 
+// How the (row tile, plane) work is split over the CTAs (chosen on the host, tb2_schedule).
+//   ITEMS:    item = (tile, chunk of chunk_len planes), items dealt round-robin over the CTAs,
+//             chunks alternating up and down in z.
+//   BALANCED: the (tile, plane) units in tile-major order cut into gridDim.x equal ranges,
+//             one per CTA (a range crossing a tile boundary makes two segments), direction
+//             alternating by CTA.
+//   ROWS:     full_rows rows of one CTA per tile, row c streaming planes [c L, (c+1) L) in
+//             the direction of chunk c; the remaining CTAs split the top row [full_rows L, nz)
+//             of every tile in tile-major order. CTAs of neighbouring tiles in a full row work
+//             on the same plane at the same time, so the halo rows they share come from L2.
+struct Tb2Sched {
+  int mode;
+  int nchunks, chunk_len;    // ITEMS
+  int full_rows, L, pdir;    // ROWS: rows of ncols CTAs, their chunk length, partial direction
+};
+constexpr int kTb2Items = 0, kTb2Balanced = 1, kTb2Rows = 2;
+
+// Tiles of the two-level 3D kernel (pf_fe3d_two.cu), chosen on the host (two_plan).
+struct TwoTiles {
+  int G;      // groups of four columns per row
+  int TY;     // output rows per tile
+  int lpad;   // staged columns left of the strip: 0 (full periodic rows) or 4
+  int S, w;   // strips and output columns per strip (the last may be narrower)
+};
+
+// They depend on the grid's sides only, so a handle keeps them.
+struct TwoPlan {
+  bool valid = false;
+  TwoTiles tiles{};
+  Tb2Sched sched{};
+  unsigned grid = 0;
+};
+
 constexpr uint32_t kGridMagic = 0x50464744u;  // "PFGD"
 
 struct AdjointState {
@@ -107,6 +140,7 @@ struct pf_grid_s {
   pf::TmaCache tma;
   pf::Tma2Cache tma2;
   pf::Tb2Cache tb2;
+  pf::TwoPlan two;
   int* d_err = nullptr;  // set by a kernel whose bounded wait ran out
   // band kernel (2D grid resident in the SMs' shared memory): exchange slots of the bands'
   // edge rows as tagged 64-bit words, allocated at its first launch, and the last tag used
@@ -153,6 +187,10 @@ cudaError_t launch_fe3d_tma_r2(pf_grid_s* g, int tma_tile, int src, int dst, cud
 // cooperative launch (pf_fe2d_bands.cu)
 cudaError_t launch_fe2d_bands(pf_grid_s* g, int src, int dst, int64_t n_steps, cudaStream_t st);
 void fe2d_bands_release(pf_grid_s* g);
+
+// The general 3D tiles with the 7-point stencil (any size): two steps a launch for AC and GS,
+// one for Models B and C (pf_fe3d_two.cu)
+cudaError_t launch_fe3d_two(pf_grid_s* g, int src, int dst, cudaStream_t st);
 
 // ---- 3D depth-2 kernel (AC, GS; full x-rows of 128 or 256, 8-row tiles)
 bool fe3d_tb2_supported(int model, int tx, int ty, const Geom& g);
