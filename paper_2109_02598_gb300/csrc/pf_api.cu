@@ -246,12 +246,19 @@ int run_tile(const pf_grid_s* g) {
   return untuned ? 0 : g->tile;
 }
 
+int sync_device_error(pf_grid_s* g);
+
 // A kernel that gave up on a bounded wait leaves a flag; report it (and clear it).
 int check_device_error(pf_grid_s* g) {
-  int flag = 0;
-  PF_CUDA_TRY(cudaMemcpyAsync(&flag, g->d_err, sizeof(int), cudaMemcpyDeviceToHost, g->stream));
+  PF_CUDA_TRY(cudaMemcpyAsync(g->err_host(), g->d_err, sizeof(int), cudaMemcpyDeviceToHost,
+                              g->stream));
+  return sync_device_error(g);
+}
+
+// The same where the work enqueued so far leaves the error word in err_host().
+int sync_device_error(pf_grid_s* g) {
   PF_CUDA_TRY(cudaStreamSynchronize(g->stream));
-  if (flag != 0) {
+  if (*g->err_host() != 0) {
     PF_CUDA_TRY(cudaMemsetAsync(g->d_err, 0, sizeof(int), g->stream));
     set_error("a kernel's bounded wait (for a TMA copy or a neighbouring band) ran out; the "
               "state is invalid");
@@ -404,8 +411,8 @@ int pf_create_grid(int dim, const int64_t* n, int n_fields, double h, void* stre
   cudaError_t e = cudaGetDevice(&g->device);
   if (e == cudaSuccess) e = cudaMalloc(&g->base, sizeof(float) * elems * 2 * n_fields);
   if (e == cudaSuccess) e = cudaMemsetAsync(g->base, 0, sizeof(float) * elems * 2 * n_fields, g->stream);
-  if (e == cudaSuccess) e = cudaMalloc(&g->red_partials, sizeof(double) * (kReduceBlocks + 1));
-  if (e == cudaSuccess) e = cudaMallocHost(&g->red_host, sizeof(double));
+  if (e == cudaSuccess) e = cudaMalloc(&g->red_partials, sizeof(double) * kReduceBlocks);
+  if (e == cudaSuccess) e = cudaMallocHost(&g->red_host, 2 * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&g->d_err, sizeof(int));
   if (e == cudaSuccess) e = cudaMemsetAsync(g->d_err, 0, sizeof(int), g->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
@@ -654,17 +661,16 @@ int pf_reduce(pf_grid_t g, int what, int field, double* out) {
     c1 = g->coeffs[0];
     c2 = g->coeffs[1];
   }
+  // the last kernel writes the sum and the device error word to pinned host memory
   if (what == PF_REDUCE_ENERGY && g->model == PF_MODEL_C) {
     PF_CUDA_TRY(launch_reduce_energy_c(grid_geom(g), g->buf[g->cur][0], g->buf[g->cur][1],
-                                       g->coeffs, g->h, g->red_partials,
-                                       g->red_partials + kReduceBlocks, g->stream));
+                                       g->coeffs, g->h, g->red_partials, g->red_host, g->stream,
+                                       g->d_err, g->err_host()));
   } else {
     PF_CUDA_TRY(launch_reduce(what, grid_geom(g), g->buf[g->cur][field], c1, c2, g->h,
-                              g->red_partials, g->red_partials + kReduceBlocks, g->stream));
+                              g->red_partials, g->red_host, g->stream, g->d_err, g->err_host()));
   }
-  PF_CUDA_TRY(cudaMemcpyAsync(g->red_host, g->red_partials + kReduceBlocks, sizeof(double),
-                              cudaMemcpyDeviceToHost, g->stream));
-  if (int rc = check_device_error(g)) return rc;
+  if (int rc = sync_device_error(g)) return rc;
   *out = *g->red_host;
   if (!std::isfinite(*out)) {
     set_error("reduction is not finite (%g): the state has blown up", *out);

@@ -134,8 +134,11 @@ struct pf_grid_s {
   int k = 0;          // temporal-blocking depth in effect
   int req_tile = -1;  // tile asked for by pf_set_tuning (-1 = library default)
   int req_k = 0;      // depth asked for (0 = library default)
-  double* red_partials = nullptr;  // kReduceBlocks partials + 1 result
-  double* red_host = nullptr;      // pinned
+  double* red_partials = nullptr;  // kReduceBlocks partials
+  // pinned host words that kernels and copies write: a reduction's result and, behind it, the
+  // device error word
+  double* red_host = nullptr;
+  int* err_host() const { return reinterpret_cast<int*>(red_host + 1); }
   pf::AdjointState adj;
   pf::TmaCache tma;
   pf::Tma2Cache tma2;

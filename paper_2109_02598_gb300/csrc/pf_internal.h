@@ -164,13 +164,16 @@ cudaError_t launch_batch_gs2d(int tile_id, int k, const BatchInst* d_insts,
                               float* out_base, cudaStream_t s);
 
 // ---- reductions -------------------------------------------------------------------
-// Writes one double to d_out. d_partials must hold kReduceBlocks doubles.
+// Writes one double to d_out (device memory, or mapped host memory); d_partials must hold
+// kReduceBlocks doubles. d_err / err_out (optional): a device word copied out beside it.
 constexpr int kReduceBlocks = 512;
 cudaError_t launch_reduce(int what, const Geom& g, const float* field, double c1, double c2,
-                          double h, double* d_partials, double* d_out, cudaStream_t s);
+                          double h, double* d_partials, double* d_out, cudaStream_t s,
+                          const int* d_err = nullptr, int* err_out = nullptr);
 // Model C free energy of (psi, m) with coefficients c[0..4] = c1..c5.
 cudaError_t launch_reduce_energy_c(const Geom& g, const float* psi, const float* m,
                                    const double* c, double h, double* d_partials,
-                                   double* d_out, cudaStream_t s);
+                                   double* d_out, cudaStream_t s, const int* d_err = nullptr,
+                                   int* err_out = nullptr);
 
 }  // namespace pf
