@@ -25,13 +25,17 @@
 //     4-byte copies, one or two per thread, of the columns the levels read.
 //
 // What bounds it (two time steps of Gray-Scott, 256^3, 640 threads, one CTA per SM): issue and
-// the latencies behind the plane barrier; a plane takes 0.37 us + 0.035 us per warp. Measured
+// the latencies behind the plane barrier; a plane takes 0.37 us + 0.035 us per warp. GLUPS
 // against the general kernels it replaces (32x16 tiles, 4-byte copies or one plane in flight):
-// GS 210x179x150 362 against 191 GLUPS, 160^3 409/197, 100x90x110 203/95; AC 210x179x150
-// 573/301; Model B 293/102; Model C 194/88, 256^3 279/110 (TMA tiles 165). NS = 5 planes leave
-// three in flight over a plane's 1.1 us. 640 threads: with 768 (80 registers) GS 256^3 gains
-// 3 %, but AC, Models B and C lose 1 to 10 %; two CTAs of 320 threads per SM lose 17 % there
-// (shorter tiles, more halo) and gain 2 to 5 % only below 100^3.
+// GS 210x179x150 380 / 191, 256^3 540 / 200; AC 210x179x150 599 / 301, 256^3 870 / 376; Model B
+// 315 / 102 and 458 / 134; Model C 207 / 88 and 302 / 110 (TMA tiles, 256^3: 369, 716, 393,
+// 165). NS = 5 planes leave three in flight over a plane's 1.1 us (4 and 6 measured the same).
+// 640 threads: with 768 (80 registers) GS 256^3 gains 3 %, but AC, Models B and C lose 1 to
+// 10 %; two CTAs of 320 threads per SM lose 17 % there (shorter tiles, more halo) and gain 2 to
+// 5 % only below 100^3. The next plane's index and the output offset advance instead of being
+// computed from j (+5 to 8 %); the ring slots do not (offsets kept instead of slot numbers cost
+// Gray-Scott 13 %, the compiler then reloading them), and level 2's rows are read after level 1
+// (before it: 1 to 4 % slower).
 #include "pf_fe3d_tb.cuh"
 #include "pf_grid.h"
 #include "pf_tma.cuh"
@@ -260,8 +264,12 @@ __global__ void __launch_bounds__(kTwoThreads, 1)
     if (tid < nitems) scalar_item(tid, sf, ssrc, sdst);
     const float* sbase = sf == 0 ? in.f[0] : in.f[NF - 1];
 
-    auto stage = [&](int i, int slot) {  // input plane i of the segment into ring slot `slot`
-      const int64_t zo = (int64_t)wrap_index(zfirst + (i - 2) * dir, g.nz) * g.plane;
+    int zin = wrap_index(zfirst - 2 * dir, g.nz);  // the next input plane to stage
+    auto stage = [&](int slot) {                   // it into ring slot `slot`; advances zin
+      const int64_t zo = (int64_t)zin * g.plane;
+      zin += dir;
+      if (zin == g.nz) zin = 0;
+      if (zin < 0) zin = g.nz - 1;
       float* st = ring + slot * C::IN_STAGE;
       if (src_a >= 0) {
 #pragma unroll
@@ -288,12 +296,13 @@ __global__ void __launch_bounds__(kTwoThreads, 1)
     const int gy = y0 + r - 1, gx = x0 - pl.lpad + 4 * q;
     const bool store = live && inner && gy < g.ny && gx >= x0 && gx < x1;
     const bool whole = gx + 3 < x1;
-    const int64_t off0 = (int64_t)gy * g.pitch + gx;
+    int64_t off = (int64_t)zfirst * g.plane + (int64_t)gy * g.pitch + gx;
+    const int64_t off_step = dir > 0 ? g.plane : -g.plane;
 
     __syncthreads();  // every thread is done with the last segment's planes
 #pragma unroll
     for (int i = 0; i < NS; ++i) {
-      if (i < nin) stage(i, i);
+      if (i < nin) stage(i);
       cp_async_commit();
     }
     cp_async_wait_group<NS - 2>();  // input planes 0 and 1
@@ -309,7 +318,7 @@ __global__ void __launch_bounds__(kTwoThreads, 1)
       constexpr int P = decltype(phase)::value;
       cp_async_wait_group<NS - 3>();  // input plane j + 2 has landed
       __syncthreads();                // ... for every thread, and plane j's slot is free
-      if (j + NS < nin) stage(j + NS, s0);
+      if (j + NS < nin) stage(s0);
       cp_async_commit();  // possibly empty: one group per iteration
       float* l1w = l1 + (j & 1) * C::L1_PLANE + o1;
       const float* l1r = l1 + ((j + 1) & 1) * C::L1_PLANE + o1;
@@ -323,7 +332,6 @@ __global__ void __launch_bounds__(kTwoThreads, 1)
         float4 res[NF];
         zs.template level2<P>(l1r, ym2, yp2, t, m, res);
         if (store) {
-          const int64_t off = (int64_t)(zfirst + (j - 2) * dir) * g.plane + off0;
           if (whole) {
 #pragma unroll
             for (int f = 0; f < NF; ++f) *reinterpret_cast<float4*>(out.f[f] + off) = res[f];
@@ -337,6 +345,7 @@ __global__ void __launch_bounds__(kTwoThreads, 1)
           }
         }
       }
+      if (j >= 2) off += off_step;
       if constexpr (MODEL == PF_MODEL_C) zs.lpsi = lpsi_next;
     };
     const int nj = n + 2;
