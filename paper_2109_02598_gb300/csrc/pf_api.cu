@@ -278,7 +278,8 @@ cudaError_t launch_step(pf_grid_s* g, int tile, int k, int src, int dst, cudaStr
     out.f[f] = g->buf[dst][f];
   }
   const Geom q = grid_geom(g);
-  if (g->model == PF_MODEL_RD) return launch_rd(q, g->nf, in, out, g->rd, st);
+  if (g->model == PF_MODEL_RD && g->dim == 2) return launch_rd2d(q, g->nf, in, out, g->rd, st);
+  if (g->model == PF_MODEL_RD) return launch_fe3d_one(g, src, dst, st);
   if (g->dim == 2 && tile == kTileCluster2D)
     return launch_fe2d_cluster(g->model, k, q, in, out, g->params, k, st);
   if (g->dim == 2 && tile == kTileBands2D) return launch_fe2d_bands(g, src, dst, k, st);
@@ -286,7 +287,10 @@ cudaError_t launch_step(pf_grid_s* g, int tile, int k, int src, int dst, cudaStr
     return launch_fe2d_strips(g->model, g->stencil, tile == kTileStrips2D ? 128 : 64, k, q, in,
                               out, g->params, st);
   if (g->dim == 2) return launch_fe2d_stencil(g->stencil, g->model, tile, k, q, in, out, g->params, st);
-  if (g->stencil != PF_ST_STD) return launch_fe3d(g->model, tile, q, in, out, g->params, st, g->stencil);
+  const bool r2 = g->model == PF_MODEL_CH || g->model == PF_MODEL_C;
+  if (g->stencil != PF_ST_STD)
+    return r2 ? launch_fe3d(g->model, tile, q, in, out, g->params, st, g->stencil)
+              : launch_fe3d_one(g, src, dst, st);
   if (tile == kTileBox3D) return launch_fe3d_box(g->model, k, q, in, out, g->params, st);
   if (k == 2 && tile >= kFirstTmaTile3D) {
     int tx, ty;
@@ -294,11 +298,8 @@ cudaError_t launch_step(pf_grid_s* g, int tile, int k, int src, int dst, cudaStr
     return launch_fe3d_tb2(g, tx, src, dst, st);
   }
   tile = k1_tile(g, tile);
-  const bool r2 = g->model == PF_MODEL_CH || g->model == PF_MODEL_C;
-  if (tile < kFirstTmaTile3D && (k == 2 || r2))
-    return launch_fe3d_two(g, src, dst, st);
   if (tile >= kFirstTmaTile3D) return launch_fe3d_tma(g, tile - kFirstTmaTile3D, src, dst, st);
-  return launch_fe3d(g->model, tile, q, in, out, g->params, st);
+  return k == 2 || r2 ? launch_fe3d_two(g, src, dst, st) : launch_fe3d_one(g, src, dst, st);
 }
 
 // Forget every recorded graph (their kernel parameters carry coefficients and tuning).
@@ -488,6 +489,7 @@ int set_model_rd(pf_grid_s* g, const double* c, int n_coeffs, double dt, int for
     for (int j = 0; j < N; ++j) packed |= ((int)E[m * N + j]) << (2 * j);
     p.E[m] = packed;
   }
+  rd_places(N, p);
   for (int i = 0; i < N; ++i) {
     p.D[i] = (float)(c[i] / (g->h * g->h));
     for (int m = 0; m < M; ++m) p.K[i][m] = (float)K[i * M + m];
@@ -834,8 +836,11 @@ int pf_autotune(pf_grid_t g, int probe_launches, int* tile_x, int* tile_y, int* 
     for (int ki = 0; ki < 4 && rc == PF_OK; ++ki) {
       const int k = ks[ki];
       if (!tile_supported(g, t, k)) continue;
-      // the two general 3D tiles run the same kernel with the 7-point stencil
-      if (g->dim == 3 && t == 1 && g->stencil == PF_ST_STD) continue;
+      // the two general 3D tiles run the same kernel, but for Models B and C with the 19- and
+      // 27-point stencils
+      if (g->dim == 3 && t == 1 &&
+          (g->stencil == PF_ST_STD || g->model == PF_MODEL_AC || g->model == PF_MODEL_GS))
+        continue;
       const int depth = launch_depth(g, t, k);
       // the cluster and band kernels run a whole pf_step in one launch: probe them that way
       const bool cluster = g->dim == 2 && (t == kTileCluster2D || t == kTileBands2D);

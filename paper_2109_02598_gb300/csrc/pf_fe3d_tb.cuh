@@ -43,11 +43,11 @@ __device__ __forceinline__ float4 lap3d_x4(const float4& c, const float4& ym, co
   return l;
 }
 
-// The work split with the shortest longest-CTA plane count (each segment streams 4 halo
-// planes besides its own), ROWS preferred when it is within one plane of the best, since it
+// The work split with the shortest longest-CTA plane count (each segment streams `halo` planes
+// besides its own), ROWS preferred when it is within one plane of the best, since it
 // keeps neighbouring tiles in step over z. span_out: the longest CTA's plane count.
 inline Tb2Sched tb2_schedule(int ncols, int nz, long long slots, long long* grid_out,
-                             long long* span_out = nullptr) {
+                             long long* span_out = nullptr, int halo = 4) {
   Tb2Sched s{};
   // ITEMS
   long long nchunks = slots / ncols;
@@ -57,23 +57,23 @@ inline Tb2Sched tb2_schedule(int ncols, int nz, long long slots, long long* grid
   nchunks = (nz + chunk_len - 1) / chunk_len;
   const long long items = (long long)ncols * nchunks;
   const long long item_grid = items < slots ? items : slots;
-  const long long item_span = (items + item_grid - 1) / item_grid * (chunk_len + 4);
+  const long long item_span = (items + item_grid - 1) / item_grid * (chunk_len + halo);
   // BALANCED: about units / slots + 8 planes (two segments at most when a range is under nz)
   const long long units = (long long)ncols * nz;
   const long long per = (units + slots - 1) / slots;
-  const long long bal_span = per + (per < nz ? 8 : 4 * ((per + nz - 1) / nz + 1));
+  const long long bal_span = per + (per < nz ? 2 * halo : halo * ((per + nz - 1) / nz + 1));
   const long long bal_grid = slots < units ? slots : units;
   // ROWS
   long long rows_span = -1, rows_L = 0;
   const long long F = slots / ncols, R = slots - F * ncols;
   for (long long L = 4; F >= 1 && L * F <= nz; ++L) {
     const long long Lp = nz - F * L;  // planes of the top row
-    long long span = L + 4;
+    long long span = L + halo;
     if (Lp > 0) {
       if (R == 0) continue;
       const long long pu = ((long long)ncols * Lp + R - 1) / R;
       const long long segs = (pu + Lp - 1) / Lp + 1;
-      span = std::max(span, pu + 4 * segs);
+      span = std::max(span, pu + halo * segs);
     }
     if (rows_span < 0 || span < rows_span) {
       rows_span = span;

@@ -27,18 +27,17 @@
 // What bounds it (two time steps of Gray-Scott, 256^3, 640 threads, one CTA per SM): issue and
 // the latencies behind the plane barrier; a plane takes 0.37 us + 0.035 us per warp. GLUPS
 // against the general kernels it replaces (32x16 tiles, 4-byte copies or one plane in flight):
-// GS 210x179x150 380 / 191, 256^3 540 / 200; AC 210x179x150 599 / 301, 256^3 870 / 376; Model B
-// 315 / 102 and 458 / 134; Model C 207 / 88 and 302 / 110 (TMA tiles, 256^3: 369, 716, 393,
+// GS 210x179x150 386 / 191, 256^3 572 / 200; AC 210x179x150 648 / 301, 256^3 979 / 376; Model B
+// 335 / 102 and 520 / 134; Model C 213 / 88 and 317 / 110 (TMA tiles, 256^3: 369, 716, 393,
 // 165). NS = 5 planes leave three in flight over a plane's 1.1 us (4 and 6 measured the same).
 // 640 threads: with 768 (80 registers) GS 256^3 gains 3 %, but AC, Models B and C lose 1 to
 // 10 %; two CTAs of 320 threads per SM lose 17 % there (shorter tiles, more halo) and gain 2 to
-// 5 % only below 100^3. The next plane's index and the output offset advance instead of being
-// computed from j (+5 to 8 %); the ring slots do not (offsets kept instead of slot numbers cost
-// Gray-Scott 13 %, the compiler then reloading them), and level 2's rows are read after level 1
-// (before it: 1 to 4 % slower).
-#include "pf_fe3d_tb.cuh"
+// 5 % only below 100^3. The copies' pointer and the output offset advance from plane to plane
+// (+5 to 13 % over computing them from j); the ring slots do not (offsets kept instead of slot
+// numbers cost Gray-Scott 13 %, the compiler then reloading them), and level 2's rows are read
+// after level 1 (before it: 1 to 4 % slower).
+#include "pf_fe3d_stream.cuh"
 #include "pf_grid.h"
-#include "pf_tma.cuh"
 
 #include <type_traits>
 
@@ -63,23 +62,6 @@ struct CfgTwo {
   static constexpr size_t SMEM = (size_t)(NS * IN_STAGE + 2 * L1_PLANE) * 4;
 };
 
-__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
-
-// A thread's place: its group's offset in a row-major plane of rows of 4 G floats.
-struct TwoPos {
-  int rw;           // floats per row
-  int dm, dp;       // offsets of the x-neighbours of the group from its first float
-  bool nl, nr;      // take them from shared memory (a warp's or a row's end)
-};
-
-__device__ __forceinline__ void two_edges(const float* own, const TwoPos& t, const float4& c,
-                                          float& xm, float& xp) {
-  xm = __shfl_up_sync(0xffffffffu, c.w, 1);
-  xp = __shfl_down_sync(0xffffffffu, c.x, 1);
-  if (t.nl) xm = own[t.dm];
-  if (t.nr) xp = own[t.dp];
-}
-
 // z-windows of one thread's column group, three slots each, slot = plane mod 3 (the plane loop
 // is unrolled by three, so they are renamed instead of moved).
 template <int MODEL>
@@ -94,7 +76,7 @@ struct TwoStream {
   // group; l1w the level-1 plane at the group (written where live).
   template <int P>
   __device__ __forceinline__ void level1(const float* sc, const float* sp, float* l1w,
-                                         const TwoPos& t, bool live, const ModelParams& m,
+                                         const GroupPos& t, bool live, const ModelParams& m,
                                          float4& lpsi_next) {
     constexpr int S0 = P, S1 = (P + 1) % 3, S2 = (P + 2) % 3;
     float4 lap[NF];
@@ -104,7 +86,7 @@ struct TwoStream {
       const float4 ym = ld4(F - t.rw), yp = ld4(F + t.rw);
       iw[f][S2] = ld4(sp + f * C::IN_FIELD);
       float xm, xp;
-      two_edges(F, t, iw[f][S1], xm, xp);
+      t.edges(F, iw[f][S1], xm, xp);
       lap[f] = lap3d_x4<MODEL>(iw[f][S1], ym, yp, iw[f][S0], iw[f][S2], xm, xp, m.lap_scale);
     }
     if constexpr (C::kSteps) {
@@ -130,7 +112,7 @@ struct TwoStream {
   // ym / yp the offsets of the rows above and below.
   template <int P>
   __device__ __forceinline__ void level2(const float* l1r, int ym_off, int yp_off,
-                                         const TwoPos& t, const ModelParams& m,
+                                         const GroupPos& t, const ModelParams& m,
                                          float4 (&res)[NF]) {
     constexpr int S0 = P, S1 = (P + 1) % 3, S2 = (P + 2) % 3;
     float4 lap[NL1];
@@ -139,7 +121,7 @@ struct TwoStream {
       const float* F = l1r + f * C::L1_FIELD;
       const float4 ym = ld4(F + ym_off), yp = ld4(F + yp_off);
       float xm, xp;
-      two_edges(F, t, lw[f][S2], xm, xp);
+      t.edges(F, lw[f][S2], xm, xp);
       lap[f] = lap3d_x4<MODEL>(lw[f][S2], ym, yp, lw[f][S1], lw[f][S0], xm, xp, m.lap_scale);
     }
     if constexpr (C::kSteps) {
@@ -155,9 +137,9 @@ struct TwoStream {
   }
 };
 
-template <int MODEL>
+template <int MODEL, int RAGGED>
 __global__ void __launch_bounds__(kTwoThreads, 1)
-    fe3d_two_kernel(FieldPtrs in, FieldOut out, Geom g, ModelParams m, TwoTiles pl, Tb2Sched sc_) {
+    fe3d_two_kernel(FieldPtrs in, FieldOut out, Geom g, ModelParams m, StreamTiles pl, Tb2Sched sc_) {
   using C = CfgTwo<MODEL>;
   constexpr int NF = C::NF, NS = C::NS;
   extern __shared__ __align__(16) float smem[];
@@ -170,59 +152,17 @@ __global__ void __launch_bounds__(kTwoThreads, 1)
   const bool live = tid < (TY + 2) * G;  // the last warp's spare threads repeat the last group
   const int t_ = live ? tid : (TY + 2) * G - 1;
   const int r = t_ / G, q = t_ - r * G;
-  TwoPos t;
-  t.rw = 4 * G;
-  t.dm = q == 0 ? 4 * G - 1 : -1;
-  t.dp = q == G - 1 ? 4 - 4 * G : 4;
-  t.nl = (tid & 31) == 0 || q == 0;
-  t.nr = (tid & 31) == 31 || q == G - 1;
+  const GroupPos t(G, q);
   const int o1 = r * t.rw + 4 * q;  // own group in a level-1 plane; in an input plane o1 + rw
   const int ym2 = r > 0 ? -t.rw : 0, yp2 = r < TY + 1 ? t.rw : 0;  // rows level 2 may read
   const bool inner = r >= 1 && r <= TY;
   const bool warp2 = __any_sync(0xffffffffu, inner && live);
 
   const int ncols = pl.S * ((g.ny + TY - 1) / TY);
-  // Work: (column tile, z-range) segments, per the schedule's mode (Tb2Sched)
-  int64_t pos = 0, pos_end = 0;
-  int item = blockIdx.x;
-  const int nfull = sc_.full_rows * ncols;
-  if (sc_.mode == kTb2Balanced) {
-    const int64_t units = (int64_t)ncols * g.nz;
-    pos = units * blockIdx.x / gridDim.x;
-    pos_end = units * (blockIdx.x + 1) / gridDim.x;
-  } else if (sc_.mode == kTb2Rows && (int)blockIdx.x >= nfull) {
-    const int64_t units = (int64_t)ncols * (g.nz - sc_.full_rows * sc_.L);
-    const int p = blockIdx.x - nfull, np = gridDim.x - nfull;
-    pos = units * p / np;
-    pos_end = units * (p + 1) / np;
-  }
+  SegmentWalk seg(sc_, ncols, g.nz);
   TwoStream<MODEL> zs;
-  for (;;) {
-    int col, zlo, zhi, dir;
-    if (sc_.mode == kTb2Items || (sc_.mode == kTb2Rows && (int)blockIdx.x < nfull)) {
-      const bool rows = sc_.mode == kTb2Rows;
-      if (item >= (rows ? nfull : ncols * sc_.nchunks)) break;
-      col = item % ncols;
-      const int chunk = item / ncols;
-      const int len = rows ? sc_.L : sc_.chunk_len;
-      zlo = chunk * len;
-      zhi = min(g.nz, zlo + len);
-      dir = (chunk & 1) ? -1 : 1;
-      item += rows ? nfull : gridDim.x;
-      if (zlo >= zhi) continue;  // uniform over the CTA
-    } else {
-      if (pos >= pos_end) break;
-      const bool rows = sc_.mode == kTb2Rows;
-      const int zbase = rows ? sc_.full_rows * sc_.L : 0;
-      const int zlen = g.nz - zbase;
-      col = (int)(pos / zlen);
-      zlo = (int)(pos - (int64_t)col * zlen);
-      zhi = (int)min((int64_t)zlen, zlo + (pos_end - pos));
-      pos += zhi - zlo;
-      zlo += zbase;
-      zhi += zbase;
-      dir = rows ? sc_.pdir : ((blockIdx.x & 1) ? -1 : 1);
-    }
+  while (seg.next(sc_, ncols, g.nz)) {
+    const int col = seg.col, zlo = seg.zlo, zhi = seg.zhi, dir = seg.dir;
     const int n = zhi - zlo;  // output planes
     const int zfirst = dir > 0 ? zlo : zhi - 1;
     const int nin = n + 4;  // input planes zfirst - 2 dir .. zlast + 2 dir
@@ -230,67 +170,8 @@ __global__ void __launch_bounds__(kTwoThreads, 1)
     const int x0 = strip * pl.w, y0 = (col / pl.S) * TY;
     const int x1 = min(g.nx, x0 + pl.w);
 
-    // Where this thread copies from, within a plane: its group of input rows r and, for the
-    // threads of rows 0 and 1, of rows TY + 2 and TY + 3 (-1: not an aligned group of the grid)
-    int64_t src_a = -1, src_b = -1;
-    {
-      int cx = x0 - pl.lpad + 4 * q;
-      if ((g.nx & 3) == 0) cx = wrap_index(cx, g.nx);  // a group wraps whole
-      if (live && cx >= 0 && cx + 3 < g.nx) {
-        src_a = (int64_t)wrap_index(y0 - 2 + r, g.ny) * g.pitch + cx;
-        if (r < 2) src_b = (int64_t)wrap_index(y0 + TY + r, g.ny) * g.pitch + cx;
-      }
-    }
-    // The columns of the groups that are not (nx % 4 != 0): two left of the first strip, and
-    // from the grid's last whole group to two past the strip's last column
-    int nl = 0, nsc = 0, fr = 0;
-    if (g.nx & 3) {
-      nl = x0 == 0 ? 2 : 0;
-      fr = g.nx & ~3;
-      nsc = nl + max(0, x1 + 2 - max(fr, x0 - 4));
-      fr = max(fr, x0 - 4);
-    }
-    const int nitems = NF * (TY + 4) * nsc;
-    auto scalar_item = [&](int i, int& f, int64_t& src, int& dst) {
-      const int k = i % nsc, rf = i / nsc;
-      const int row = rf % (TY + 4);
-      f = rf / (TY + 4);
-      const int cx = k < nl ? k - 2 : fr + (k - nl);
-      src = (int64_t)wrap_index(y0 - 2 + row, g.ny) * g.pitch + wrap_index(cx, g.nx);
-      dst = f * C::IN_FIELD + row * t.rw + (cx - (x0 - 4));
-    };
-    int sf = 0, sdst = 0;
-    int64_t ssrc = -1;
-    if (tid < nitems) scalar_item(tid, sf, ssrc, sdst);
-    const float* sbase = sf == 0 ? in.f[0] : in.f[NF - 1];
-
-    int zin = wrap_index(zfirst - 2 * dir, g.nz);  // the next input plane to stage
-    auto stage = [&](int slot) {                   // it into ring slot `slot`; advances zin
-      const int64_t zo = (int64_t)zin * g.plane;
-      zin += dir;
-      if (zin == g.nz) zin = 0;
-      if (zin < 0) zin = g.nz - 1;
-      float* st = ring + slot * C::IN_STAGE;
-      if (src_a >= 0) {
-#pragma unroll
-        for (int f = 0; f < NF; ++f)
-          cp_async16(st + f * C::IN_FIELD + o1, in.f[f] + (zo + src_a));
-      }
-      if (src_b >= 0) {
-#pragma unroll
-        for (int f = 0; f < NF; ++f)
-          cp_async16(st + f * C::IN_FIELD + o1 + (TY + 2) * t.rw, in.f[f] + (zo + src_b));
-      }
-      if (nitems > 0) {
-        if (ssrc >= 0) cp_async4(st + sdst, sbase + (zo + ssrc));
-        for (int k = tid + blockDim.x; k < nitems; k += blockDim.x) {  // short rows only
-          int f, d;
-          int64_t s;
-          scalar_item(k, f, s, d);
-          cp_async4(st + d, (f == 0 ? in.f[0] : in.f[NF - 1]) + (zo + s));
-        }
-      }
-    };
+    PlaneCopy<NF, 2, C::IN_FIELD, RAGGED> cp(in, g, x0, x1, y0, pl.lpad, G, TY, TY + 2, r, q, live,
+                                             zfirst - 2 * dir, dir);
 
     // where this thread stores: its output row and columns
     const int gy = y0 + r - 1, gx = x0 - pl.lpad + 4 * q;
@@ -302,7 +183,7 @@ __global__ void __launch_bounds__(kTwoThreads, 1)
     __syncthreads();  // every thread is done with the last segment's planes
 #pragma unroll
     for (int i = 0; i < NS; ++i) {
-      if (i < nin) stage(i);
+      if (i < nin) cp.stage(in, g, ring + i * C::IN_STAGE);
       cp_async_commit();
     }
     cp_async_wait_group<NS - 2>();  // input planes 0 and 1
@@ -318,7 +199,7 @@ __global__ void __launch_bounds__(kTwoThreads, 1)
       constexpr int P = decltype(phase)::value;
       cp_async_wait_group<NS - 3>();  // input plane j + 2 has landed
       __syncthreads();                // ... for every thread, and plane j's slot is free
-      if (j + NS < nin) stage(s0);
+      if (j + NS < nin) cp.stage(in, g, ring + s0 * C::IN_STAGE);
       cp_async_commit();  // possibly empty: one group per iteration
       float* l1w = l1 + (j & 1) * C::L1_PLANE + o1;
       const float* l1r = l1 + ((j + 1) & 1) * C::L1_PLANE + o1;
@@ -360,65 +241,33 @@ __global__ void __launch_bounds__(kTwoThreads, 1)
   }
 }
 
-// Tiles and work split of a grid. Rows of at most 256 columns whole, longer ones in equal
-// strips; the tile height that makes the launch shortest by span * (kTwoPlaneWarps + warps):
-// the longest CTA's plane count times a plane's time, which is linear in the CTA's warps above
-// a fixed part for the barrier and the latencies behind it. Fitted to 450 timed (grid, height)
-// pairs of all four models, 64^3 to 256^3 (a plane of Gray-Scott 0.37 + 0.035 warps us, of
-// Allen-Cahn 0.25 + 0.021); its choice was within 1 % of the best height on eight of nine grids
-// (4 % on the ninth), where the tallest tile lost up to 55 % (64^3).
+// The plan's fixed part, in warps. Fitted to 450 timed (grid, height) pairs of all four models,
+// 64^3 to 256^3 (a plane of Gray-Scott 0.37 + 0.035 warps us, of Allen-Cahn 0.25 + 0.021); its
+// choice was within 1 % of the best height on eight of nine grids (4 % on the ninth), where the
+// tallest tile lost up to 55 % (64^3).
 constexpr int kTwoPlaneWarps = 11;
 
-TwoPlan two_plan(const Geom& g, long long sms) {
-  TwoPlan pl{};
-  TwoTiles& p = pl.tiles;
-  if (g.nx % 4 == 0 && g.nx <= 4 * kTwoMaxGroups) {
-    p.G = g.nx / 4;
-    p.S = 1;
-    p.w = g.nx;
-  } else {
-    constexpr int wmax = 4 * kTwoMaxGroups - 8;
-    p.lpad = 4;
-    p.S = (g.nx + wmax - 1) / wmax;
-    p.w = p.S == 1 ? g.nx : ((g.nx + p.S - 1) / p.S + 3) / 4 * 4;
-    p.S = (g.nx + p.w - 1) / p.w;
-    p.G = (4 + p.w + 2 + 3) / 4;  // the halo group, w columns, and two more columns
-  }
-  const int tmax = std::min(kTwoThreads / p.G - 2, g.ny);
-  long long best = -1;
-  int last = 0;
-  for (int t = tmax; t >= 1; --t) {
-    const int tiles = (g.ny + t - 1) / t;
-    const int ty = (g.ny + tiles - 1) / tiles;  // spread evenly
-    if (ty == last) continue;
-    last = ty;
-    long long gr = 0, span = 0;
-    const long long ncols = (long long)p.S * tiles;
-    if (pl.valid && ncols > 64 * sms) break;  // enough tiles: taller ones have less halo
-    const Tb2Sched s = tb2_schedule((int)ncols, g.nz, sms, &gr, &span);
-    const long long cost = span * (kTwoPlaneWarps + ((ty + 2) * p.G + 31) / 32);
-    if (best < 0 || cost < best) {
-      best = cost;
-      p.TY = ty;
-      pl.sched = s;
-      pl.grid = (unsigned)gr;
-      pl.valid = true;
-    }
-  }
-  return pl;
+template <int MODEL, int RAGGED>
+cudaError_t launch_two_(pf_grid_s* gr, FieldPtrs in, FieldOut out, cudaStream_t st) {
+  using C = CfgTwo<MODEL>;
+  auto kern = fe3d_two_kernel<MODEL, RAGGED>;
+  static unsigned long long attr_mask = 0;  // per instantiation and device
+  cudaError_t e = ensure_smem_attr(kern, C::SMEM, &attr_mask);
+  if (e != cudaSuccess) return e;
+  const StreamTiles& p = gr->two.tiles;
+  const int nt = ((p.TY + 2) * p.G + 31) / 32 * 32;
+  kern<<<gr->two.grid, nt, C::SMEM, st>>>(in, out, grid_geom(gr), gr->params, p, gr->two.sched);
+  return cudaGetLastError();
 }
 
 template <int MODEL>
 cudaError_t launch_two(pf_grid_s* gr, FieldPtrs in, FieldOut out, cudaStream_t st) {
-  using C = CfgTwo<MODEL>;
-  auto kern = fe3d_two_kernel<MODEL>;
-  static unsigned long long attr_mask = 0;  // per instantiation and device
-  cudaError_t e = ensure_smem_attr(kern, C::SMEM, &attr_mask);
-  if (e != cudaSuccess) return e;
-  const TwoTiles& p = gr->two.tiles;
-  const int nt = ((p.TY + 2) * p.G + 31) / 32 * 32;
-  kern<<<gr->two.grid, nt, C::SMEM, st>>>(in, out, grid_geom(gr), gr->params, p, gr->two.sched);
-  return cudaGetLastError();
+  const StreamTiles& p = gr->two.tiles;
+  switch (copy_form(grid_geom(gr), p, CfgTwo<MODEL>::NF, 2, (p.TY + 2) * p.G)) {
+    case 0: return launch_two_<MODEL, 0>(gr, in, out, st);
+    case 1: return launch_two_<MODEL, 1>(gr, in, out, st);
+  }
+  return launch_two_<MODEL, 2>(gr, in, out, st);
 }
 
 }  // namespace
@@ -429,7 +278,7 @@ cudaError_t launch_fe3d_two(pf_grid_s* gr, int src, int dst, cudaStream_t st) {
     int sms = 0;
     cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, gr->device);
     if (e != cudaSuccess) return e;
-    gr->two = two_plan(grid_geom(gr), sms);
+    gr->two = stream_plan(grid_geom(gr), sms, kTwoThreads, kTwoMaxGroups, 2, 2, kTwoPlaneWarps);
   }
   FieldPtrs in{};
   FieldOut out{};

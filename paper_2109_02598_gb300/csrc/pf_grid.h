@@ -68,8 +68,9 @@ struct Tb2Sched {
 };
 constexpr int kTb2Items = 0, kTb2Balanced = 1, kTb2Rows = 2;
 
-// Tiles of the two-level 3D kernel (pf_fe3d_two.cu), chosen on the host (two_plan).
-struct TwoTiles {
+// Tiles of the 3D kernels that stream rows of any length (pf_fe3d_stream.cuh), chosen on the
+// host (stream_plan).
+struct StreamTiles {
   int G;      // groups of four columns per row
   int TY;     // output rows per tile
   int lpad;   // staged columns left of the strip: 0 (full periodic rows) or 4
@@ -77,9 +78,9 @@ struct TwoTiles {
 };
 
 // They depend on the grid's sides only, so a handle keeps them.
-struct TwoPlan {
+struct StreamPlan {
   bool valid = false;
-  TwoTiles tiles{};
+  StreamTiles tiles{};
   Tb2Sched sched{};
   unsigned grid = 0;
 };
@@ -143,7 +144,9 @@ struct pf_grid_s {
   pf::TmaCache tma;
   pf::Tma2Cache tma2;
   pf::Tb2Cache tb2;
-  pf::TwoPlan two;
+  pf::StreamPlan two;  // pf_fe3d_two.cu
+  pf::StreamPlan one;  // pf_fe3d_one.cu
+  int one_key = -1;    // the kernel it was made for
   int* d_err = nullptr;  // set by a kernel whose bounded wait ran out
   // band kernel (2D grid resident in the SMs' shared memory): exchange slots of the bands'
   // edge rows as tagged 64-bit words, allocated at its first launch, and the last tag used
@@ -194,6 +197,9 @@ void fe2d_bands_release(pf_grid_s* g);
 // The general 3D tiles with the 7-point stencil (any size): two steps a launch for AC and GS,
 // one for Models B and C (pf_fe3d_two.cu)
 cudaError_t launch_fe3d_two(pf_grid_s* g, int src, int dst, cudaStream_t st);
+// One step of Allen-Cahn and Gray-Scott (any stencil) or of N species on 3D grids of any size
+// (pf_fe3d_one.cu)
+cudaError_t launch_fe3d_one(pf_grid_s* g, int src, int dst, cudaStream_t st);
 
 // ---- 3D depth-2 kernel (AC, GS; full x-rows of 128 or 256, 8-row tiles)
 bool fe3d_tb2_supported(int model, int tx, int ty, const Geom& g);

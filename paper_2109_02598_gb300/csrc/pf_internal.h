@@ -32,17 +32,20 @@ struct FieldOut {
 
 // N coupled species (PF_MODEL_RD): du_i/dt = D_i lap u_i + sum_m K[i][m] prod_j u_j^E[m][j],
 // as the kernel takes it (pf_rdn.cu): D_i times the stencil factor 1/h^2 and the rates rounded
-// once to float32; monomial m's exponents packed two bits per field (field j at bits 2j).
+// once to float32; monomial m's exponents packed two bits per field (field j at bits 2j), and its
+// place in the written-out list of pf_rd.cuh (rd_places).
 constexpr int kRdMonomials = 8;
 struct RdParams {
   int nmono;
   int E[kRdMonomials];
+  int place[kRdMonomials];
   float D[PF_MAX_FIELDS];
   float K[PF_MAX_FIELDS][kRdMonomials];
   float dt;
 };
-cudaError_t launch_rd(const Geom& g, int nf, FieldPtrs in, FieldOut out, const RdParams& p,
-                      cudaStream_t s);
+void rd_places(int nf, RdParams& p);  // fills place from nmono and E
+cudaError_t launch_rd2d(const Geom& g, int nf, FieldPtrs in, FieldOut out, const RdParams& p,
+                        cudaStream_t s);
 
 // Set a kernel's dynamic shared-memory limit once per device (the attribute is per device;
 // `mask` has one bit per device ordinal below 64, set after success).
@@ -131,8 +134,9 @@ cudaError_t launch_fe3d_box(int model, int k, const Geom& g, FieldPtrs in, Field
                             const ModelParams& m, cudaStream_t s);
 void tile3d_shape(int tile_id, int* tx, int* ty);
 int tile3d_id(int tx, int ty);
+// Models B and C with the 19- or 27-point stencil on tile 0 or 1 (pf_fe3d.cu).
 cudaError_t launch_fe3d(int model, int tile_id, const Geom& g, FieldPtrs in, FieldOut out,
-                        const ModelParams& m, cudaStream_t s, int stencil = PF_ST_STD);
+                        const ModelParams& m, cudaStream_t s, int stencil);
 
 // ---- batched 2D Gray-Scott (many independent grids, one launch per k steps) -------
 // Instance i: fields at buffer base + off (u) and base + off + pitch * ny (v).

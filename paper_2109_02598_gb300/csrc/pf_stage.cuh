@@ -36,32 +36,4 @@ __device__ __forceinline__ void stage_rows4(const FieldPtrs& in, const Geom& g, 
   }
 }
 
-// CTAs of a kernel that the device holds at once (cached per device; 0 on error).
-template <class KernelT>
-int resident_ctas(KernelT kernel, int threads, size_t smem, int* cache) {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev >= 64) return 0;
-  if (cache[dev] == 0) {
-    int b = 0, sms = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, threads, smem) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-      cudaGetLastError();
-      return 0;
-    }
-    cache[dev] = (b > 0 ? b : 1) * (sms > 0 ? sms : 1);
-  }
-  return cache[dev];
-}
-
-// Planes per z-chunk for a grid of tiles_xy columns: as many chunks as fit the device in one
-// wave beside the other columns (a partial second wave leaves most SMs idle), at least four
-// planes each.
-inline int one_wave_tz(int nz, int tiles_xy, int resident) {
-  int nzc = resident > 0 ? resident / tiles_xy : 1;
-  nzc = nzc < 1 ? 1 : nzc;
-  const int max_chunks = nz / 4 > 1 ? nz / 4 : 1;
-  nzc = nzc > max_chunks ? max_chunks : nzc;
-  return (nz + nzc - 1) / nzc;
-}
-
 }  // namespace pf
