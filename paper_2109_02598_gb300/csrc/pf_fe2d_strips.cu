@@ -399,17 +399,35 @@ __global__ void __launch_bounds__(kStripThreads, (StripCfg<PF_MODEL_GS, K, C>::M
   r.run(in, out, I.nx, I.ny, I.pitch, t.x0, t.wo, t.y0, t.hy, I.m);
 }
 
-// Rows per task. A task's first and last rows carry the levels' start-up and drain, which
-// argues for long tasks, and every warp slot should stay busy: so as many tasks as the
-// device holds warps at once (one wave, rows split evenly), unless that makes them shorter
-// than min_rows; then tasks of min_rows rows in several waves.
-int strip_rows(int tasks_x, int ny, int resident_warps, int min_rows) {
-  const int per_col = resident_warps / tasks_x;
-  if (per_col >= 1) {
-    const int hy = (ny + per_col - 1) / per_col;
-    if (hy >= min_rows || hy >= ny) return hy;
+// Rows per task: the height that makes the launch shortest by waves * (rows + T0) * (100 + w), w
+// the warps per SM of a wave. A task takes T0 iterations beside its rows, and an iteration is
+// mostly latency: its time grows with the resident warps only as 100 + w (fitted to 2200 timed
+// launches, all four models, depths 2 and 4, both widths, 256^2 to 4096^2; its choice is within
+// 5 % of the best height timed on nine of ten). So a wave is filled with the lowest tasks that
+// still fit it, and grids of many rows take a few waves. The rule before (one wave unless that
+// makes tasks of fewer than 4 T0 rows, then that height) left a 1502 x 1111 grid with four warps
+// per SM: Gray-Scott, 64 columns, k = 4: 7.4 -> 3.45 us a step (the tiled kernel 3.8), 2048^2
+// 8.6 -> 6.2; Allen-Cahn 4096^2 at 128 columns 11.4 -> 10.5, Model B 4096^2 20.1 -> 18.2.
+constexpr int kStripMinRows = 4;
+int strip_rows(int tasks_x, int ny, int resident_warps, int sms, int t0) {
+  int best = ny;
+  double cost = -1.0;
+  for (int waves = 1; waves <= 8; ++waves) {
+    const long long per_col = (long long)waves * resident_warps / tasks_x;  // tasks down a strip
+    if (per_col < 1) continue;
+    int hy = (int)((ny + per_col - 1) / per_col);
+    hy = hy < kStripMinRows ? kStripMinRows : hy;
+    hy = hy < ny ? hy : ny;
+    const long long n = (long long)tasks_x * ((ny + hy - 1) / hy);
+    const double w = (double)(n < resident_warps ? n : resident_warps) / sms;
+    const double c = (double)((n + resident_warps - 1) / resident_warps) * (hy + t0) * (100.0 + w);
+    if (cost < 0 || c < cost) {
+      cost = c;
+      best = hy;
+    }
   }
-  return min_rows < ny ? min_rows : ny;
+  // (more strips than eight waves of warps: whole columns would be too long a tail)
+  return cost < 0 ? (ny < 4 * t0 ? ny : 4 * t0) : best;
 }
 
 template <int MODEL, int K, int C, int ST>
@@ -417,7 +435,7 @@ cudaError_t launch_strip(const Geom& g, FieldPtrs in, FieldOut out, const ModelP
                          cudaStream_t s) {
   using S = StripCfg<MODEL, K, C>;
   using Run = StripRun<MODEL, K, C, ST>;
-  static int resident[64] = {};  // resident warps of this kernel on the whole device
+  static int resident[64] = {}, sms_of[64] = {};  // resident warps of this kernel, SMs
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -428,10 +446,11 @@ cudaError_t launch_strip(const Geom& g, FieldPtrs in, FieldOut out, const ModelP
                                                       kStripThreads, 0);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    resident[dev] = (b > 0 ? b : 1) * (sms > 0 ? sms : 1) * kStripWarps;
+    sms_of[dev] = sms > 0 ? sms : 1;
+    resident[dev] = (b > 0 ? b : 1) * sms_of[dev] * kStripWarps;
   }
   const int tasks_x = (g.nx + S::WO - 1) / S::WO;
-  const int hy = strip_rows(tasks_x, g.ny, resident[dev], 4 * Run::T0);
+  const int hy = strip_rows(tasks_x, g.ny, resident[dev], sms_of[dev], Run::T0);
   const int ntasks = tasks_x * ((g.ny + hy - 1) / hy);
   const int blocks = (ntasks + kStripWarps - 1) / kStripWarps;
   fe2d_strip_kernel<MODEL, K, C, ST><<<blocks, kStripThreads, 0, s>>>(in, out, g, m, hy,
