@@ -236,14 +236,34 @@ int launch_depth(const pf_grid_s* g, int tile, int k) {
   return pairs ? 2 : k;
 }
 
-// The tile pf_step runs. Where a 3D grid's tuning is the library's own choice (nothing asked
-// for), the general tile's kernel takes the place of the depth-1 TMA tile that pf_get_tuning
-// names: it passes the TMA tiles wherever both run (256^3 GS 510 against 369 GLUPS, AC 816/716,
-// Model B 419/393, Model C 279/165; 64^3 GS 90/60, Model B 58/38), with the same bits.
-int run_tile(const pf_grid_s* g) {
-  const bool untuned = g->dim == 3 && g->stencil == PF_ST_STD && g->model != PF_MODEL_RD &&
-                       g->req_tile < 0 && g->req_k == 0;
-  return untuned ? 0 : g->tile;
+// The tile and depth that run a 2D grid with the standard stencil where nothing was asked for
+// (us a step, against the 128x16 tiles at depth 1 that pf_get_tuning names; the same bits):
+//   up to 2^21 sites 32x32 tiles at the model's greatest depth (GS 128^2 0.78/2.38, 512^2
+//     1.05/2.52, 1502x1111 3.8/6.2; AC 512^2 0.76/2.11; Model B 512^2 1.57/2.55; Model C 512^2
+//     1.89/3.02);
+//   above, strips at that depth, 64 columns for two fields and 128 for one (2048^2 GS 6.2/11.5,
+//     AC 3.9/7.3, Model B 7.6/10.7, Model C 12.0/15.3; at 1502x1111 32x32 tiles are still level:
+//     GS 3.8/3.65, AC 2.25/2.36, Model B 4.7/4.65, Model C 6.8/7.0).
+void plan2d(const pf_grid_s* g, int* tile, int* depth) {
+  const bool r1 = g->model == PF_MODEL_AC || g->model == PF_MODEL_GS;
+  const bool big = (int64_t)g->nx * g->ny > (int64_t)1 << 21;
+  *tile = big ? kTileStrips2D + (g->nf == 2 ? 1 : 0) : 2;
+  *depth = r1 ? 4 : 2;
+}
+
+// The tile and depth pf_step runs: the tuning in effect, except where it is the library's own
+// choice (nothing asked for) and the stencil the standard one. Then a kernel that passes the one
+// pf_get_tuning names takes its place, with the same bits: plan2d's, and in 3D the general tile's
+// for the depth-1 TMA tiles (256^3 GS 572 against 369 GLUPS, AC 979/716, Model B 520/393, Model C
+// 317/165; 64^3 GS 117/60, Model B 74/38).
+void run_plan(const pf_grid_s* g, int* tile, int* depth) {
+  const bool untuned = g->stencil == PF_ST_STD && g->model != PF_MODEL_RD && g->req_tile < 0 &&
+                       g->req_k == 0;
+  *tile = g->tile;
+  int k = g->k;
+  if (untuned && g->dim == 3) *tile = 0;
+  if (untuned && g->dim == 2) plan2d(g, tile, &k);
+  *depth = launch_depth(g, *tile, k);
 }
 
 int sync_device_error(pf_grid_s* g);
@@ -609,14 +629,14 @@ int pf_step(pf_grid_t g, int64_t n_steps) {
     g->cur = 1 - g->cur;
     return PF_OK;
   }
-  const int tile = run_tile(g);
-  const int depth = launch_depth(g, tile, g->k);
+  int tile = 0, depth = 1;
+  run_plan(g, &tile, &depth);
   if (count_launches(n_steps, depth) >= kGraphMinLaunches) {
     // replay a recorded graph of the whole launch sequence (one host call)
     pf_grid_s::StepGraph* hit = nullptr;
     pf_grid_s::StepGraph* victim = &g->step_graphs[0];
     for (auto& sg : g->step_graphs) {
-      if (sg.exec && sg.steps == n_steps && sg.tile == tile && sg.k == g->k &&
+      if (sg.exec && sg.steps == n_steps && sg.tile == tile && sg.k == depth &&
           sg.start == g->cur)
         hit = &sg;
       if (sg.used < victim->used) victim = &sg;
@@ -627,7 +647,7 @@ int pf_step(pf_grid_t g, int64_t n_steps) {
       if (int rc = record_step_graph(g, tile, depth, n_steps, &victim->exec, &victim->flip)) return rc;
       victim->steps = n_steps;
       victim->tile = tile;
-      victim->k = g->k;
+      victim->k = depth;
       victim->start = g->cur;
       hit = victim;
     }
