@@ -303,9 +303,12 @@ int pf_batch_info(pf_batch_t b, int64_t* sites, int64_t* bytes_per_copy);
 /* Forward pass that records checkpoints for pf_adj_backward: advances the grid's current
  * state (2D grid; Gray-Scott, Allen-Cahn or Cahn-Hilliard model) by n_steps forward-Euler
  * steps exactly like
- * pf_step, storing the state every ckpt_interval steps (0 = ceil(sqrt(n_steps))), i.e.
- * sqrt(N) checkpointing of the time loop of Sec. 2.4.1. Allocates the checkpoints
- * (ceil(N/C) states), one segment of C-1 states and the adjoint buffers on first use.
+ * pf_step, storing the state every ckpt_interval steps. 0 leaves the interval C to the library:
+ * where they fit 4 GiB of device memory the states the reverse pass starts its launches from
+ * (every 4th, for Model B every 2nd), else C = ceil(sqrt(n_steps)), i.e.
+ * sqrt(N) checkpointing of the time loop of Sec. 2.4.1. The gradients do not depend on C.
+ * Allocates the checkpoints (ceil(N/C) states), a segment's states between them and the adjoint
+ * buffers on first use.
  * Errors: PF_ERR_STATE (no Gray-Scott model), PF_ERR_INVALID_ARG (3D grid, n < 1),
  * PF_ERR_OOM, PF_ERR_CUDA. */
 int pf_adj_forward(pf_grid_t g, int64_t n_steps, int64_t ckpt_interval);

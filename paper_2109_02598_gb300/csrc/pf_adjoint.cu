@@ -18,13 +18,14 @@
 //   B: w = lap lambda, lambda^n = lambda + dt M [(3 c2 x^2 - c1) w - lap w];
 //      sums S = (sum w x, sum w x^3, sum w mu), dL/d(c1, c2, M) = dt (-M S0, M S1, S2).
 //
-// Memory/recompute: the forward pass stores x at every C-th step (C ~ sqrt(N)); the
-// backward pass walks the segments from last to first, recomputes the segment's states
-// from its checkpoint with the forward kernel, then runs the segment's adjoint steps.
-// Parameter-gradient partials are summed per CTA in FP64 (each CTA owns one slot, so the
-// order is fixed and the result deterministic) and added up in a fixed order at the end.
+// Memory/recompute: the forward pass stores x at every C-th step; the backward pass walks the
+// segments from last to first and goes back through each in blocks of up to four steps (two for
+// Model B) a launch, from the state at the block's first step; the states inside a block are
+// recomputed on chip. The blocks' first states are stored where the library chooses C and they
+// fit, else the segment's are recomputed from its checkpoint with the forward kernel
+// (C ~ sqrt(N)). Parameter-gradient partials are summed per CTA in FP64 (each CTA owns one slot,
+// so the order is fixed and the result deterministic) and added up in a fixed order at the end.
 #include <cmath>
-#include <vector>
 
 #include "pf_fe2d_tile.cuh"
 #include "pf_grid.h"
@@ -34,18 +35,19 @@ namespace pf {
 
 namespace {
 
+// Bytes of stored states up to which the forward pass keeps every block's first one.
+constexpr double kAllStates = 4.0 * (1 << 30);
+
 constexpr int kATX = 64, kATY = 16;  // adjoint tile
-constexpr int kAW = kATX + 2, kAH = kATY + 2, kAPL = kAW * kAH;
 
 // Warp sum of per-thread float partials, in float (a fixed tree, so the same bits on every
-// run), widened to double for the per-warp and per-CTA sums. FP64 arithmetic is a small
+// run); the per-warp sums are added in double. FP64 arithmetic and conversions are a small
 // fraction of FP32 throughput on this GPU: a double-precision shuffle tree in every CTA of
 // every reverse step took most of the kernel's time.
-__device__ __forceinline__ double warp_sum_f(double v) {
-  float f = (float)v;
+__device__ __forceinline__ float warp_sum_f(float f) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) f = __fadd_rn(f, __shfl_down_sync(0xffffffffu, f, o));
-  return (double)f;
+  return f;
 }
 
 // Double-precision warp sum, for the final fixed-order sum over the CTAs' slots (once per
@@ -56,213 +58,468 @@ __device__ __forceinline__ double warp_sum_d(double v) {
   return v;
 }
 
-// One reverse step on a 64 x TY tile: stage u, v (the state x^n) and a, b (lambda^{n+1})
-// with a periodic halo of 1 as aligned float4 groups (the forward tile body's staging), then
-// four sites per thread: update (a, b) and add the parameter-gradient terms to per-thread
-// sums, which go to this tile's FP64 slot in a fixed order.
-// TY = 8 on grids too small to give every SM several 16-row tiles (more CTAs in flight hide
-// the L2 latency of the staging: 512^2 reverse step 8.4 -> 7.6 us), else 16 (2048^2: 49.5 us
-// with 16 rows, 58.8 with 8).
-template <int TY>
-__global__ void __launch_bounds__(kNT2) adj_gs2d_kernel(FieldPtrs x, FieldPtrs lam,
-                                                        FieldOut lam_out, Geom g,
-                                                        ModelParams m, double* gpart) {
-  using AdjCfg = Cfg2<PF_MODEL_GS, 1, kATX, TY>;
-  constexpr int WS = AdjCfg::WS, PL = AdjCfg::PL, HP = AdjCfg::HP, H = AdjCfg::H;
-  __shared__ __align__(16) float sm[4 * PL];  // u, v, a, b
-  __shared__ double red[4][kNT2 / 32];
-  const int x0 = blockIdx.x * kATX;
-  const int y0 = blockIdx.y * TY;
-  canary_fill(sm, 4 * PL);
-  load_region2d<AdjCfg, false>(x, g.nx, g.ny, g.pitch, x0, y0, sm);  // waits with the next
-  load_region2d<AdjCfg>(lam, g.nx, g.ny, g.pitch, x0, y0, sm + 2 * PL);
-  __syncthreads();
-  const float* su = sm;
-  const float* sv = sm + PL;
-  const float* sa = sm + 2 * PL;
-  const float* sb = sm + 3 * PL;
-  float pDu = 0.f, pDv = 0.f, pF = 0.f, pk = 0.f;
-  constexpr int NG = kATX / 4;  // float4 groups per tile row
-  for (int i = threadIdx.x; i < TY * NG; i += kNT2) {
-    const int rr = i / NG, j = i - rr * NG;
-    const int gy = y0 + rr;
-    const int gx = x0 + 4 * j;
-    if (gy >= g.ny || gx >= g.nx) continue;
-    const int p = (rr + H) * WS + HP + 4 * j;
-    const float4 u4 = *reinterpret_cast<const float4*>(su + p);
-    const float4 v4 = *reinterpret_cast<const float4*>(sv + p);
-    const float4 a4 = *reinterpret_cast<const float4*>(sa + p);
-    const float4 b4 = *reinterpret_cast<const float4*>(sb + p);
-    const float4 la4 = lap2d_x4(sa, p, WS, m.lap_scale);
-    const float4 lb4 = lap2d_x4(sb, p, WS, m.lap_scale);
-    const float4 lu4 = lap2d_x4(su, p, WS, m.lap_scale);
-    const float4 lv4 = lap2d_x4(sv, p, WS, m.lap_scale);
-    const float uu[4] = {u4.x, u4.y, u4.z, u4.w}, vv_[4] = {v4.x, v4.y, v4.z, v4.w};
-    const float aa[4] = {a4.x, a4.y, a4.z, a4.w}, bb[4] = {b4.x, b4.y, b4.z, b4.w};
-    const float la[4] = {la4.x, la4.y, la4.z, la4.w}, lb[4] = {lb4.x, lb4.y, lb4.z, lb4.w};
-    const float lu[4] = {lu4.x, lu4.y, lu4.z, lu4.w}, lv[4] = {lv4.x, lv4.y, lv4.z, lv4.w};
-    float na[4], nb[4];
-    const int nvalid = g.nx - gx < 4 ? g.nx - gx : 4;
+// LEN reverse steps of Gray-Scott on a 64 x 16 tile in one launch, from the state x^s at the
+// block's first step and lambda^{s+LEN}: both are staged with their halos (2 (LEN - 1) and LEN
+// sites), the states x^{s+1} .. x^{s+LEN-1} are recomputed in shared memory on regions that
+// shrink by a site a step (the forward step's functions, so its bits), and lambda goes back
+// through them on regions of the tile plus j sites, j = LEN - 1 .. 0. So of the states only every
+// LEN-th goes through memory, and a launch and its round trips through L2 are paid once per LEN
+// steps. Groups past the grid's edge are computed as what they are, periodic images.
+//
+// The parameter-gradient terms are summed over the tile as a reverse step of its own would: per
+// thread over its group of four sites, per warp (two rows of the tile) by a fixed tree, both in
+// float, then in FP64 over the warps, and step after step into the CTA's slot, so the sums do not
+// depend on how the steps are cut into blocks.
+//
+// Bound by the latency of its chain (staging, LEN - 1 forward and LEN reverse stages, each behind
+// a barrier: about 8 us for four steps on a 64^2 grid, 12 at 512^2) and by shared memory on large
+// grids. The reverse pass of 400 steps, against one launch per step with the states recomputed on
+// a second stream: 512^2 2.09 -> 1.20 ms, 128^2 1.27 -> 0.80, 1024^2 4.7 -> 3.4, 2048^2 14.4 ->
+// 12.3. 64 x 32 tiles (less halo, one CTA per SM): the same at 512^2, 20 to 45 % slower on smaller
+// and larger grids.
+template <int LEN>
+struct AdjBlock {
+  static constexpr int TY = kATY;
+  static constexpr int TILE = 16 * TY;                           // groups of the tile
+  static constexpr int H = LEN > 1 ? 2 * (LEN - 1) : 1;          // staged halo rows of the state
+  static constexpr int HP = (H + 3) / 4 * 4;                     // and columns
+  static constexpr int WS = kATX + 2 * HP, ROWS = TY + 2 * H;
+  static constexpr int PL = WS * ROWS;                           // floats of a field
+  static constexpr int SMEM_FLOATS = (2 * LEN + 4) * PL;         // the states, lambda twice
+  // Threads: every region in one pass where 1024 do it: the first recomputed state, and the tile
+  // with its widest ring (a group each)
+  static constexpr int FIRST = LEN > 1 ? (TY + 2 * (H - 1)) * (kATX / 4 + 2 * ((H + 2) / 4)) : 0;
+  static constexpr int RING = LEN > 1 ? 2 * (LEN - 1) * (kATX / 4 + 2) + 2 * TY : 0;
+  static constexpr int WANT = FIRST > TILE + RING ? FIRST : TILE + RING;
+  static constexpr int NT = WANT > 1024 ? 1024 : (WANT + 31) / 32 * 32;
+  static_assert(NT >= TILE && (LEN == 1 || NT > TILE), "threads beside the tile's for its ring");
+  static_assert(H >= LEN && HP >= 4, "lambda's halo fits the states' geometry");
+  // offset of the group of tile row r, group q (four columns from 4 q)
+  static __device__ __forceinline__ int at(int r, int q) { return (r + H) * WS + HP + 4 * q; }
+};
+
+template <int LEN>
+__global__ void __launch_bounds__(AdjBlock<LEN>::NT)
+    adj_gs2d_kernel(FieldPtrs x, FieldPtrs lam, FieldOut lam_out, Geom g, ModelParams m,
+                    double* gpart) {
+  using B = AdjBlock<LEN>;
+  constexpr int TY = B::TY, WS = B::WS, PL = B::PL, NT = B::NT, H = B::H;
+  extern __shared__ __align__(16) float sm[];  // state j: u at 2 j PL, v behind it
+  constexpr int TILE = B::TILE, NW = TILE / 32;  // warps of the tile
+  __shared__ float red[LEN][4][NW];
+  __shared__ double step_sum[LEN][4];
+  float* la = sm + 2 * LEN * PL;  // lambda: a, b; then the other buffer
+  const int tid = threadIdx.x;
+  const int x0 = blockIdx.x * kATX, y0 = blockIdx.y * TY;
+  canary_fill(sm, B::SMEM_FLOATS);
+  chain_wait();
+  // rows y0 - h .. y0 + TY + h - 1, columns x0 - hp .. x0 + 63 + hp of two fields
+  auto stage = [&](const FieldPtrs& in, int h, int hp, float* dst) {
+    const int gpr = (kATX + 2 * hp) / 4;
+    for (int i = tid; i < (TY + 2 * h) * gpr; i += NT) {
+      const int r = i / gpr, q = i - r * gpr - hp / 4;
+      const int64_t row = (int64_t)wrap_index(y0 - h + r, g.ny) * g.pitch;
+      const int gx = x0 + 4 * q;
+      float* d = dst + B::at(r - h, q);
+      if (gx >= 0 && gx + 3 < g.nx) {
+        cp_async16(d, in.f[0] + row + gx);
+        cp_async16(d + PL, in.f[1] + row + gx);
+      } else {
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float u = uu[e], v = vv_[e], a = aa[e], b = bb[e];
-      const float vv = __fmul_rn(v, v);
-      const float uv2 = __fmul_rn(2.0f, __fmul_rn(u, v));
-      // a' = a + dt [Du la - (v^2 + F) a + v^2 b]
-      float fa = __fmaf_rn(-__fadd_rn(vv, m.a2), a, __fmul_rn(vv, b));
-      fa = __fmaf_rn(m.a0, la[e], fa);
-      // b' = b + dt [Dv lb - 2uv a + (2uv - F - k) b]
-      float fb = __fmaf_rn(__fsub_rn(uv2, m.a3), b, -__fmul_rn(uv2, a));
-      fb = __fmaf_rn(m.a1, lb[e], fb);
-      na[e] = __fmaf_rn(m.dt, fa, a);
-      nb[e] = __fmaf_rn(m.dt, fb, b);
-      if (e < nvalid) {
-        pDu = __fmaf_rn(a, lu[e], pDu);
-        pDv = __fmaf_rn(b, lv[e], pDv);
-        pF = __fadd_rn(pF, __fsub_rn(__fmul_rn(__fsub_rn(1.0f, u), a), __fmul_rn(v, b)));
-        pk = __fsub_rn(pk, __fmul_rn(v, b));
+        for (int c = 0; c < 4; ++c) {
+          const int64_t o = row + wrap_index(gx + c, g.nx);
+          cp_async4(d + c, in.f[0] + o);
+          cp_async4(d + PL + c, in.f[1] + o);
+        }
       }
     }
-    const int64_t off = (int64_t)gy * g.pitch + gx;
-    if (nvalid == 4) {
-      *reinterpret_cast<float4*>(lam_out.f[0] + off) = make_float4(na[0], na[1], na[2], na[3]);
-      *reinterpret_cast<float4*>(lam_out.f[1] + off) = make_float4(nb[0], nb[1], nb[2], nb[3]);
-    } else {
-      for (int e = 0; e < nvalid; ++e) {
-        lam_out.f[0][off + e] = na[e];
-        lam_out.f[1][off + e] = nb[e];
+  };
+  stage(x, H, B::HP, sm);
+  stage(lam, LEN, 4, la);
+  cp_async_wait_all();
+  __syncthreads();
+  // the block's states: x^{j+1} on the tile plus H - 1 - j sites
+#pragma unroll
+  for (int j = 0; j + 1 < LEN; ++j) {
+    const float* s = sm + 2 * j * PL;
+    float* d = sm + 2 * (j + 1) * PL;
+    const int h = H - 1 - j;
+    const int q0 = -((h + 3) / 4), gpr = kATX / 4 - 2 * q0;
+    for (int i = tid; i < (TY + 2 * h) * gpr; i += NT) {
+      const int r = i / gpr;
+      const int p = B::at(r - h, i - r * gpr + q0);
+      const float4 u = *reinterpret_cast<const float4*>(s + p);
+      const float4 v = *reinterpret_cast<const float4*>(s + PL + p);
+      const float4 lu = lap2d_x4<PF_ST_STD, PF_MODEL_GS>(s, p, WS, 1.0f);
+      const float4 lv = lap2d_x4<PF_ST_STD, PF_MODEL_GS>(s + PL, p, WS, 1.0f);
+      float4 un, vn;
+      gs_update(u.x, v.x, lu.x, lv.x, m, un.x, vn.x);
+      gs_update(u.y, v.y, lu.y, lv.y, m, un.y, vn.y);
+      gs_update(u.z, v.z, lu.z, lv.z, m, un.z, vn.z);
+      gs_update(u.w, v.w, lu.w, lv.w, m, un.w, vn.w);
+      *reinterpret_cast<float4*>(d + p) = un;
+      *reinterpret_cast<float4*>(d + PL + p) = vn;
+    }
+    __syncthreads();
+  }
+  // lambda back through them
+  const int rr = tid / 16, jj = tid % 16;  // the thread's group of the tile
+  const int gy = y0 + rr, gx = x0 + 4 * jj;
+  const int nvalid = gy < g.ny ? (g.nx - gx < 4 ? (g.nx > gx ? g.nx - gx : 0) : 4) : 0;
+#pragma unroll
+  for (int j = LEN - 1; j >= 0; --j) {
+    const float* s = sm + 2 * j * PL;
+    const float* l = la + 2 * ((LEN - 1 - j) & 1) * PL;
+    float* d = la + 2 * ((LEN - j) & 1) * PL;
+    // lambda^{s+j} of the four sites at p
+    auto back = [&](int p, float4& na, float4& nb) {
+      const float4 u4 = *reinterpret_cast<const float4*>(s + p);
+      const float4 v4 = *reinterpret_cast<const float4*>(s + PL + p);
+      const float4 a4 = *reinterpret_cast<const float4*>(l + p);
+      const float4 b4 = *reinterpret_cast<const float4*>(l + PL + p);
+      const float4 la4 = lap2d_x4<PF_ST_STD, PF_MODEL_GS>(l, p, WS, 1.0f);
+      const float4 lb4 = lap2d_x4<PF_ST_STD, PF_MODEL_GS>(l + PL, p, WS, 1.0f);
+      auto site = [&](float u, float v, float a, float b, float lae, float lbe, float& ra,
+                      float& rb) {
+        const float vv = __fmul_rn(v, v);
+        const float uv2 = __fmul_rn(2.0f, __fmul_rn(u, v));
+        // a' = a + dt [Du la - (v^2 + F) a + v^2 b]
+        float fa = __fmaf_rn(-__fadd_rn(vv, m.a2), a, __fmul_rn(vv, b));
+        fa = __fmaf_rn(m.a0, lae, fa);
+        // b' = b + dt [Dv lb - 2uv a + (2uv - F - k) b]
+        float fb = __fmaf_rn(__fsub_rn(uv2, m.a3), b, -__fmul_rn(uv2, a));
+        fb = __fmaf_rn(m.a1, lbe, fb);
+        ra = __fmaf_rn(m.dt, fa, a);
+        rb = __fmaf_rn(m.dt, fb, b);
+      };
+      site(u4.x, v4.x, a4.x, b4.x, la4.x, lb4.x, na.x, nb.x);
+      site(u4.y, v4.y, a4.y, b4.y, la4.y, lb4.y, na.y, nb.y);
+      site(u4.z, v4.z, a4.z, b4.z, la4.z, lb4.z, na.z, nb.z);
+      site(u4.w, v4.w, a4.w, b4.w, la4.w, lb4.w, na.w, nb.w);
+    };
+    if (tid < TILE) {  // the tile, with the gradient terms
+      const int p = B::at(rr, jj);
+      float4 na, nb;
+      back(p, na, nb);
+      if (j > 0) {
+        *reinterpret_cast<float4*>(d + p) = na;
+        *reinterpret_cast<float4*>(d + PL + p) = nb;
+      } else if (nvalid == 4) {
+        const int64_t off = (int64_t)gy * g.pitch + gx;
+        *reinterpret_cast<float4*>(lam_out.f[0] + off) = na;
+        *reinterpret_cast<float4*>(lam_out.f[1] + off) = nb;
+      } else if (nvalid > 0) {
+        const int64_t off = (int64_t)gy * g.pitch + gx;
+        const float ra[3] = {na.x, na.y, na.z}, rb[3] = {nb.x, nb.y, nb.z};
+#pragma unroll
+        for (int e = 0; e < 3; ++e)
+          if (e < nvalid) {
+            lam_out.f[0][off + e] = ra[e];
+            lam_out.f[1][off + e] = rb[e];
+          }
+      }
+      const float4 u4 = *reinterpret_cast<const float4*>(s + p);
+      const float4 v4 = *reinterpret_cast<const float4*>(s + PL + p);
+      const float4 a4 = *reinterpret_cast<const float4*>(l + p);
+      const float4 b4 = *reinterpret_cast<const float4*>(l + PL + p);
+      const float4 lu4 = lap2d_x4<PF_ST_STD, PF_MODEL_GS>(s, p, WS, 1.0f);
+      const float4 lv4 = lap2d_x4<PF_ST_STD, PF_MODEL_GS>(s + PL, p, WS, 1.0f);
+      float t[4] = {0.f, 0.f, 0.f, 0.f};  // Du, Dv, F, k
+      auto term = [&](int e, float u, float v, float a, float b, float lu, float lv) {
+        if (e < nvalid) {
+          t[0] = __fmaf_rn(a, lu, t[0]);
+          t[1] = __fmaf_rn(b, lv, t[1]);
+          t[2] = __fadd_rn(t[2], __fsub_rn(__fmul_rn(__fsub_rn(1.0f, u), a), __fmul_rn(v, b)));
+          t[3] = __fsub_rn(t[3], __fmul_rn(v, b));
+        }
+      };
+      term(0, u4.x, v4.x, a4.x, b4.x, lu4.x, lv4.x);
+      term(1, u4.y, v4.y, a4.y, b4.y, lu4.y, lv4.y);
+      term(2, u4.z, v4.z, a4.z, b4.z, lu4.z, lv4.z);
+      term(3, u4.w, v4.w, a4.w, b4.w, lu4.w, lv4.w);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float w = warp_sum_f(t[q]);
+        if ((tid & 31) == 0) red[j][q][tid >> 5] = w;
+      }
+    } else if (j > 0) {  // the ring of j sites around it: rows above and below, a group a side
+      constexpr int gpr = kATX / 4 + 2;
+      const int nring = 2 * j * gpr + 2 * TY;
+      for (int i = tid - TILE; i < nring; i += NT - TILE) {
+        int r, q;
+        if (i < 2 * j * gpr) {
+          r = i / gpr;
+          q = i - r * gpr - 1;
+          r = r < j ? r - j : TY + r - j;
+        } else {
+          r = (i - 2 * j * gpr) >> 1;
+          q = (i - 2 * j * gpr) & 1 ? kATX / 4 : -1;
+        }
+        const int p = B::at(r, q);
+        float4 na, nb;
+        back(p, na, nb);
+        *reinterpret_cast<float4*>(d + p) = na;
+        *reinterpret_cast<float4*>(d + PL + p) = nb;
       }
     }
+    __syncthreads();
   }
-  double t[4] = {pDu, pDv, pF, pk};
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (tid < 32) {  // the warps' sums per step (side by side: FP64 additions are slow), the steps'
+    if (tid < 4 * LEN) {
+      double v = 0.0;
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    t[q] = warp_sum_f(t[q]);
-    if (lane == 0) red[q][wid] = t[q];
-  }
-  __syncthreads();
-  if (threadIdx.x < 4) {
-    double s = 0.0;
-    for (int w = 0; w < kNT2 / 32; ++w) s += red[threadIdx.x][w];
-    double* slot = gpart + 4 * ((int64_t)blockIdx.y * gridDim.x + blockIdx.x);
-    slot[threadIdx.x] += s;
+      for (int w = 0; w < NW; ++w) v += (double)red[tid >> 2][tid & 3][w];
+      step_sum[tid >> 2][tid & 3] = v;
+    }
+    __syncwarp();
+    if (tid < 4) {
+      double* slot = gpart + 4 * ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) + tid;
+      double t = *slot;
+#pragma unroll
+      for (int j = LEN - 1; j >= 0; --j) t += step_sum[j][tid];
+      *slot = t;
+    }
   }
 }
 
-// Add this CTA's per-thread sums t[0..NG) into its FP64 slot (fixed order).
-template <int NG>
-__device__ __forceinline__ void add_to_slot(double (&t)[4], double (&red)[4][kNT2 / 32],
-                                            double* gpart) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int q = 0; q < NG; ++q) {
-    t[q] = warp_sum_f(t[q]);
-    if (lane == 0) red[q][wid] = t[q];
-  }
-  __syncthreads();
-  if (threadIdx.x < NG) {
-    double s = 0.0;
-    for (int w = 0; w < kNT2 / 32; ++w) s += red[threadIdx.x][w];
-    gpart[4 * ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) + threadIdx.x] += s;
-  }
+template <int LEN>
+cudaError_t launch_gs_block(dim3 grid, const FieldPtrs& x, const FieldPtrs& lam,
+                            const FieldOut& out, const Geom& g, const ModelParams& m,
+                            double* gpart, cudaStream_t st) {
+  using B = AdjBlock<LEN>;
+  constexpr size_t smem = sizeof(float) * B::SMEM_FLOATS;
+  static unsigned long long attr_mask = 0;  // per instantiation and device
+  cudaError_t e = ensure_smem_attr(adj_gs2d_kernel<LEN>, smem, &attr_mask);
+  if (e != cudaSuccess) return e;
+  return launch_chained(adj_gs2d_kernel<LEN>, grid, B::NT, smem, st, x, lam, out, g, m, gpart);
 }
 
-// Model A reverse step on a tile (halo 1 of x = phi^n and lambda^{n+1}).
-__global__ void __launch_bounds__(kNT2) adj_ac2d_kernel(FieldPtrs x, FieldPtrs lam,
-                                                        FieldOut lam_out, Geom g,
-                                                        ModelParams m, double* gpart) {
-  __shared__ float sp[kAPL], sl[kAPL];
-  __shared__ double red[4][kNT2 / 32];
-  const int x0 = blockIdx.x * kATX;
-  const int y0 = blockIdx.y * kATY;
-  canary_fill(sp, kAPL);
-  canary_fill(sl, kAPL);
-  for (int i = threadIdx.x; i < kAPL; i += kNT2) {
-    const int r = i / kAW;
-    const int c = i - r * kAW;
-    const int64_t off =
-        (int64_t)wrap_index(y0 - 1 + r, g.ny) * g.pitch + wrap_index(x0 - 1 + c, g.nx);
-    cp_async4(&sp[i], x.f[0] + off);
-    cp_async4(&sl[i], lam.f[0] + off);
-  }
+// LEN reverse steps of Model A or B on a 64 x 16 tile in one launch: the block of
+// adj_gs2d_kernel for one field. A step, forward or reverse, reaches R sites (Model B: 2, through
+// mu and through w = lap lambda, which pass through one more plane of shared memory); Model B's
+// blocks are two steps long, since four would stage a halo of 12. The gradient terms are summed
+// per thread over four sites (every fourth row), per warp (half a row) in float, then in FP64.
+//
+// Bound by latency on small grids and by shared memory on large ones, as the Gray-Scott blocks.
+// Reverse pass of 400 steps, against one launch per step with the states recomputed on a second
+// stream: Model A 64^2 1.07 -> 0.61 ms, 512^2 1.42 -> 0.78, 2048^2 7.9 -> 5.8; Model B 64^2
+// 1.28 -> 0.99, 512^2 2.09 -> 1.25, 2048^2 11.4 -> 9.0. 256 threads and four CTAs per SM: with a
+// thread for every group of the widest region instead (544 and 416) 512^2 takes 0.93 and 1.53,
+// 2048^2 6.2 and 10.1.
+template <int MODEL, int LEN>
+struct AdjBlock1 {
+  static constexpr int R = MODEL == PF_MODEL_CH ? 2 : 1;
+  static constexpr int NG = MODEL == PF_MODEL_CH ? 3 : 2;        // gradient sums
+  static constexpr int HX = LEN > 1 ? 2 * R * (LEN - 1) : 1;     // staged halo of the state
+  static constexpr int HL = R * LEN;                             // and of lambda
+  static constexpr int H = HX > HL ? HX : HL;
+  static constexpr int HP = (H + 3) / 4 * 4;
+  static constexpr int WS = kATX + 2 * HP, ROWS = kATY + 2 * H;
+  static constexpr int PL = WS * ROWS;
+  static constexpr int NL = MODEL == PF_MODEL_CH ? 1 : 2;        // lambda buffers (B: in place)
+  static constexpr int SMEM_FLOATS = (LEN + NL + (MODEL == PF_MODEL_CH ? 1 : 0)) * PL;
+  static __device__ __forceinline__ int at(int r, int c) { return (r + H) * WS + HP + c; }
+};
+
+template <int MODEL, int LEN>
+__global__ void __launch_bounds__(kNT2, 4)
+    adj_one2d_kernel(FieldPtrs x, FieldPtrs lam, FieldOut lam_out, Geom g, ModelParams m,
+                     double* gpart) {
+  using B = AdjBlock1<MODEL, LEN>;
+  constexpr bool CH = MODEL == PF_MODEL_CH;
+  constexpr int WS = B::WS, PL = B::PL, NT = kNT2, R = B::R, NG = B::NG;
+  constexpr int NW = NT / 32;
+  extern __shared__ __align__(16) float sm[];  // state j at j PL
+  __shared__ float red[LEN][NG][NW];
+  __shared__ double step_sum[LEN][NG];
+  float* la = sm + LEN * PL;         // lambda (Model A: twice)
+  float* sw = la + B::NL * PL;       // Model B: mu, then w
+  const int tid = threadIdx.x;
+  const int x0 = blockIdx.x * kATX, y0 = blockIdx.y * kATY;
+  canary_fill(sm, B::SMEM_FLOATS);
+  chain_wait();
+  // f(p, r, q) for the groups of the tile and h sites around it
+  auto region = [&](int h, auto f) {
+    const int q0 = -((h + 3) / 4), gpr = kATX / 4 - 2 * q0;
+    for (int i = tid; i < (kATY + 2 * h) * gpr; i += NT) {
+      const int r = i / gpr - h, q = i % gpr + q0;
+      f(B::at(r, 4 * q), r, q);
+    }
+  };
+  auto stage = [&](const float* in, int h, float* dst) {
+    region(h, [&](int p, int r, int q) {
+      const float* row = in + (int64_t)wrap_index(y0 + r, g.ny) * g.pitch;
+      const int gx = x0 + 4 * q;
+      if (gx >= 0 && gx + 3 < g.nx) {
+        cp_async16(dst + p, row + gx);
+      } else {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) cp_async4(dst + p + c, row + wrap_index(gx + c, g.nx));
+      }
+    });
+  };
+  stage(x.f[0], B::HX, sm);
+  stage(lam.f[0], B::HL, la);
   cp_async_wait_all();
   __syncthreads();
-  const float c2x3 = __fmul_rn(3.0f, m.a1);
-  float s0 = 0.f, s1 = 0.f;
-  for (int i = threadIdx.x; i < kATX * kATY; i += kNT2) {
-    const int rr = i / kATX;
-    const int cc = i - rr * kATX;
-    const int gx = x0 + cc, gy = y0 + rr;
-    if (gx >= g.nx || gy >= g.ny) continue;
-    const int p = (rr + 1) * kAW + (cc + 1);
-    const float ph = sp[p], l = sl[p];
-    const float ll = lap2d(l, sl[p - 1], sl[p + 1], sl[p - kAW], sl[p + kAW], m.lap_scale);
-    const float sfac = __fmaf_rn(-c2x3, __fmul_rn(ph, ph), m.a0);  // c1 - 3 c2 phi^2
-    const float f = __fmaf_rn(sfac, l, ll);
-    lam_out.f[0][(int64_t)gy * g.pitch + gx] = __fmaf_rn(m.dt, f, l);
-    const float lp = __fmul_rn(l, ph);
-    s0 = __fadd_rn(s0, lp);
-    s1 = __fmaf_rn(lp, __fmul_rn(ph, ph), s1);
+  // the block's states: x^{j+1} on the tile plus HX - R (j + 1) sites
+#pragma unroll
+  for (int j = 0; j + 1 < LEN; ++j) {
+    const float* s = sm + j * PL;
+    float* d = sm + (j + 1) * PL;
+    const int h = B::HX - R * (j + 1);
+    if constexpr (CH) {
+      region(h + 1, [&](int p, int, int) {
+        site4_mu<MODEL, PF_ST_STD>(s, p, WS, PL, m, sw);
+      });
+      __syncthreads();
+    }
+    region(h, [&](int p, int, int) {
+      float4 v[1];
+      site4_update<MODEL, PF_ST_STD>(s, sw, p, WS, PL, m, v);
+      *reinterpret_cast<float4*>(d + p) = v[0];
+    });
+    __syncthreads();
   }
-  double t[4] = {s0, s1, 0.0, 0.0};
-  add_to_slot<2>(t, red, gpart);
+  // lambda back through them
+  const float c2x3 = __fmul_rn(3.0f, m.a1);
+#pragma unroll
+  for (int j = LEN - 1; j >= 0; --j) {
+    const float* s = sm + j * PL;
+    const float* l = CH ? la : la + ((LEN - 1 - j) & 1) * PL;
+    float* d = CH ? la : la + ((LEN - j) & 1) * PL;
+    if constexpr (CH) {  // w = lap lambda^{s+j+1}
+      region(R * j + 1, [&](int p, int, int) {
+        *reinterpret_cast<float4*>(sw + p) = lap2d_x4(l, p, WS, m.lap_scale);
+      });
+      __syncthreads();
+    }
+    // lambda^{s+j} on the tile plus R j sites
+    region(R * j, [&](int p, int r, int q) {
+      const float4 p4 = *reinterpret_cast<const float4*>(s + p);
+      const float4 l4 = *reinterpret_cast<const float4*>(l + p);
+      float4 n;
+      if constexpr (CH) {  // + dt M [(3 c2 x^2 - c1) w - lap w]
+        const float4 w4 = *reinterpret_cast<const float4*>(sw + p);
+        const float4 lw = lap2d_x4(sw, p, WS, m.lap_scale);
+        auto site = [&](float ph, float la_, float w, float lwe) {
+          const float sfac = __fmaf_rn(c2x3, __fmul_rn(ph, ph), -m.a0);
+          return __fmaf_rn(m.a2, __fmaf_rn(sfac, w, -lwe), la_);
+        };
+        n = make_float4(site(p4.x, l4.x, w4.x, lw.x), site(p4.y, l4.y, w4.y, lw.y),
+                        site(p4.z, l4.z, w4.z, lw.z), site(p4.w, l4.w, w4.w, lw.w));
+      } else {  // + dt [lap lambda + (c1 - 3 c2 x^2) lambda]
+        const float4 ll = lap2d_x4(l, p, WS, m.lap_scale);
+        auto site = [&](float ph, float la_, float lle) {
+          const float sfac = __fmaf_rn(-c2x3, __fmul_rn(ph, ph), m.a0);
+          return __fmaf_rn(m.dt, __fmaf_rn(sfac, la_, lle), la_);
+        };
+        n = make_float4(site(p4.x, l4.x, ll.x), site(p4.y, l4.y, ll.y),
+                        site(p4.z, l4.z, ll.z), site(p4.w, l4.w, ll.w));
+      }
+      if (j > 0) {
+        *reinterpret_cast<float4*>(d + p) = n;
+      } else {
+        const int gy = y0 + r, gx = x0 + 4 * q;
+        if (gy < g.ny && gx < g.nx) {
+          float* o = lam_out.f[0] + (int64_t)gy * g.pitch + gx;
+          if (gx + 3 < g.nx) {
+            *reinterpret_cast<float4*>(o) = n;
+          } else {
+            const float e[3] = {n.x, n.y, n.z};
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+              if (gx + c < g.nx) o[c] = e[c];
+          }
+        }
+      }
+    });
+    float acc[NG] = {};  // the gradient terms
+#pragma unroll
+    for (int k = 0; k < kATX * kATY / NT; ++k) {
+      const int rr = (tid + NT * k) / kATX, cc = tid % kATX;
+      if (x0 + cc < g.nx && y0 + rr < g.ny) {
+        const int p = B::at(rr, cc);
+        const float ph = s[p], ph2 = __fmul_rn(ph, ph);
+        if constexpr (CH) {
+          const float w = sw[p];
+          const float mu =
+              ch_mu(ph, lap2d(ph, s[p - 1], s[p + 1], s[p - WS], s[p + WS], m.lap_scale), m);
+          const float wp = __fmul_rn(w, ph);
+          acc[0] = __fadd_rn(acc[0], wp);
+          acc[1] = __fmaf_rn(wp, ph2, acc[1]);
+          acc[2] = __fmaf_rn(w, mu, acc[2]);
+        } else {
+          const float lp = __fmul_rn(l[p], ph);
+          acc[0] = __fadd_rn(acc[0], lp);
+          acc[1] = __fmaf_rn(lp, ph2, acc[1]);
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < NG; ++q) {
+      const float w = warp_sum_f(acc[q]);
+      if ((tid & 31) == 0) red[j][q][tid >> 5] = w;
+    }
+    __syncthreads();
+  }
+  if (tid < 32) {  // the warps' sums per step, then the steps'
+    if (tid < NG * LEN) {
+      double v = 0.0;
+#pragma unroll
+      for (int w = 0; w < NW; ++w) v += (double)red[tid / NG][tid % NG][w];
+      step_sum[tid / NG][tid % NG] = v;
+    }
+    __syncwarp();
+    if (tid < NG) {
+      double* slot = gpart + 4 * ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) + tid;
+      double t = *slot;
+#pragma unroll
+      for (int j = LEN - 1; j >= 0; --j) t += step_sum[j][tid];
+      *slot = t;
+    }
+  }
 }
 
-// Model B reverse step on a tile: stage phi^n and lambda^{n+1} with a halo of 2, form
-// w = lap lambda on the tile plus one ring, then lambda^n on the tile.
-constexpr int kBW = kATX + 4, kBH = kATY + 4, kBPL = kBW * kBH;
-__global__ void __launch_bounds__(kNT2) adj_ch2d_kernel(FieldPtrs x, FieldPtrs lam,
-                                                        FieldOut lam_out, Geom g,
-                                                        ModelParams m, double* gpart) {
-  __shared__ float sp[kBPL], sl[kBPL], sw[kBPL];
-  __shared__ double red[4][kNT2 / 32];
-  const int x0 = blockIdx.x * kATX;
-  const int y0 = blockIdx.y * kATY;
-  canary_fill(sp, kBPL);
-  canary_fill(sl, kBPL);
-  canary_fill(sw, kBPL);
-  for (int i = threadIdx.x; i < kBPL; i += kNT2) {
-    const int r = i / kBW;
-    const int c = i - r * kBW;
-    const int64_t off =
-        (int64_t)wrap_index(y0 - 2 + r, g.ny) * g.pitch + wrap_index(x0 - 2 + c, g.nx);
-    cp_async4(&sp[i], x.f[0] + off);
-    cp_async4(&sl[i], lam.f[0] + off);
+template <int MODEL, int LEN>
+cudaError_t launch_one_block(dim3 grid, const FieldPtrs& x, const FieldPtrs& lam,
+                             const FieldOut& out, const Geom& g, const ModelParams& m,
+                             double* gpart, cudaStream_t st) {
+  using B = AdjBlock1<MODEL, LEN>;
+  constexpr size_t smem = sizeof(float) * B::SMEM_FLOATS;
+  static unsigned long long attr_mask = 0;  // per instantiation and device
+  cudaError_t e = ensure_smem_attr(adj_one2d_kernel<MODEL, LEN>, smem, &attr_mask);
+  if (e != cudaSuccess) return e;
+  return launch_chained(adj_one2d_kernel<MODEL, LEN>, grid, kNT2, smem, st, x, lam, out, g, m,
+                        gpart);
+}
+
+// One block of len reverse steps
+cudaError_t launch_block(int model, int len, dim3 grid, const FieldPtrs& x, const FieldPtrs& lam,
+                         const FieldOut& out, const Geom& g, const ModelParams& m, double* gpart,
+                         cudaStream_t st) {
+  constexpr int A = PF_MODEL_AC, B = PF_MODEL_CH;
+  if (model == PF_MODEL_GS) {
+    switch (len) {
+      case 1: return launch_gs_block<1>(grid, x, lam, out, g, m, gpart, st);
+      case 2: return launch_gs_block<2>(grid, x, lam, out, g, m, gpart, st);
+      case 3: return launch_gs_block<3>(grid, x, lam, out, g, m, gpart, st);
+      case 4: return launch_gs_block<4>(grid, x, lam, out, g, m, gpart, st);
+    }
+  } else if (model == PF_MODEL_AC) {
+    switch (len) {
+      case 1: return launch_one_block<A, 1>(grid, x, lam, out, g, m, gpart, st);
+      case 2: return launch_one_block<A, 2>(grid, x, lam, out, g, m, gpart, st);
+      case 3: return launch_one_block<A, 3>(grid, x, lam, out, g, m, gpart, st);
+      case 4: return launch_one_block<A, 4>(grid, x, lam, out, g, m, gpart, st);
+    }
+  } else if (model == PF_MODEL_CH) {
+    switch (len) {
+      case 1: return launch_one_block<B, 1>(grid, x, lam, out, g, m, gpart, st);
+      case 2: return launch_one_block<B, 2>(grid, x, lam, out, g, m, gpart, st);
+    }
   }
-  cp_async_wait_all();
-  __syncthreads();
-  // w on rows/cols 1 .. kBH-2 / kBW-2 (the tile and one ring)
-  for (int i = threadIdx.x; i < (kATX + 2) * (kATY + 2); i += kNT2) {
-    const int r = 1 + i / (kATX + 2);
-    const int c = 1 + i % (kATX + 2);
-    const int p = r * kBW + c;
-    sw[p] = lap2d(sl[p], sl[p - 1], sl[p + 1], sl[p - kBW], sl[p + kBW], m.lap_scale);
-  }
-  __syncthreads();
-  const float c2x3 = __fmul_rn(3.0f, m.a1);
-  float s0 = 0.f, s1 = 0.f, s2 = 0.f;
-  for (int i = threadIdx.x; i < kATX * kATY; i += kNT2) {
-    const int rr = i / kATX;
-    const int cc = i - rr * kATX;
-    const int gx = x0 + cc, gy = y0 + rr;
-    if (gx >= g.nx || gy >= g.ny) continue;
-    const int p = (rr + 2) * kBW + (cc + 2);
-    const float ph = sp[p], l = sl[p], w = sw[p];
-    const float lw = lap2d(w, sw[p - 1], sw[p + 1], sw[p - kBW], sw[p + kBW], m.lap_scale);
-    const float ph2 = __fmul_rn(ph, ph);
-    const float sfac = __fmaf_rn(c2x3, ph2, -m.a0);  // 3 c2 phi^2 - c1
-    const float f = __fmaf_rn(sfac, w, -lw);
-    lam_out.f[0][(int64_t)gy * g.pitch + gx] = __fmaf_rn(m.a2, f, l);  // a2 = dt M
-    const float lph = lap2d(ph, sp[p - 1], sp[p + 1], sp[p - kBW], sp[p + kBW], m.lap_scale);
-    const float mu = ch_mu(ph, lph, m);
-    const float wp = __fmul_rn(w, ph);
-    s0 = __fadd_rn(s0, wp);
-    s1 = __fmaf_rn(wp, ph2, s1);
-    s2 = __fmaf_rn(w, mu, s2);
-  }
-  double t[4] = {s0, s1, s2, 0.0};
-  add_to_slot<3>(t, red, gpart);
+  return cudaErrorInvalidValue;
 }
 
 // out[q] = sum over CTAs of gpart[4 * cta + q], in CTA order split over 256 threads.
@@ -290,35 +547,21 @@ __global__ void __launch_bounds__(256) adj_final_kernel(const double* gpart, int
   }
 }
 
-// Tile height of the Gray-Scott reverse step on this grid (see adj_gs2d_kernel): 8 when
-// 16-row tiles would give fewer than four per SM, else 16.
-int gs_adj_ty(const Geom& q, int device) {
-  static int sms_by_dev[64] = {};
-  int sms = device >= 0 && device < 64 ? sms_by_dev[device] : 0;
-  if (sms == 0) {
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
-      cudaGetLastError();
-      sms = 1;
-    } else if (device >= 0 && device < 64) {
-      sms_by_dev[device] = sms;
-    }
-  }
-  const int64_t tiles16 = (int64_t)((q.nx + kATX - 1) / kATX) * ((q.ny + 15) / 16);
-  return tiles16 < 4 * (int64_t)sms ? 8 : 16;
-}
+// Steps per reverse launch: states at the blocks' first steps are stored or recomputed, those
+// between live only inside a launch.
+int block_len(int model) { return model == PF_MODEL_CH ? 2 : 4; }
 
-// Reverse-step launch grid for the grid's model.
+// Reverse-step launch grid (the same tiles for every model).
 dim3 adj_grid(const pf_grid_s* g) {
   const Geom q = grid_geom(g);
-  const int ty = g->model == PF_MODEL_GS ? gs_adj_ty(q, g->device) : kATY;
-  return dim3((q.nx + kATX - 1) / kATX, (q.ny + ty - 1) / ty, 1);
+  return dim3((q.nx + kATX - 1) / kATX, (q.ny + kATY - 1) / kATY, 1);
 }
 
 float* ckpt_field(pf_grid_s* g, int64_t i, int f) {
   return g->adj.ckpt + (i * g->nf + f) * g->field_elems;
 }
-float* seg_field(pf_grid_s* g, int b, int64_t j, int f) {
-  return g->adj.seg + (((int64_t)b * (g->adj.interval - 1) + j) * g->nf + f) * g->field_elems;
+float* seg_field(pf_grid_s* g, int64_t j, int f) {
+  return g->adj.seg + (j * g->nf + f) * g->field_elems;
 }
 float* lam_field(pf_grid_s* g, int b, int f) {
   return g->adj.lam + (b * g->nf + f) * g->field_elems;
@@ -342,104 +585,102 @@ void adjoint_release(pf_grid_s* g) {
   if (a.ckpt) cudaFree(a.ckpt);
   if (a.seg) cudaFree(a.seg);
   if (a.lam) cudaFree(a.lam);
-  if (a.gpart) cudaFree(a.gpart);
-  if (a.gout) cudaFree(a.gout);
-  if (a.ghost) cudaFreeHost(a.ghost);
   a = AdjointState();
 }
 
-// Enqueue the whole reverse pass on stream st, which the caller is recording into a graph:
-// zero the gradient slots, then per segment from last to first recompute its states and
-// run its reverse steps, then sum the slots. *lb_out receives the buffer holding lambda^0.
-//
-// Two branches: the reverse steps on st, the recomputation on st2 (forked into the same
-// capture). With two segment buffers, segment s - 1 is recomputed into one buffer while
-// segment s's reverse steps read the other, so the two chains of small launches overlap:
-// recomputing segment s waits for its checkpoint only and for the reverse steps of segment
-// s + 2 (the last reader of its buffer); the reverse steps of segment s wait for its
-// recomputation. Each chain keeps its order, so every kernel sees the same inputs as in a
-// serial pass and the result is the same bits.
+// Enqueue the whole reverse pass on stream st: zero the gradient slots, then per segment from
+// last to first recompute its blocks' first states from its checkpoint and run its reverse
+// blocks, then sum the slots. *lb_out receives the buffer holding lambda^0.
 static cudaError_t enqueue_reverse(pf_grid_s* g, const ModelParams& m, cudaStream_t st,
-                                   cudaStream_t st2, int* lb_out) {
+                                   int* lb_out) {
   AdjointState& a = g->adj;
   const Geom q = grid_geom(g);
   const dim3 grid = adj_grid(g);
-  const int gs_ty = gs_adj_ty(q, g->device);
   const int64_t nctas = (int64_t)grid.x * grid.y;
   const int64_t C = a.interval;
-  const int nb = a.seg_bufs > 0 ? a.seg_bufs : 1;
-  // per segment: its recomputation done (on st2), its reverse steps done (on st)
-  std::vector<cudaEvent_t> rec((size_t)a.n_ckpt, nullptr), rev((size_t)a.n_ckpt, nullptr);
-  cudaEvent_t fork = nullptr, join = nullptr;
-  cudaError_t e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&join, cudaEventDisableTiming);
-  for (int64_t s = 0; s < a.n_ckpt && e == cudaSuccess; ++s) {
-    e = cudaEventCreateWithFlags(&rec[(size_t)s], cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&rev[(size_t)s], cudaEventDisableTiming);
-  }
-  if (e == cudaSuccess) e = cudaEventRecord(fork, st);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(st2, fork, 0);
-  if (e == cudaSuccess) e = cudaMemsetAsync(a.gpart, 0, sizeof(double) * 4 * nctas, st);
+  const int B = block_len(g->model);
+  int tile = 0, depth = 1;
+  plan2d(g, &tile, &depth);  // (depth: B)
+  cudaError_t e = cudaMemsetAsync(a.gpart, 0, sizeof(double) * 4 * nctas, st);
   int lb = 0;  // lambda ping-pong buffer holding the current adjoint state
   for (int64_t s = a.n_ckpt - 1; s >= 0 && e == cudaSuccess; --s) {
-    const int64_t s0 = s * C;
-    const int64_t len = std::min(C, a.n_steps - s0);
-    const int b = (int)(s % nb);
-    // states x^{s0} .. x^{s0+len-1}: slot 0 is the checkpoint, slots 1.. are recomputed
-    auto state = [&](int64_t j, int f) -> float* {
-      return j == 0 ? ckpt_field(g, s, f) : seg_field(g, b, j - 1, f);
+    const int64_t len = std::min(C, a.n_steps - s * C);
+    const int64_t nb = (len + B - 1) / B;  // blocks
+    // first state of block b: the checkpoint, or recomputed
+    auto state = [&](int64_t b, int f) -> float* {
+      return b == 0 ? ckpt_field(g, s, f) : seg_field(g, b - 1, f);
     };
-    // recompute on st2, once the buffer's previous reader (segment s + nb) is done
-    if (s + nb < a.n_ckpt) e = cudaStreamWaitEvent(st2, rev[(size_t)(s + nb)], 0);
-    for (int64_t j = 1; j < len && e == cudaSuccess; ++j) {
+    for (int64_t b = 1; b < nb && e == cudaSuccess; ++b) {
       FieldPtrs in{};
       FieldOut out{};
       for (int f = 0; f < g->nf; ++f) {
-        in.f[f] = state(j - 1, f);
-        out.f[f] = state(j, f);
+        in.f[f] = state(b - 1, f);
+        out.f[f] = state(b, f);
       }
-      e = launch_fe2d(g->model, 0, 1, q, in, out, m, st2);
+      e = launch_2d(g, tile, B, in, out, m, st);
     }
-    if (e == cudaSuccess) e = cudaEventRecord(rec[(size_t)s], st2);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, rec[(size_t)s], 0);
-    for (int64_t j = len - 1; j >= 0 && e == cudaSuccess; --j) {
+    for (int64_t b = nb - 1; b >= 0 && e == cudaSuccess; --b) {
       FieldPtrs xs{}, li{};
       FieldOut lo{};
       for (int f = 0; f < g->nf; ++f) {
-        xs.f[f] = state(j, f);
+        xs.f[f] = state(b, f);
         li.f[f] = lam_field(g, lb, f);
         lo.f[f] = lam_field(g, 1 - lb, f);
       }
-      if (g->model == PF_MODEL_GS)
-        if (gs_ty == 8)
-          adj_gs2d_kernel<8><<<grid, kNT2, 0, st>>>(xs, li, lo, q, m, a.gpart);
-        else
-          adj_gs2d_kernel<16><<<grid, kNT2, 0, st>>>(xs, li, lo, q, m, a.gpart);
-      else if (g->model == PF_MODEL_AC)
-        adj_ac2d_kernel<<<grid, kNT2, 0, st>>>(xs, li, lo, q, m, a.gpart);
-      else
-        adj_ch2d_kernel<<<grid, kNT2, 0, st>>>(xs, li, lo, q, m, a.gpart);
-      e = cudaGetLastError();
+      const int n = (int)std::min<int64_t>(B, len - b * B);
+      e = launch_block(g->model, n, grid, xs, li, lo, q, m, a.gpart, st);
       lb = 1 - lb;
     }
-    if (e == cudaSuccess) e = cudaEventRecord(rev[(size_t)s], st);
   }
-  // join the second branch before the capture ends (also on an error, so that it can end)
-  cudaError_t ej = cudaEventRecord(join, st2);
-  if (ej == cudaSuccess) ej = cudaStreamWaitEvent(st, join, 0);
-  if (e == cudaSuccess) e = ej;
   if (e == cudaSuccess) {
     adj_final_kernel<<<1, 256, 0, st>>>(a.gpart, nctas, a.gout);
     e = cudaGetLastError();
   }
-  for (cudaEvent_t ev : rec)
-    if (ev) cudaEventDestroy(ev);
-  for (cudaEvent_t ev : rev)
-    if (ev) cudaEventDestroy(ev);
-  if (fork) cudaEventDestroy(fork);
-  if (join) cudaEventDestroy(join);
   *lb_out = lb;
   return e;
+}
+
+// Steps the grid's state from checkpoint 0 (set by the caller) through all n_steps, every segment
+// from its checkpoint into the next one without a copy between; the result lands in a grid
+// buffer. For the kernels that take any buffers; the on-chip ones run per segment, with copies,
+// where segments are long enough for the state's way in and out of the chip (400 steps of GS 128^2
+// with the cluster kernel: 0.45 ms in segments of 20, 1.03 in segments of 4, tiles 0.50 in either).
+static int forward_segments(pf_grid_s* g, int64_t n_steps, int64_t C, int64_t n_ckpt) {
+  int tile = 0, depth = 1;
+  run_plan(g, &tile, &depth);
+  const size_t state = sizeof(float) * g->nf * g->field_elems;
+  const bool on_chip = tile == kTileCluster2D || tile == kTileBands2D;
+  if (on_chip && C < 16) {
+    plan2d(g, &tile, &depth);
+  } else if (on_chip) {
+    for (int64_t s = 0; s < n_ckpt; ++s) {
+      if (s > 0)
+        PF_CUDA_TRY(cudaMemcpyAsync(ckpt_field(g, s, 0), g->buf[g->cur][0], state,
+                                    cudaMemcpyDeviceToDevice, g->stream));
+      if (int rc = pf_step(g, std::min(C, n_steps - s * C))) return rc;
+    }
+    return PF_OK;
+  }
+  int last = g->cur;  // the grid buffer written last
+  for (int64_t s = 0; s < n_ckpt; ++s) {
+    FieldPtrs in{};
+    for (int f = 0; f < g->nf; ++f) in.f[f] = ckpt_field(g, s, f);
+    int64_t left = std::min(C, n_steps - s * C);
+    while (left > 0) {
+      int k = depth;
+      while (k > left) k >>= 1;
+      left -= k;
+      FieldOut out{};
+      const bool to_ckpt = left == 0 && s + 1 < n_ckpt;
+      if (!to_ckpt) last = 1 - last;
+      for (int f = 0; f < g->nf; ++f)
+        out.f[f] = to_ckpt ? ckpt_field(g, s + 1, f) : g->buf[last][f];
+      PF_CUDA_TRY(launch_2d(g, tile, k, in, out, g->params, g->stream));
+      for (int f = 0; f < g->nf; ++f) in.f[f] = out.f[f];
+    }
+  }
+  g->cur = last;
+  return PF_OK;
 }
 
 }  // namespace pf
@@ -454,54 +695,58 @@ int pf_adj_forward(pf_grid_t g, int64_t n_steps, int64_t ckpt_interval) {
   if (int rc = check_gs2d(g)) return rc;
   if (n_steps < 1) return invalid("n_steps must be >= 1");
   if (ckpt_interval < 0) return invalid("ckpt_interval must be >= 0");
-  int64_t C = ckpt_interval > 0 ? ckpt_interval : (int64_t)std::ceil(std::sqrt((double)n_steps));
-  if (C > n_steps) C = n_steps;
-  const int64_t n_ckpt = (n_steps + C - 1) / C;
   AdjointState& a = g->adj;
   const size_t state = sizeof(float) * g->nf * g->field_elems;
+  const int B = block_len(g->model);
+  // The library's choice: every block's first state where they fit kAllStates bytes (nothing to
+  // recompute between blocks then), else sqrt(N) checkpoints.
+  const int64_t root = (int64_t)std::ceil(std::sqrt((double)n_steps));
+  const bool all = (double)((n_steps + B - 1) / B) * (double)state <= kAllStates;
+  int64_t C = ckpt_interval > 0 ? ckpt_interval : all ? B : root;
+  if (C > n_steps) C = n_steps;
+  int64_t n_ckpt = (n_steps + C - 1) / C;
   if (a.n_ckpt != n_ckpt || a.interval != C) {
-    // (re)allocate for this schedule
+    // (re)allocate for this schedule; a recorded pass or graph of the old one is void
+    a.ready = 0;
+    if (g->adj_exec) cudaGraphExecDestroy(g->adj_exec);
+    g->adj_exec = nullptr;
+    g->adj_exec_steps = -1;
     if (a.ckpt) cudaFree(a.ckpt);
     if (a.seg) cudaFree(a.seg);
     a.ckpt = nullptr;
     a.seg = nullptr;
-    a.seg_bufs = 0;
-    PF_CUDA_TRY(cudaMalloc(&a.ckpt, state * n_ckpt));
-    if (C > 1) {
-      // two segment buffers where there are two segments and the memory allows, else one
-      // (the reverse pass then recomputes and reverses one segment after the other)
-      if (n_ckpt > 1 && cudaMalloc(&a.seg, 2 * state * (C - 1)) == cudaSuccess) {
-        a.seg_bufs = 2;
-      } else {
-        cudaGetLastError();  // a failed first try leaves no sticky error
-        PF_CUDA_TRY(cudaMalloc(&a.seg, state * (C - 1)));
-        a.seg_bufs = 1;
-      }
+    a.n_ckpt = 0;
+    cudaError_t e = cudaMalloc(&a.ckpt, state * n_ckpt);
+    if (e != cudaSuccess && ckpt_interval == 0 && C < root) {
+      cudaGetLastError();  // no room for all of them
+      C = root < n_steps ? root : n_steps;
+      n_ckpt = (n_steps + C - 1) / C;
+      e = cudaMalloc(&a.ckpt, state * n_ckpt);
     }
+    if (e != cudaSuccess) return cuda_fail(e, "pf_adj_forward checkpoints");
+    if (C > B) PF_CUDA_TRY(cudaMalloc(&a.seg, state * ((C + B - 1) / B - 1)));
     a.n_ckpt = n_ckpt;
     a.interval = C;
   }
-  if (a.lam == nullptr) {
-    PF_CUDA_TRY(cudaMalloc(&a.lam, 2 * state));
+  if (a.lam == nullptr) {  // lambda twice, the gradient slots of every CTA and the four sums
+    const dim3 grid = adj_grid(g);
+    const int64_t nctas = (int64_t)grid.x * grid.y;
+    const size_t lam = (2 * state + 255) / 256 * 256;
+    PF_CUDA_TRY(cudaMalloc(&a.lam, lam + sizeof(double) * (4 * nctas + 4)));
     PF_CUDA_TRY(cudaMemsetAsync(a.lam, 0, 2 * state, g->stream));
+    a.gpart = reinterpret_cast<double*>(reinterpret_cast<char*>(a.lam) + lam);
+    a.gout = a.gpart + 4 * nctas;
   }
-  const dim3 grid = adj_grid(g);
-  const int64_t nctas = (int64_t)grid.x * grid.y;
-  if (a.gpart_cap < nctas) {
-    if (a.gpart) cudaFree(a.gpart);
-    a.gpart = nullptr;
-    PF_CUDA_TRY(cudaMalloc(&a.gpart, sizeof(double) * 4 * nctas));
-    a.gpart_cap = nctas;
-  }
-  if (a.gout == nullptr) PF_CUDA_TRY(cudaMalloc(&a.gout, sizeof(double) * 4));
-  if (a.ghost == nullptr) PF_CUDA_TRY(cudaMallocHost(&a.ghost, sizeof(double) * 4));
-  for (int64_t s = 0; s < n_ckpt; ++s) {
-    for (int f = 0; f < g->nf; ++f)
-      PF_CUDA_TRY(cudaMemcpyAsync(ckpt_field(g, s, f), g->buf[g->cur][f],
-                                  sizeof(float) * g->field_elems, cudaMemcpyDeviceToDevice,
-                                  g->stream));
-    const int64_t len = std::min(C, n_steps - s * C);
-    if (int rc = pf_step(g, len)) return rc;
+  // (a grid buffer's fields lie one after the other, as a checkpoint's)
+  PF_CUDA_TRY(cudaMemcpyAsync(ckpt_field(g, 0, 0), g->buf[g->cur][0], state,
+                              cudaMemcpyDeviceToDevice, g->stream));
+  if (int rc = forward_segments(g, n_steps, C, n_ckpt)) return rc;
+  bool same = a.dt == g->dt;
+  for (int i = 0; i < 4; ++i) same = same && a.coeffs[i] == g->coeffs[i];
+  if (!same) {  // a recorded graph carries the old coefficients
+    if (g->adj_exec) cudaGraphExecDestroy(g->adj_exec);
+    g->adj_exec = nullptr;
+    g->adj_exec_steps = -1;
   }
   for (int i = 0; i < 4; ++i) a.coeffs[i] = g->coeffs[i];
   a.dt = g->dt;
@@ -530,36 +775,39 @@ int pf_adj_backward(pf_grid_t g, const float* dLdu_N, const float* dLdv_N, int o
   for (int f = 0; f < g->nf; ++f)
     PF_CUDA_TRY(cudaMemcpy2DAsync(lam_field(g, 0, f), sizeof(float) * g->pitch, src[f], w, w,
                                   (size_t)g->ny, kin, g->stream));
-  if (g->adj_exec == nullptr || g->adj_exec_steps != a.n_steps ||
-      g->adj_exec_interval != a.interval) {
+  // A first pass of a schedule is enqueued launch by launch; a second one is recorded as a graph,
+  // which later ones replay (recording costs more than the launches it saves once).
+  int lb = 0;
+  const bool same = g->adj_exec_steps == a.n_steps && g->adj_exec_interval == a.interval;
+  if (!same) {
     if (g->adj_exec) cudaGraphExecDestroy(g->adj_exec);
     g->adj_exec = nullptr;
-    if (g->capture == nullptr)
-      PF_CUDA_TRY(cudaStreamCreateWithFlags(&g->capture, cudaStreamNonBlocking));
-    if (g->capture2 == nullptr)
-      PF_CUDA_TRY(cudaStreamCreateWithFlags(&g->capture2, cudaStreamNonBlocking));
-    PF_CUDA_TRY(cudaStreamBeginCapture(g->capture, cudaStreamCaptureModeRelaxed));
-    int lb = 0;
-    cudaError_t e = enqueue_reverse(g, m, g->capture, g->capture2, &lb);
-    cudaGraph_t graph = nullptr;
-    cudaError_t e2 = cudaStreamEndCapture(g->capture, &graph);
-    if (e != cudaSuccess || e2 != cudaSuccess) {
-      if (graph) cudaGraphDestroy(graph);
-      return cuda_fail(e != cudaSuccess ? e : e2, "pf_adj_backward graph capture");
-    }
-    e = cudaGraphInstantiate(&g->adj_exec, graph, 0);
-    cudaGraphDestroy(graph);
-    if (e != cudaSuccess) {
-      g->adj_exec = nullptr;
-      return cuda_fail(e, "pf_adj_backward cudaGraphInstantiate");
-    }
+    PF_CUDA_TRY(enqueue_reverse(g, m, g->stream, &lb));
     g->adj_exec_steps = a.n_steps;
     g->adj_exec_interval = a.interval;
-    g->adj_exec_lb = lb;
+  } else {
+    if (g->adj_exec == nullptr) {
+      if (g->capture == nullptr)
+        PF_CUDA_TRY(cudaStreamCreateWithFlags(&g->capture, cudaStreamNonBlocking));
+      PF_CUDA_TRY(cudaStreamBeginCapture(g->capture, cudaStreamCaptureModeRelaxed));
+      cudaError_t e = enqueue_reverse(g, m, g->capture, &g->adj_exec_lb);
+      cudaGraph_t graph = nullptr;
+      cudaError_t e2 = cudaStreamEndCapture(g->capture, &graph);
+      if (e != cudaSuccess || e2 != cudaSuccess) {
+        if (graph) cudaGraphDestroy(graph);
+        return cuda_fail(e != cudaSuccess ? e : e2, "pf_adj_backward graph capture");
+      }
+      e = cudaGraphInstantiate(&g->adj_exec, graph, 0);
+      cudaGraphDestroy(graph);
+      if (e != cudaSuccess) {
+        g->adj_exec = nullptr;
+        return cuda_fail(e, "pf_adj_backward cudaGraphInstantiate");
+      }
+    }
+    PF_CUDA_TRY(cudaGraphLaunch(g->adj_exec, g->stream));
+    lb = g->adj_exec_lb;
   }
-  PF_CUDA_TRY(cudaGraphLaunch(g->adj_exec, g->stream));
-  const int lb = g->adj_exec_lb;
-  PF_CUDA_TRY(cudaMemcpyAsync(a.ghost, a.gout, sizeof(double) * 4, cudaMemcpyDeviceToHost,
+  PF_CUDA_TRY(cudaMemcpyAsync(g->sums_host(), a.gout, sizeof(double) * 4, cudaMemcpyDeviceToHost,
                               g->stream));
   float* dst[2] = {dLdu0, dLdv0};
   for (int f = 0; f < g->nf; ++f)
@@ -568,7 +816,7 @@ int pf_adj_backward(pf_grid_t g, const float* dLdu_N, const float* dLdv_N, int o
                                     (size_t)g->ny, kout, g->stream));
   PF_CUDA_TRY(cudaStreamSynchronize(g->stream));
   if (dtheta != nullptr) {
-    const double* S = a.ghost;
+    const double* S = g->sums_host();
     if (g->model == PF_MODEL_GS) {
       // the kernel's Laplacians of u and v are unscaled (the parameters carry 1/h^2 in
       // D_u and D_v), so the sums for D_u and D_v take the factor here

@@ -289,6 +289,15 @@ int sync_device_error(pf_grid_s* g) {
 
 int k1_tile(pf_grid_s* g, int tile);
 
+cudaError_t launch_2d(const pf_grid_s* g, int tile, int k, const FieldPtrs& in,
+                      const FieldOut& out, const ModelParams& m, cudaStream_t st) {
+  const Geom q = grid_geom(g);
+  if (tile >= kTileStrips2D && tile < kTileStrips2D + kNumStrips2D)
+    return launch_fe2d_strips(g->model, g->stencil, tile == kTileStrips2D ? 128 : 64, k, q, in,
+                              out, m, st);
+  return launch_fe2d_stencil(g->stencil, g->model, tile, k, q, in, out, m, st);
+}
+
 // One launch advancing `k` steps from buffer `src` into buffer `dst`.
 cudaError_t launch_step(pf_grid_s* g, int tile, int k, int src, int dst, cudaStream_t st) {
   FieldPtrs in{};
@@ -303,10 +312,7 @@ cudaError_t launch_step(pf_grid_s* g, int tile, int k, int src, int dst, cudaStr
   if (g->dim == 2 && tile == kTileCluster2D)
     return launch_fe2d_cluster(g->model, k, q, in, out, g->params, k, st);
   if (g->dim == 2 && tile == kTileBands2D) return launch_fe2d_bands(g, src, dst, k, st);
-  if (g->dim == 2 && tile >= kTileStrips2D && tile < kTileStrips2D + kNumStrips2D)
-    return launch_fe2d_strips(g->model, g->stencil, tile == kTileStrips2D ? 128 : 64, k, q, in,
-                              out, g->params, st);
-  if (g->dim == 2) return launch_fe2d_stencil(g->stencil, g->model, tile, k, q, in, out, g->params, st);
+  if (g->dim == 2) return launch_2d(g, tile, k, in, out, g->params, st);
   const bool r2 = g->model == PF_MODEL_CH || g->model == PF_MODEL_C;
   if (g->stencil != PF_ST_STD)
     return r2 ? launch_fe3d(g->model, tile, q, in, out, g->params, st, g->stencil)
@@ -430,12 +436,16 @@ int pf_create_grid(int dim, const int64_t* n, int n_fields, double h, void* stre
   g->plane = plane;
   g->field_elems = elems;
   cudaError_t e = cudaGetDevice(&g->device);
-  if (e == cudaSuccess) e = cudaMalloc(&g->base, sizeof(float) * elems * 2 * n_fields);
-  if (e == cudaSuccess) e = cudaMemsetAsync(g->base, 0, sizeof(float) * elems * 2 * n_fields, g->stream);
-  if (e == cudaSuccess) e = cudaMalloc(&g->red_partials, sizeof(double) * kReduceBlocks);
-  if (e == cudaSuccess) e = cudaMallocHost(&g->red_host, 2 * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&g->d_err, sizeof(int));
-  if (e == cudaSuccess) e = cudaMemsetAsync(g->d_err, 0, sizeof(int), g->stream);
+  // one allocation: the fields twice, a reduction's partials, the error word
+  const size_t fields = (sizeof(float) * elems * 2 * n_fields + 255) / 256 * 256;
+  const size_t bytes = fields + sizeof(double) * (kReduceBlocks + 1);
+  if (e == cudaSuccess) e = cudaMalloc(&g->base, bytes);
+  if (e == cudaSuccess) e = cudaMemsetAsync(g->base, 0, bytes, g->stream);
+  if (e == cudaSuccess) {
+    g->red_partials = reinterpret_cast<double*>(reinterpret_cast<char*>(g->base) + fields);
+    g->d_err = reinterpret_cast<int*>(g->red_partials + kReduceBlocks);
+    e = cudaMallocHost(&g->red_host, 6 * sizeof(double));
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
   if (e != cudaSuccess) {
     int rc = cuda_fail(e, "pf_create_grid allocation");
@@ -459,11 +469,8 @@ void pf_destroy(pf_grid_t g) {
   pf::fe2d_bands_release(g);
   drop_graphs(g);
   if (g->capture) cudaStreamDestroy(g->capture);
-  if (g->capture2) cudaStreamDestroy(g->capture2);
   if (g->base) cudaFree(g->base);
-  if (g->red_partials) cudaFree(g->red_partials);
   if (g->red_host) cudaFreeHost(g->red_host);
-  if (g->d_err) cudaFree(g->d_err);
   g->magic = 0;
   delete g;
 }

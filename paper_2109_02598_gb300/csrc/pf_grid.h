@@ -92,15 +92,11 @@ struct AdjointState {
   int64_t interval = 0;      // checkpoint interval C
   int64_t n_ckpt = 0;        // checkpoints stored (states 0, C, 2C, ...)
   float* ckpt = nullptr;     // n_ckpt * nf * field_elems floats
-  float* seg = nullptr;      // seg_bufs * (C - 1) * nf * field_elems floats: recomputed
-                             // segments (two buffers: one is recomputed while the reverse
-                             // steps read the other)
-  int seg_bufs = 0;          // 2, or 1 where the second buffer could not be allocated
-  float* lam = nullptr;      // 2 * nf * field_elems floats: adjoint ping-pong
-  double* gpart = nullptr;   // per-CTA parameter-gradient partials (4 per CTA)
-  double* gout = nullptr;    // 4 final sums (device)
-  double* ghost = nullptr;   // 4 final sums (pinned host)
-  int64_t gpart_cap = 0;     // CTAs the partial buffer holds
+  float* seg = nullptr;      // a segment's recomputed states: the first of each block of
+                             // reverse steps but the segment's own first
+  float* lam = nullptr;      // 2 * nf * field_elems floats: adjoint ping-pong; and behind them
+  double* gpart = nullptr;   //   per-CTA parameter-gradient partials (4 per CTA)
+  double* gout = nullptr;    //   and the 4 final sums
   double coeffs[4] = {0, 0, 0, 0};
   double dt = 0;
   int ready = 0;             // a forward pass is recorded
@@ -135,11 +131,12 @@ struct pf_grid_s {
   int k = 0;          // temporal-blocking depth in effect
   int req_tile = -1;  // tile asked for by pf_set_tuning (-1 = library default)
   int req_k = 0;      // depth asked for (0 = library default)
-  double* red_partials = nullptr;  // kReduceBlocks partials
-  // pinned host words that kernels and copies write: a reduction's result and, behind it, the
-  // device error word
+  double* red_partials = nullptr;  // kReduceBlocks partials (behind the fields, as d_err)
+  // pinned host words that kernels and copies write: a reduction's result, behind it the device
+  // error word, then the adjoint's four parameter sums
   double* red_host = nullptr;
   int* err_host() const { return reinterpret_cast<int*>(red_host + 1); }
+  double* sums_host() const { return red_host + 2; }
   pf::AdjointState adj;
   pf::TmaCache tma;
   pf::Tma2Cache tma2;
@@ -156,7 +153,6 @@ struct pf_grid_s {
   // CUDA-graph cache of pf_step: a few recorded launch sequences, keyed by
   // (steps, tile, k, starting buffer), least recently used replaced first
   cudaStream_t capture = nullptr;  // private stream used only to record graphs
-  cudaStream_t capture2 = nullptr;  // second branch of the adjoint's reverse-pass graph
   struct StepGraph {
     cudaGraphExec_t exec = nullptr;
     int64_t steps = -1;
@@ -178,6 +174,12 @@ int check_grid(pf_grid_s* g);
 Geom grid_geom(const pf_grid_s* g);
 ModelParams make_params(int model, const double* c, double dt, double h, int stencil = 0);
 cudaError_t launch_step(pf_grid_s* g, int tile, int k, int src, int dst, cudaStream_t st);
+// A 2D launch on any buffers of the grid's layout (the tiled and strip kernels)
+cudaError_t launch_2d(const pf_grid_s* g, int tile, int k, const FieldPtrs& in,
+                      const FieldOut& out, const ModelParams& m, cudaStream_t st);
+// The tile and depth of an untuned 2D grid with the standard stencil, and those pf_step runs
+void plan2d(const pf_grid_s* g, int* tile, int* depth);
+void run_plan(const pf_grid_s* g, int* tile, int* depth);
 
 // ---- 3D TMA kernels (AC, GS; Models B and C in pf_fe3d_tma2.cu): TMA tile ids 0 = 64x16,
 // 1 = 128x8, 2 = 128x16

@@ -298,6 +298,14 @@ __device__ __forceinline__ void mc_update4(const float4& psi, const float4& m4,
   m_n = fma4(p.dt, lap_mu, m4);
 }
 
+// In a kernel launched by launch_chained: wait until the preceding kernel of the stream has
+// finished and its writes are visible, then let the following one begin to launch. Without a
+// programmatic predecessor or successor both are no-ops.
+__device__ __forceinline__ void chain_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Checked builds (PF_CHECK): fill n floats of shared memory with NaN before they are staged,
 // so a read of a slot that staging or an earlier sub-step did not write turns results into
 // NaN, which the parity tests see. Every thread of the CTA calls it; it ends with a CTA
