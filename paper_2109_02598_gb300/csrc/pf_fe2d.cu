@@ -24,6 +24,7 @@ __global__ void __launch_bounds__(kNT2) fe2d_kernel(FieldPtrs in, FieldOut out, 
   extern __shared__ __align__(16) float sm[];
   const int x0 = blockIdx.x * TX;
   const int y0 = blockIdx.y * TY;
+  chain_wait();
   fe2d_tile<MODEL, K, TX, TY>(in, out, g.nx, g.ny, g.pitch, x0, y0, m, sm);
 }
 
@@ -78,8 +79,7 @@ cudaError_t launch_one(const Geom& g, FieldPtrs in, FieldOut out, const ModelPar
   cudaError_t e = ensure_smem_attr(fe2d_kernel<MODEL, K, TX, TY>, smem, &attr_mask);
   if (e != cudaSuccess) return e;
   dim3 grid((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, 1);
-  fe2d_kernel<MODEL, K, TX, TY><<<grid, kNT2, smem, s>>>(in, out, g, m);
-  return cudaGetLastError();
+  return launch_chained(fe2d_kernel<MODEL, K, TX, TY>, grid, kNT2, smem, s, in, out, g, m);
 }
 
 template <int MODEL, int K>

@@ -13,6 +13,7 @@ template <int MODEL, int K, int TX, int TY, int ST>
 __global__ void __launch_bounds__(kNT2) fe2d_st_kernel(FieldPtrs in, FieldOut out, Geom g,
                                                        ModelParams m) {
   extern __shared__ __align__(16) float sm[];
+  chain_wait();
   fe2d_tile<MODEL, K, TX, TY, ST>(in, out, g.nx, g.ny, g.pitch, blockIdx.x * TX, blockIdx.y * TY,
                                   m, sm);
 }
@@ -26,8 +27,7 @@ cudaError_t launch_st(const Geom& g, FieldPtrs in, FieldOut out, const ModelPara
   cudaError_t e = ensure_smem_attr(fe2d_st_kernel<MODEL, K, TX, TY, ST>, smem, &attr_mask);
   if (e != cudaSuccess) return e;
   dim3 grid((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, 1);
-  fe2d_st_kernel<MODEL, K, TX, TY, ST><<<grid, kNT2, smem, s>>>(in, out, g, m);
-  return cudaGetLastError();
+  return launch_chained(fe2d_st_kernel<MODEL, K, TX, TY, ST>, grid, kNT2, smem, s, in, out, g, m);
 }
 
 template <int MODEL, int ST>

@@ -125,6 +125,7 @@ __global__ void __launch_bounds__(kNT3) fe3d_r2_kernel(FieldPtrs in, FieldOut ou
   auto plane = [&](int p) { return ph + pslot(p) * NF * PL; };
   // prologue: mu(z0-1) from phi(z0-2..z0), then mu(z0) from phi(z0-1..z0+1)
   canary_fill(sm, C::SMEM_FLOATS);
+  chain_wait();
   load_plane3d<C>(in, g, x0, y0, z0 - 2, pslot(z0 - 2), ph);
   load_plane3d<C>(in, g, x0, y0, z0 - 1, pslot(z0 - 1), ph);
   load_plane3d<C>(in, g, x0, y0, z0, pslot(z0), ph);
@@ -191,8 +192,7 @@ cudaError_t launch3(const Geom& g, FieldPtrs in, FieldOut out, const ModelParams
   dim3 grid(bx, by, (g.nz + tz - 1) / tz);
   cudaError_t e = ensure_smem_attr(fe3d_r2_kernel<MODEL, TX, TY, ST>, smem, &attr_mask);
   if (e != cudaSuccess) return e;
-  fe3d_r2_kernel<MODEL, TX, TY, ST><<<grid, kNT3, smem, s>>>(in, out, g, m, tz);
-  return cudaGetLastError();
+  return launch_chained(fe3d_r2_kernel<MODEL, TX, TY, ST>, grid, kNT3, smem, s, in, out, g, m, tz);
 }
 
 template <int MODEL>

@@ -110,6 +110,7 @@ __global__ void __launch_bounds__(BoxCfg<MODEL, K>::THREADS)
   float* s1 = mu + M0::SIZE;       // K = 2: state after one step, field f at f * S1::SIZE
   const int x0 = blockIdx.x * kBX, y0 = blockIdx.y * kBY, z0 = blockIdx.z * kBZ;
   canary_fill(sm, B::SMEM_FLOATS);
+  chain_wait();
 
   // stage: (field, plane, row, 16-byte group)
   constexpr int G = S0::X / 4;
@@ -167,8 +168,7 @@ cudaError_t launch_box(const Geom& g, FieldPtrs in, FieldOut out, const ModelPar
   cudaError_t e = ensure_smem_attr(fe3d_box_kernel<MODEL, K>, smem, &attr_mask);
   if (e != cudaSuccess) return e;
   dim3 grid((g.nx + kBX - 1) / kBX, (g.ny + kBY - 1) / kBY, (g.nz + kBZ - 1) / kBZ);
-  fe3d_box_kernel<MODEL, K><<<grid, B::THREADS, smem, s>>>(in, out, g, m);
-  return cudaGetLastError();
+  return launch_chained(fe3d_box_kernel<MODEL, K>, grid, B::THREADS, smem, s, in, out, g, m);
 }
 
 }  // namespace

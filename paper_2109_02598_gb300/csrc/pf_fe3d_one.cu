@@ -192,6 +192,7 @@ __global__ void __launch_bounds__(U::NT, U::CTAS)
   const int ncols = pl.S * ((g.ny + TY - 1) / TY);
   SegmentWalk seg(sc_, ncols, g.nz);
   U u;
+  chain_wait();
   while (seg.next(sc_, ncols, g.nz)) {
     const int n = seg.zhi - seg.zlo, dir = seg.dir;  // output planes
     const int zfirst = dir > 0 ? seg.zlo : seg.zhi - 1;
@@ -268,8 +269,8 @@ cudaError_t launch_one_(pf_grid_s* gr, FieldPtrs in, FieldOut out, const typenam
   if (e != cudaSuccess) return e;
   const StreamTiles& p = gr->one.tiles;
   const int nt = (std::max(p.TY, 2) * p.G + 31) / 32 * 32;
-  kern<<<gr->one.grid, nt, smem, st>>>(in, out, grid_geom(gr), arg, p, gr->one.sched);
-  return cudaGetLastError();
+  return launch_chained(kern, gr->one.grid, nt, smem, st, in, out, grid_geom(gr), arg, p,
+                        gr->one.sched);
 }
 
 template <class U>

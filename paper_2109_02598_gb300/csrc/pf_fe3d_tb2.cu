@@ -196,6 +196,7 @@ __global__ void __launch_bounds__(CfgB<MODEL, W, TY, NS, V_>::NT, 1)
   }
   __syncthreads();
 
+  chain_wait();
   uint32_t q_base = 0, q_issued = 0;
   bool err = false;
   auto stage_ptr = [&](uint32_t q) { return ring + (q % NS) * C::IN_STAGE; };
@@ -370,8 +371,8 @@ cudaError_t launch_tb2(pf_grid_s* gr, const Tb2Maps& maps, FieldOut out, cudaStr
   const Geom g = grid_geom(gr);
   long long grid = 0;
   const Tb2Sched sc = tb2_schedule(g.ny / TY, g.nz, (long long)sms * occ, &grid);
-  kern<<<(unsigned)grid, C::NT, C::SMEM, st>>>(maps, out, g, gr->params, sc, gr->d_err);
-  return cudaGetLastError();
+  return launch_chained(kern, (unsigned)grid, C::NT, C::SMEM, st, maps, out, g, gr->params, sc,
+                        gr->d_err);
 }
 
 }  // namespace

@@ -161,6 +161,7 @@ __global__ void __launch_bounds__(kTwoThreads, 1)
   const int ncols = pl.S * ((g.ny + TY - 1) / TY);
   SegmentWalk seg(sc_, ncols, g.nz);
   TwoStream<MODEL> zs;
+  chain_wait();
   while (seg.next(sc_, ncols, g.nz)) {
     const int col = seg.col, zlo = seg.zlo, zhi = seg.zhi, dir = seg.dir;
     const int n = zhi - zlo;  // output planes
@@ -256,8 +257,8 @@ cudaError_t launch_two_(pf_grid_s* gr, FieldPtrs in, FieldOut out, cudaStream_t 
   if (e != cudaSuccess) return e;
   const StreamTiles& p = gr->two.tiles;
   const int nt = ((p.TY + 2) * p.G + 31) / 32 * 32;
-  kern<<<gr->two.grid, nt, C::SMEM, st>>>(in, out, grid_geom(gr), gr->params, p, gr->two.sched);
-  return cudaGetLastError();
+  return launch_chained(kern, gr->two.grid, nt, C::SMEM, st, in, out, grid_geom(gr), gr->params, p,
+                        gr->two.sched);
 }
 
 template <int MODEL>

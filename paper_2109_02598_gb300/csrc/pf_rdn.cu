@@ -49,6 +49,7 @@ __global__ void __launch_bounds__(kRd2Threads) rd2d_kernel(FieldPtrs in, FieldOu
   extern __shared__ __align__(16) float sm[];
   const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
   canary_fill(sm, (size_t)NF * C::PL);
+  chain_wait();
   stage_rows4<NF>(in, g, x0, y0, 0, C::WS, C::HT, C::PL, sm, kRd2Threads);
   cp_async_wait_all();
   __syncthreads();
@@ -82,8 +83,7 @@ cudaError_t launch_rd2d_nf(const Geom& g, FieldPtrs in, FieldOut out, const RdPa
   cudaError_t e = ensure_smem_attr(rd2d_kernel<NF, TX, TY>, smem, &attr_mask);
   if (e != cudaSuccess) return e;
   const dim3 grid((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY);
-  rd2d_kernel<NF, TX, TY><<<grid, kRd2Threads, smem, s>>>(in, out, g, p);
-  return cudaGetLastError();
+  return launch_chained(rd2d_kernel<NF, TX, TY>, grid, kRd2Threads, smem, s, in, out, g, p);
 }
 
 }  // namespace
