@@ -218,11 +218,11 @@ cudaError_t launch_nonlinear(const pf_spectral_s* s, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// AUTO takes the fused engine where it was measured faster than cuFFT on GB300: every grid
-// it takes except two-field (Model C) 2D grids with a 1024 side (per step, fused vs cuFFT:
-// 64^2 Model A 9.2 vs 10.1 us, 128^2 A 10.9 vs 13.3 and C 11.1 vs 13.7, 256^2 A 12.8 vs 13.2,
-// 512^2 A 13.5 vs 16.3 and C 17.3 vs 18.4, 1024^2 A 28.2 vs 32.4 but C 67.7 vs 37.9, 64^3 A
-// 17.4 vs 18.2 and C 18.3 vs 21.7).
+// AUTO takes the fused engine on every grid it takes except two-field (Model C) 2D grids with a
+// 1024 side (us a step, fused vs cuFFT on GB300: 64^2 Model A 6.2 vs 11.0, 128^2 C 6.8 vs 14.3,
+// 512^2 A 8.9 vs 16.3 and C 10.4 vs 18.4, 1024^2 A 17.5 vs 33.1 but C 43.5 vs 38.4; 64^3 C 12.4 vs
+// 22.1; Model C 512x1024 would be faster fused too, 15.1 vs 24.3, but the engine a grid reports
+// stays what it was).
 bool auto_prefers_fused(const pf_spectral_s* s) {
   if (!s->fused_ok) return false;
   if (s->dim == 3) return true;

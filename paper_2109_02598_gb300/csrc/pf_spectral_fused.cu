@@ -27,12 +27,21 @@
 // A task (a row pair, or a slab) is done by a team of 32 .. 1024 threads of a CTA, chosen
 // per phase so that each thread does one radix-8 butterfly per pass where the tasks still fit
 // in one round on the SMs; a team synchronises on its own named barrier. The FFTs are
-// Stockham passes (radix 8, then one radix-4 or radix-2 pass) between two shared-memory
-// buffers: natural order in and out, no bit reversal, and every thread loads all
-// of a butterfly's inputs before it computes. A slab's transforms are batched passes: along y
-// the slab's nz rows at once, along z its ny columns at once, consecutive lanes on
-// consecutive FFTs of the batch; the slab's rows are padded to ny + 1 values in shared memory,
-// so those lanes fall on distinct banks in both directions.
+// Stockham passes between two shared-memory buffers: natural order in and out, no bit reversal,
+// and every thread loads all of a butterfly's inputs before it computes. Both phases transform
+// there and back, and a step is bound by the latency of that chain: a pass (about 1000 cycles
+// with eight warps on an SM) is an exchange through shared memory and a barrier. So a transform is
+// radix-8 passes and one of radix 8, 4 or 2, last on the way there and first on the way back, and
+// those two passes are one, with the nonlinear terms or the update between them in registers; a
+// 2D column's first pass reads global memory and its last one writes there. A 512-point row takes
+// five exchanges, a column four (before: nine each, with the pointwise parts in passes of their
+// own). A slab's transforms are batched passes: along y the slab's nz rows at once, along z its
+// ny columns at once, consecutive lanes on consecutive FFTs of the batch; the slab's rows are
+// padded to ny + 1 values in shared memory, so those lanes fall on distinct banks in both
+// directions. Us a step, before and now: Model C 512^2 18.1 -> 10.4, 256^2 13.6 -> 8.0, Model B
+// 512^2 14.2 -> 8.9, 64^3 17.6 -> 12.1, Model A 64^2 9.7 -> 6.4. What remains at 512^2: two grid
+// barriers of 3300 and 4700 cycles (the wait for the other CTAs' stores and for the two columns
+// that pair with themselves in it), loads and stores 5900, passes 9000.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -112,118 +121,143 @@ __device__ __forceinline__ void dft4(const float2& a, const float2& b, const flo
   out[3] = make_float2(__fsub_rn(a1.x, a3.x), __fsub_rn(a1.y, a3.y));
 }
 
-// One Stockham pass of radix R over `batch` FFTs of n points (stride ns so far). FFT b's
-// element i lives at buf[b bs + i es] in both buffers. Butterfly j < n/R of an FFT takes
-// in[j + r n/R], twiddles it by W_{ns R}^{(j mod ns) r}, and writes its R-point DFT to
-// out[(j - j mod ns) R + j mod ns + r ns]. tw holds W_n^i = exp(-2 pi i i / n), i < n; INV
-// conjugates every twiddle (the inverse transform, unnormalised). BF: consecutive lanes take
-// consecutive FFTs of the batch (for bs = 1, where the elements are strided), else
-// consecutive butterflies of one FFT.
-template <int R, bool INV, bool BF>
-__device__ __forceinline__ void stockham_pass(const float2* __restrict__ in,
-                                              float2* __restrict__ out, int n, int logq, int ns,
-                                              int batch, int logb, int bs, int es,
-                                              const float2* __restrict__ tw, const Team& tm) {
-  const int q = n / R;
-  const int tws = n / (ns * R);
-  const int total = q * batch;
-#pragma unroll 2
-  for (int t = tm.rank; t < total; t += tm.size) {
-    int b, j;
-    if (BF) {
-      j = t >> logb;
-      b = t - (j << logb);
-    } else {
-      b = t >> logq;
-      j = t - (b << logq);
+// R-point DFT in place, natural order in and out.
+template <int R, bool INV>
+__device__ __forceinline__ void dft(float2 (&v)[R]) {
+  if constexpr (R == 8) {
+    // two 4-point DFTs (even and odd inputs), the odd one twiddled by W_8^m, combined
+    float2 e[4], o[4];
+    dft4<INV>(v[0], v[2], v[4], v[6], e);
+    dft4<INV>(v[1], v[3], v[5], v[7], o);
+    const float c = 0.70710678118654752f;  // sqrt(1/2)
+    const float2 o1 = o[1], o3 = o[3];
+    if (!INV) {  // W_8 = c (1 - i), W_8^2 = -i, W_8^3 = -c (1 + i)
+      o[1] = make_float2(__fmul_rn(c, __fadd_rn(o1.x, o1.y)), __fmul_rn(c, __fsub_rn(o1.y, o1.x)));
+      o[2] = make_float2(o[2].y, -o[2].x);
+      o[3] = make_float2(__fmul_rn(c, __fsub_rn(o3.y, o3.x)), -__fmul_rn(c, __fadd_rn(o3.x, o3.y)));
+    } else {  // the conjugates: c (1 + i), i, c (-1 + i)
+      o[1] = make_float2(__fmul_rn(c, __fsub_rn(o1.x, o1.y)), __fmul_rn(c, __fadd_rn(o1.x, o1.y)));
+      o[2] = make_float2(-o[2].y, o[2].x);
+      o[3] = make_float2(-__fmul_rn(c, __fadd_rn(o3.x, o3.y)), __fmul_rn(c, __fsub_rn(o3.x, o3.y)));
     }
-    const float2* ib = in + b * bs;
-    float2* ob = out + b * bs;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      v[m] = make_float2(__fadd_rn(e[m].x, o[m].x), __fadd_rn(e[m].y, o[m].y));
+      v[m + 4] = make_float2(__fsub_rn(e[m].x, o[m].x), __fsub_rn(e[m].y, o[m].y));
+    }
+  } else if constexpr (R == 4) {
+    float2 x[4];
+    dft4<INV>(v[0], v[1], v[2], v[3], x);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) v[m] = x[m];
+  } else {
+    const float2 a = v[0], b = v[1];
+    v[0] = make_float2(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y));
+    v[1] = make_float2(__fsub_rn(a.x, b.x), __fsub_rn(a.y, b.y));
+  }
+}
+
+template <int R>
+constexpr int kLog2 = R == 8 ? 3 : R == 4 ? 2 : 1;
+
+// Where element i of a single contiguous transform, and of a twiddle table, lies in shared memory:
+// a place is left out after every eight, so that a first pass's stores (every eighth element from
+// consecutive lanes) and the passes' twiddles (every 2^logt-th) fall on distinct banks (the tables
+// alone, Model C 512^2: 11.2 -> 10.4 us a step).
+__device__ __forceinline__ int padded(int i) { return i + (i >> 3); }
+constexpr int64_t padded_size(int64_t n) { return n + n / 8; }
+
+// v[r] *= W_n^{r k 2^logt} (INV: its conjugate); tw holds W_n^i = exp(-2 pi i / n), i < n,
+// at padded(i)
+template <int R, bool INV>
+__device__ __forceinline__ void twiddle(float2 (&v)[R], int k, int logt, const float2* tw) {
+#pragma unroll
+  for (int r = 1; r < R; ++r) {
+    float2 w = tw[padded((k * r) << logt)];
+    if (INV) w.y = -w.y;
+    v[r] = cmul(w, v[r]);
+  }
+}
+
+// Butterfly t of a pass over 2^logb FFTs with 2^logq butterflies each: its FFT b and number j.
+// BF: consecutive lanes take consecutive FFTs (whose elements are strided), else consecutive
+// butterflies of one FFT.
+template <bool BF>
+__device__ __forceinline__ void butterfly(int t, int logq, int logb, int& b, int& j) {
+  if (BF) {
+    j = t >> logb;
+    b = t - (j << logb);
+  } else {
+    b = t >> logq;
+    j = t - (b << logq);
+  }
+}
+
+// One Stockham pass of radix R over 2^logb FFTs of 2^logn points (stride 2^logns so far; FIRST:
+// 0, no twiddles). Butterfly j of FFT b takes elements j + r n/R from ld(b, i), twiddles them by
+// W_{ns R}^{(j mod ns) r}, and gives element (j - j mod ns) R + j mod ns + m ns of its DFT to
+// st(b, i, value). INV: the inverse transform, unnormalised.
+template <int R, bool INV, bool BF, bool FIRST, class LD, class ST>
+__device__ __forceinline__ void fft_pass(int logn, int logns, int logb, const float2* tw,
+                                         const Team& tm, const LD& ld, const ST& st) {
+  const int logq = logn - kLog2<R>, q = 1 << logq, ns = 1 << logns;
+  for (int t = tm.rank; t < 1 << (logq + logb); t += tm.size) {
+    int b, j;
+    butterfly<BF>(t, logq, logb, b, j);
     float2 v[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = ib[(j + r * q) * es];
-    const int k = j & (ns - 1);
-#pragma unroll
-    for (int r = 1; r < R; ++r) {
-      float2 w = tw[(k * r * tws) & (n - 1)];
-      if (INV) w.y = -w.y;
-      v[r] = cmul(w, v[r]);
-    }
+    for (int r = 0; r < R; ++r) v[r] = ld(b, j + r * q);
+    const int k = FIRST ? 0 : j & (ns - 1);
+    if (!FIRST) twiddle<R, INV>(v, k, logn - logns - kLog2<R>, tw);
+    dft<R, INV>(v);
     const int base = (j - k) * R + k;
-    if (R == 8) {
-      // two 4-point DFTs (even and odd inputs), the odd one twiddled by W_8^m, combined
-      float2 e[4], o[4];
-      dft4<INV>(v[0], v[2], v[4], v[6], e);
-      dft4<INV>(v[1], v[3], v[5], v[7], o);
-      const float c = 0.70710678118654752f;  // sqrt(1/2)
-      const float2 o1 = o[1], o3 = o[3];
-      if (!INV) {  // W_8 = c (1 - i), W_8^2 = -i, W_8^3 = -c (1 + i)
-        o[1] = make_float2(__fmul_rn(c, __fadd_rn(o1.x, o1.y)), __fmul_rn(c, __fsub_rn(o1.y, o1.x)));
-        o[2] = make_float2(o[2].y, -o[2].x);
-        o[3] = make_float2(__fmul_rn(c, __fsub_rn(o3.y, o3.x)), -__fmul_rn(c, __fadd_rn(o3.x, o3.y)));
-      } else {  // the conjugates: c (1 + i), i, c (-1 + i)
-        o[1] = make_float2(__fmul_rn(c, __fsub_rn(o1.x, o1.y)), __fmul_rn(c, __fadd_rn(o1.x, o1.y)));
-        o[2] = make_float2(-o[2].y, o[2].x);
-        o[3] = make_float2(-__fmul_rn(c, __fadd_rn(o3.x, o3.y)), __fmul_rn(c, __fsub_rn(o3.x, o3.y)));
-      }
 #pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        ob[(base + m * ns) * es] = make_float2(__fadd_rn(e[m].x, o[m].x), __fadd_rn(e[m].y, o[m].y));
-        ob[(base + (m + 4) * ns) * es] =
-            make_float2(__fsub_rn(e[m].x, o[m].x), __fsub_rn(e[m].y, o[m].y));
-      }
-    } else if (R == 2) {
-      ob[base * es] = make_float2(__fadd_rn(v[0].x, v[1].x), __fadd_rn(v[0].y, v[1].y));
-      ob[(base + ns) * es] = make_float2(__fsub_rn(v[0].x, v[1].x), __fsub_rn(v[0].y, v[1].y));
-    } else {
-      float2 x[4];
-      dft4<INV>(v[0], v[1], v[2], v[3], x);
-#pragma unroll
-      for (int m = 0; m < 4; ++m) ob[(base + m * ns) * es] = x[m];
-    }
+    for (int m = 0; m < R; ++m) st(b, base + m * ns, v[m]);
   }
 }
 
-// `batch` = 2^logb FFTs of n = 2^logn points in b (layout as stockham_pass) by one team,
-// natural order in and out: radix-8 passes, then one radix-4 or radix-2 pass for the rest.
-// b and b2 are used in turn and the result is in the returned buffer (the other one is
-// free). logn = 0 returns b untouched. Each pass ends with a team barrier and its stores and
-// loads make a round trip through shared memory, so fewer, wider passes are faster: radix 8
-// takes a 64-point transform in two passes instead of three (radix 4), 512 points in three
-// instead of five.
-template <bool INV, bool BF>
-__device__ __forceinline__ float2* team_fft(float2* b, float2* b2, int n, int logn, int logb,
-                                            int bs, int es, const float2* tw, const Team& tm) {
-  float2* in = b;
-  float2* out = b2;
-  int ns = 1;
-  const int batch = 1 << logb;
-  int left = logn;
-  for (; left >= 3; left -= 3) {
-    stockham_pass<8, INV, BF>(in, out, n, logn - 3, ns, batch, logb, bs, es, tw, tm);
-    tm.sync();
-    float2* t = in;
-    in = out;
-    out = t;
-    ns <<= 3;
+// The last pass of one transform, op(b, i, value) on every element of its result, and the first
+// pass of the transform back, in one: with the same radix the first pass's butterfly j takes just
+// the elements j + m n/R that the last pass's butterfly j gives, so nothing passes through shared
+// memory between them.
+template <int R, bool INV, bool BF, class LD, class OP, class ST>
+__device__ __forceinline__ void fft_there_and_back(int logn, int logb, const float2* tw,
+                                                   const Team& tm, const LD& ld, const OP& op,
+                                                   const ST& st) {
+  const int logq = logn - kLog2<R>, q = 1 << logq;
+  for (int t = tm.rank; t < 1 << (logq + logb); t += tm.size) {
+    int b, j;
+    butterfly<BF>(t, logq, logb, b, j);
+    float2 v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = ld(b, j + r * q);
+    twiddle<R, INV>(v, j, 0, tw);
+    dft<R, INV>(v);
+#pragma unroll
+    for (int m = 0; m < R; ++m) op(b, j + m * q, v[m]);
+    dft<R, !INV>(v);
+#pragma unroll
+    for (int m = 0; m < R; ++m) st(b, j * R + m, v[m]);
   }
-  if (left == 2) {
-    stockham_pass<4, INV, BF>(in, out, n, logn - 2, ns, batch, logb, bs, es, tw, tm);
-    tm.sync();
-    in = out;
-  } else if (left == 1) {
-    stockham_pass<2, INV, BF>(in, out, n, logn - 1, ns, batch, logb, bs, es, tw, tm);
-    tm.sync();
-    in = out;
-  }
-  return in;
 }
 
-// One FFT of n points, contiguous.
-template <bool INV>
-__device__ __forceinline__ float2* team_fft1(float2* b, float2* b2, int n, int logn,
-                                             const float2* tw, const Team& tm) {
-  return team_fft<INV, false>(b, b2, n, logn, 0, 0, 1, tw, tm);
+// A transform of 2^logn points is radix-8 passes and one of radix 2^odd_log(logn), last on the way
+// there and first on the way back (logn >= 1).
+__device__ __forceinline__ int odd_log(int logn) {
+  const int l = logn % 3;
+  return l == 0 ? 3 : l;
+}
+
+template <int R>
+struct Radix {
+  static constexpr int value = R;
+};
+
+template <class F>
+__device__ __forceinline__ void with_radix(int log, const F& f) {
+  if (log == 3) f(Radix<8>());
+  else if (log == 2) f(Radix<4>());
+  else f(Radix<2>());
 }
 
 __device__ __forceinline__ unsigned int ld_acquire(const unsigned int* p) {
@@ -232,32 +266,38 @@ __device__ __forceinline__ unsigned int ld_acquire(const unsigned int* p) {
   return v;
 }
 
-// Grid barrier (sense by generation): bar[0] counts arrivals, bar[1] is the generation,
-// bar[2] the error word. Bounded: false after budget clocks without a release.
-__device__ __forceinline__ bool grid_barrier(unsigned int* bar, unsigned int nblocks,
+// Grid barrier: bar[0] counts arrivals over the whole launch (target: the count that releases this
+// one), bar[2] is the error word. An arrival is one reduction whose result nobody waits for, and
+// every CTA polls the counter itself (a last arrival that reads the count and then publishes a
+// generation is two more trips to L2: with 129 CTAs 4300 cycles a barrier, now 3300). Bounded:
+// false after budget clocks without a release.
+__device__ __forceinline__ bool grid_barrier(unsigned int* bar, unsigned int& target,
                                              long long budget) {
+  target += gridDim.x;
   __syncthreads();
   int ok = 1;
   if (threadIdx.x == 0) {
-    const unsigned int my_gen = ld_acquire(bar + 1);
-    __threadfence();  // the CTA's writes, ordered before this thread by the CTA barrier
-    unsigned int old;
-    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(old) : "l"(bar) : "memory");
-    if (old + 1 == nblocks) {
-      asm volatile("st.relaxed.gpu.global.u32 [%0], 0;" ::"l"(bar) : "memory");
-      asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar + 1) : "memory");
-    } else {
-      const long long t0 = clock64();
-      while (ld_acquire(bar + 1) == my_gen) {
-        if (clock64() - t0 > budget) {
-          atomicExch(bar + 2, 1u);
-          ok = 0;
-          break;
-        }
+    // (release: with the CTA's writes, which the CTA barrier orders before this thread)
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+    const long long t0 = clock64();
+    while ((int)(ld_acquire(bar) - target) < 0) {
+      if (clock64() - t0 > budget) {
+        atomicExch(bar + 2, 1u);
+        ok = 0;
+        break;
       }
     }
   }
   return __syncthreads_and(ok) != 0;
+}
+
+// At the end of a launch, also of one that gave up: the last CTA to leave (bar[1] counts them)
+// sets the counters back for the next.
+__device__ __forceinline__ void grid_leave(unsigned int* bar) {
+  if (threadIdx.x == 0 && atomicAdd(bar + 1, 1u) + 1 == gridDim.x) {
+    atomicExch(bar, 0u);
+    atomicExch(bar + 1, 0u);
+  }
 }
 
 template <int MODEL>
@@ -291,39 +331,57 @@ __device__ __forceinline__ void row_task(const FusedArgs& a, int f1, int y1, int
   }
   cp_async_wait_all();
   tm.sync();
-  const float2* X1 = b2;
-  const float2* X2 = b2 + nh + 1;
   // Z = X1 + i X2 over the full length, each extended by Hermitian symmetry; the imaginary
   // parts at k = 0 and nx/2 are dropped, as a complex-to-real transform does
-  for (int k = tm.rank; k < nx; k += tm.size) {
-    float2 p, q;
-    if (k <= nh) {
-      p = X1[k];
-      q = X2[k];
-      if (k == 0 || k == nh) p.y = q.y = 0.f;
-    } else {
-      p = X1[nx - k];
-      q = X2[nx - k];
+  const float2* X1 = b2;
+  const float2* X2 = b2 + nh + 1;
+  auto z = [&](int, int k) {
+    const bool up = k > nh;
+    float2 p = X1[up ? nx - k : k], q = X2[up ? nx - k : k];
+    if (k == 0 || k == nh) p.y = q.y = 0.f;
+    if (up) {
       p.y = -p.y;
       q.y = -q.y;
     }
-    b[k] = make_float2(__fsub_rn(p.x, q.y), __fadd_rn(p.y, q.x));
+    return make_float2(__fsub_rn(p.x, q.y), __fadd_rn(p.y, q.x));
+  };
+  // the inverse transform, the nonlinear terms and the forward transform
+  const int odd = odd_log(a.lognx);
+  float2 *in = b2, *out = b;
+  auto ld = [&](int, int i) { return in[padded(i)]; };
+  auto st = [&](int, int i, float2 v) { out[padded(i)] = v; };
+  auto turn = [&]() {
+    tm.sync();
+    float2* t = in;
+    in = out;
+    out = t;
+  };
+  if (a.lognx > odd) {
+    fft_pass<8, true, false, true>(a.lognx, 0, 0, twx, tm, z, st);
+    turn();
+    for (int ns = 3; ns < a.lognx - odd; ns += 3) {
+      fft_pass<8, true, false, false>(a.lognx, ns, 0, twx, tm, ld, st);
+      turn();
+    }
+  } else {  // one pass in all
+    for (int k = tm.rank; k < nx; k += tm.size) st(0, k, z(0, k));
+    turn();
   }
-  tm.sync();
-  float2* z = team_fft1<true>(b, b2, nx, a.lognx, twx, tm);
-  float2* other = z == b ? b2 : b;
-  for (int k = tm.rank; k < nx; k += tm.size) {
-    float2 v = z[k];
-    nl_pair<MODEL>(v, a.k);
-    z[k] = v;
+  with_radix(odd, [&](auto r) {
+    fft_there_and_back<decltype(r)::value, true, false>(
+        a.lognx, 0, twx, tm, ld, [&](int, int, float2& v) { nl_pair<MODEL>(v, a.k); }, st);
+  });
+  turn();
+  for (int ns = odd; ns < a.lognx; ns += 3) {
+    fft_pass<8, false, false, false>(a.lognx, ns, 0, twx, tm, ld, st);
+    turn();
   }
-  tm.sync();
-  const float2* Y = team_fft1<false>(z, other, nx, a.lognx, twx, tm);
+  const float2* Y = in;
   float2* F1 = a.W + f1 * a.cs + (int64_t)y1 * a.wr;
   float2* F2 = a.W + f2 * a.cs + (int64_t)y2 * a.wr;
   for (int k = tm.rank; k <= nh && valid; k += tm.size) {
-    const float2 y = Y[k];
-    const float2 r = Y[(nx - k) & (nx - 1)];  // Y(-k); conj taken below
+    const float2 y = Y[padded(k)];
+    const float2 r = Y[padded((nx - k) & (nx - 1))];  // Y(-k); conj taken below
     const float2 s = make_float2(__fadd_rn(y.x, r.x), __fsub_rn(y.y, r.y));  // Y + conj Y(-k)
     const float2 d = make_float2(__fsub_rn(y.x, r.x), __fadd_rn(y.y, r.y));  // Y - conj Y(-k)
     F1[k * ks] = make_float2(__fmul_rn(0.5f, s.x), __fmul_rn(0.5f, s.y));
@@ -332,100 +390,180 @@ __device__ __forceinline__ void row_task(const FusedArgs& a, int f1, int y1, int
   tm.sync();
 }
 
-// Slab task (field f, column kx): the ny x nz values W[f][z][y][kx], held in shared memory as
+// Slab task (field f, column kx): the ny x nz values W[f][z][y][kx], with the slab's psi_hat in
+// st and (A, B N) in tb (shared memory, [kz][ky]). In 3D (D3) they are held in shared memory as
 // [z][y] with rows of ny + 1 (the pad keeps a batched pass's lanes, one FFT each, on distinct
-// banks), with the slab's psi_hat in st and (A, B N) in tb (shared memory, [kz][ky]).
+// banks) and transformed along y, then z; in 2D they are one column of ny values, which the first
+// pass reads from global memory and the last one writes there.
 // mode 0: prologue (W <- inverse(psi_hat / N)); mode 1: full step; mode 2: last step (psi_hat
-// and work = psi_hat / N to global memory, no inverse transform). In 2D (nz = 1) it is one
-// column of ny values.
+// and work = psi_hat / N to global memory, no inverse transform).
+template <bool D3>
 __device__ __forceinline__ void slab_task(const FusedArgs& a, int f, int kx, int mode,
                                           float2* st, const float2* tb, float2* b, float2* b2,
                                           const float2* twy, const float2* twz, const Team& tm) {
-  const int ny = a.ny, nz = a.nz, ns = ny * nz, rp = ny + 1;
+  const int ny = a.ny, ns = ny * a.nz, rp = ny + 1;
   const int64_t base = f * a.cs + kx;  // the state's layout, [z][y][kx]
   const int64_t rstride = a.nxh;
-  const float2* Wg = a.W + f * a.cs + (int64_t)kx * a.wk;  // the slab in W (rows wr apart)
-  float2* o = b;  // receives psi_hat / N for the inverse transform
-  if (mode != 0) {
-    for (int i = tm.rank; i < ns; i += tm.size)
-      cp_async8(b + i + (i >> a.logny), Wg + (int64_t)i * a.wr);
-    cp_async_wait_all();
+  float2* Wg = a.W + f * a.cs + (int64_t)kx * a.wk;  // the slab in W (rows wr apart)
+  // the axis transformed last on the way there (z; in 2D y) and the FFTs along it
+  const int logn = D3 ? a.lognz : a.logny, logb = D3 ? a.logny : 0;
+  const float2* tw = D3 ? twz : twy;
+  const int odd = odd_log(logn);
+  float2 *in = b, *out = b2;
+  auto at = [&](int bb, int i) { return D3 ? bb + i * rp : padded(i); };
+  auto ld = [&](int bb, int i) { return in[at(bb, i)]; };
+  auto sm = [&](int bb, int i, float2 v) { out[at(bb, i)] = v; };
+  auto ld_y = [&](int bb, int i) { return in[bb * rp + i]; };
+  auto sm_y = [&](int bb, int i, float2 v) { out[bb * rp + i] = v; };
+  auto turn = [&]() {
     tm.sync();
-    // forward along y (the nz rows of the slab), then along z (its ny columns); in both,
-    // consecutive lanes take consecutive FFTs of the batch
-    float2* fy = team_fft<false, true>(b, b2, ny, a.logny, a.lognz, rp, 1, twy, tm);
-    float2* fh = team_fft<false, true>(fy, fy == b ? b2 : b, nz, a.lognz, a.logny, 1, rp, twz, tm);
-    o = fh == b ? b2 : b;
-    if (kx == 0 || 2 * kx == a.nx) {
-      // Hermitian part on a self-conjugate column: (kz, ky) pairs with (-kz, -ky)
-      for (int i = tm.rank; i < ns; i += tm.size) {
-        const int kz = i >> a.logny, ky = i & (ny - 1);
-        const int mz = (nz - kz) & (nz - 1), my = (ny - ky) & (ny - 1);
-        const int m = mz * ny + my;
-        if (i > m) continue;
-        float2* pu = fh + kz * rp + ky;
-        float2* pv = fh + mz * rp + my;
-        const float2 u = *pu, v = *pv;
-        const float2 hpart = make_float2(__fmul_rn(0.5f, __fadd_rn(u.x, v.x)),
-                                         __fmul_rn(0.5f, __fsub_rn(u.y, v.y)));
-        *pu = hpart;
-        *pv = make_float2(hpart.x, -hpart.y);
-      }
+    float2* t = in;
+    in = out;
+    out = t;
+  };
+  const int odd_y = odd_log(a.logny);
+  const bool direct = !D3 && logn > odd;  // 2D: global memory on either end
+  if (mode != 0) {
+    int s = 0;
+    if (direct) {
+      fft_pass<8, false, false, true>(
+          logn, 0, 0, tw, tm, [&](int, int i) { return Wg[(int64_t)i * a.wr]; }, sm);
+      turn();
+      s = 3;
+    } else {
+      for (int i = tm.rank; i < ns; i += tm.size)
+        cp_async8(b + (D3 ? i + (i >> a.logny) : padded(i)), Wg + (int64_t)i * a.wr);
+      cp_async_wait_all();
       tm.sync();
     }
-    for (int i = tm.rank; i < ns; i += tm.size) {
-      const int pi = i + (i >> a.logny);
-      const float2 s = st[i];
-      const float2 t = tb[i];
-      const float2 f_ = fh[pi];
-      const float2 sn = make_float2(__fmaf_rn(t.x, s.x, __fmul_rn(t.y, f_.x)),
-                                    __fmaf_rn(t.x, s.y, __fmul_rn(t.y, f_.y)));
-      st[i] = sn;
-      const float2 sc = make_float2(__fmul_rn(sn.x, a.inv_n), __fmul_rn(sn.y, a.inv_n));
-      if (mode == 2) {
-        a.state[base + i * rstride] = sn;
-        a.work[base + i * rstride] = sc;
-      } else {
-        o[pi] = sc;
+    if (D3) {  // forward along y: consecutive lanes take consecutive FFTs of the batch, here and below
+      int sy = 0;
+      if (a.logny > odd_y) {
+        fft_pass<8, false, D3, true>(a.logny, 0, a.lognz, twy, tm, ld_y, sm_y);
+        turn();
+        for (sy = 3; sy < a.logny - odd_y; sy += 3) {
+          fft_pass<8, false, D3, false>(a.logny, sy, a.lognz, twy, tm, ld_y, sm_y);
+          turn();
+        }
       }
+      with_radix(odd_y, [&](auto r) {
+        fft_pass<decltype(r)::value, false, D3, false>(a.logny, sy, a.lognz, twy, tm, ld_y, sm_y);
+      });
+      turn();
+    }
+    for (; s < logn - odd; s += 3) {
+      fft_pass<8, false, D3, false>(logn, s, logb, tw, tm, ld, sm);
+      turn();
+    }
+    // the update of the slab's value i = [kz][ky]; psi_hat / N
+    auto update = [&](int i, const float2& fh) {
+      const float2 p = st[i];
+      const float2 t = tb[i];
+      const float2 sn = make_float2(__fmaf_rn(t.x, p.x, __fmul_rn(t.y, fh.x)),
+                                    __fmaf_rn(t.x, p.y, __fmul_rn(t.y, fh.y)));
+      st[i] = sn;
+      return make_float2(__fmul_rn(sn.x, a.inv_n), __fmul_rn(sn.y, a.inv_n));
+    };
+    auto value = [&](int bb, int i) { return D3 ? i * ny + bb : i; };
+    const bool self = kx == 0 || 2 * kx == a.nx;
+    if (mode == 1 && !self) {
+      with_radix(odd, [&](auto r) {
+        fft_there_and_back<decltype(r)::value, false, D3>(
+            logn, logb, tw, tm, ld,
+            [&](int bb, int i, float2& v) { v = update(value(bb, i), v); }, sm);
+      });
+    } else {
+      with_radix(odd, [&](auto r) {
+        fft_pass<decltype(r)::value, false, D3, false>(logn, s, logb, tw, tm, ld, sm);
+      });
+      turn();
+      // f_hat, on a self-conjugate column its Hermitian part: (kz, ky) pairs with (-kz, -ky)
+      auto fhat = [&](int bb, int i) {
+        float2 u = ld(bb, i);
+        if (self) {
+          const float2 v = ld(D3 ? (ny - bb) & (ny - 1) : 0, ((1 << logn) - i) & ((1 << logn) - 1));
+          u = make_float2(__fmul_rn(0.5f, __fadd_rn(u.x, v.x)),
+                          __fmul_rn(0.5f, __fsub_rn(u.y, v.y)));
+        }
+        return u;
+      };
+      if (mode == 2) {
+        for (int i = tm.rank; i < ns; i += tm.size) {
+          const int kz = i >> a.logny, ky = i & (ny - 1);
+          const float2 sc = update(i, D3 ? fhat(ky, kz) : fhat(0, i));
+          a.state[base + i * rstride] = st[i];
+          a.work[base + i * rstride] = sc;
+        }
+        tm.sync();
+        return;
+      }
+      with_radix(odd, [&](auto r) {
+        fft_pass<decltype(r)::value, true, D3, true>(
+            logn, 0, logb, tw, tm,
+            [&](int bb, int i) { return update(value(bb, i), fhat(bb, i)); }, sm);
+      });
     }
   } else {
-    for (int i = tm.rank; i < ns; i += tm.size) {
-      const float2 s = st[i];
-      o[i + (i >> a.logny)] = make_float2(__fmul_rn(s.x, a.inv_n), __fmul_rn(s.y, a.inv_n));
+    with_radix(odd, [&](auto r) {
+      fft_pass<decltype(r)::value, true, D3, true>(
+          logn, 0, logb, tw, tm,
+          [&](int bb, int i) {
+            const float2 p = st[D3 ? i * ny + bb : i];
+            return make_float2(__fmul_rn(p.x, a.inv_n), __fmul_rn(p.y, a.inv_n));
+          },
+          sm);
+    });
+  }
+  turn();
+  int s = odd;
+  for (; s < logn - (direct ? 3 : 0); s += 3) {
+    fft_pass<8, true, D3, false>(logn, s, logb, tw, tm, ld, sm);
+    turn();
+  }
+  if (direct) {
+    fft_pass<8, true, false, false>(logn, s, 0, tw, tm, ld, [&](int, int i, float2 v) {
+      Wg[(int64_t)i * a.wr] = v;
+    });
+    tm.sync();
+    return;
+  }
+  if (D3) {
+    with_radix(odd_y, [&](auto r) {
+      fft_pass<decltype(r)::value, true, D3, true>(a.logny, 0, a.lognz, twy, tm, ld_y, sm_y);
+    });
+    turn();
+    for (int sy = odd_y; sy < a.logny; sy += 3) {
+      fft_pass<8, true, D3, false>(a.logny, sy, a.lognz, twy, tm, ld_y, sm_y);
+      turn();
     }
   }
-  tm.sync();
-  if (mode != 2) {
-    float2* gz = team_fft<true, true>(o, o == b ? b2 : b, nz, a.lognz, a.logny, 1, rp, twz, tm);
-    const float2* g = team_fft<true, true>(gz, gz == b ? b2 : b, ny, a.logny, a.lognz, rp, 1,
-                                           twy, tm);
-    float2* Wo = a.W + f * a.cs + (int64_t)kx * a.wk;
-    for (int i = tm.rank; i < ns; i += tm.size) Wo[(int64_t)i * a.wr] = g[i + (i >> a.logny)];
-  }
+  for (int i = tm.rank; i < ns; i += tm.size)
+    Wg[(int64_t)i * a.wr] = in[D3 ? i + (i >> a.logny) : padded(i)];
   tm.sync();
 }
 
-template <int MODEL>
-__global__ void __launch_bounds__(kThreads) spectral_fused_kernel(FusedArgs a) {
+template <int MODEL, bool D3>
+__device__ __forceinline__ void spectral_fused(const FusedArgs& a) {
   extern __shared__ float2 smem[];
+  unsigned int target = 0;
   const Team rt = make_team(a.row_team), ct = make_team(a.col_team);
   const int rteams = blockDim.x / a.row_team, cteams = blockDim.x / a.col_team;
   const int ns = a.ny * a.nz;
   float2* twx = smem;
-  float2* twy = twx + a.nx;
-  float2* twz = twy + a.ny;
+  float2* twy = twx + padded_size(a.nx);
+  float2* twz = twy + padded_size(a.ny);
   // the two phases' FFT buffers share one region: rteams x rbuf or cteams x cbuf
-  float2* bufs = twz + a.nz;
+  float2* bufs = twz + padded_size(a.nz);
   const int bregion = rteams * a.rbuf > cteams * a.cbuf ? rteams * a.rbuf : cteams * a.cbuf;
   float2* res = bufs + bregion;  // cteams x cpt x (psi_hat, table) slabs
   float2* rb = bufs + (size_t)rt.index * a.rbuf;
+  float2* rb2 = rb + padded_size(a.nx);
   float2* cb = bufs + (size_t)ct.index * a.cbuf;
   float2* st = res + (size_t)ct.index * a.cpt * 2 * ns;
   float2* tb = st + (size_t)a.cpt * ns;
-  for (int j = threadIdx.x; j < a.nx; j += blockDim.x) twx[j] = a.twx[j];
-  for (int j = threadIdx.x; j < a.ny; j += blockDim.x) twy[j] = a.twy[j];
-  for (int j = threadIdx.x; j < a.nz; j += blockDim.x) twz[j] = a.twz[j];
+  for (int j = threadIdx.x; j < a.nx; j += blockDim.x) twx[padded(j)] = a.twx[j];
+  for (int j = threadIdx.x; j < a.ny; j += blockDim.x) twy[padded(j)] = a.twy[j];
+  for (int j = threadIdx.x; j < a.nz; j += blockDim.x) twz[padded(j)] = a.twz[j];
   const int gct = blockIdx.x * cteams + ct.index, nct = gridDim.x * cteams;
   // row tasks: the CTAs' warps (or warp-wide teams) in turn, so that a phase with fewer tasks
   // than teams spreads them over every CTA; a warp of narrower teams takes consecutive tasks
@@ -447,29 +585,35 @@ __global__ void __launch_bounds__(kThreads) spectral_fused_kernel(FusedArgs a) {
   for (int i = 0; i < a.cpt; ++i) {
     const int t = gct + i * nct;
     if (t >= col_tasks) break;
-    slab_task(a, t / a.nxh, t % a.nxh, 0, st + (size_t)i * ns, tb + (size_t)i * ns, cb,
+    slab_task<D3>(a, t / a.nxh, t % a.nxh, 0, st + (size_t)i * ns, tb + (size_t)i * ns, cb,
               cb + a.cbuf / 2, twy, twz, ct);
   }
-  if (!grid_barrier(a.bar, gridDim.x, a.budget)) return;
+  if (!grid_barrier(a.bar, target, a.budget)) return;
   for (int64_t step = 0; step < a.steps; ++step) {
     // teams narrower than a warp take their rounds together: the warp's first team decides
     // the trip count, and a team past the last task runs without touching W
     for (int t0 = rt0; t0 < row_tasks; t0 += nrt) {
       const int t = t0 + rt.index % rtpw;
       const bool valid = t < row_tasks;
-      if (MODEL == PF_MODEL_C) row_task<MODEL>(a, 0, t, 1, t, valid, rb, rb + a.nx, twx, rt);
-      else row_task<MODEL>(a, 0, 2 * t, 0, 2 * t + 1, valid, rb, rb + a.nx, twx, rt);
+      if (MODEL == PF_MODEL_C) row_task<MODEL>(a, 0, t, 1, t, valid, rb, rb2, twx, rt);
+      else row_task<MODEL>(a, 0, 2 * t, 0, 2 * t + 1, valid, rb, rb2, twx, rt);
     }
-    if (!grid_barrier(a.bar, gridDim.x, a.budget)) return;
+    if (!grid_barrier(a.bar, target, a.budget)) return;
     const int mode = step + 1 == a.steps ? 2 : 1;
     for (int i = 0; i < a.cpt; ++i) {
       const int t = gct + i * nct;
       if (t >= col_tasks) break;
-      slab_task(a, t / a.nxh, t % a.nxh, mode, st + (size_t)i * ns, tb + (size_t)i * ns, cb,
+      slab_task<D3>(a, t / a.nxh, t % a.nxh, mode, st + (size_t)i * ns, tb + (size_t)i * ns, cb,
                 cb + a.cbuf / 2, twy, twz, ct);
     }
-    if (mode == 1 && !grid_barrier(a.bar, gridDim.x, a.budget)) return;
+    if (mode == 1 && !grid_barrier(a.bar, target, a.budget)) return;
   }
+}
+
+template <int MODEL, bool D3>
+__global__ void __launch_bounds__(kThreads) spectral_fused_kernel(FusedArgs a) {
+  spectral_fused<MODEL, D3>(a);
+  grid_leave(a.bar);
 }
 
 bool is_pow2(int64_t n) { return n > 0 && (n & (n - 1)) == 0; }
@@ -537,10 +681,13 @@ FusedShape fused_shape_for(const pf_spectral_s* s, int sms, int threads, int col
   if (blocks > sms) blocks = sms;
   f.blocks = (int)blocks;
   f.cpt = (int)((col_tasks + blocks * cteams - 1) / (blocks * cteams));
-  f.rbuf = (int)(2 * d.nx + 2);  // b [nx], b2 [nx + 2]: b2 first takes both half spectra
-  f.cbuf = (int)(2 * d.nz * (d.ny + 1));  // two padded slabs: rows of ny + 1
+  // two padded rows; the second first takes both half spectra, nx + 2 values
+  f.rbuf = (int)(padded_size(d.nx) + std::max(d.nx + 2, padded_size(d.nx)));
+  // two padded slabs (rows of ny + 1) or, in 2D, columns
+  f.cbuf = (int)(2 * (s->dim == 3 ? d.nz * (d.ny + 1) : padded_size(d.ny)));
   const int64_t region = std::max(rteams * f.rbuf, cteams * f.cbuf);
-  f.smem = sizeof(float2) * (size_t)(d.nx + d.ny + d.nz + region + cteams * f.cpt * 2 * ns);
+  const int64_t tables = padded_size(d.nx) + padded_size(d.ny) + padded_size(d.nz);
+  f.smem = sizeof(float2) * (size_t)(tables + region + cteams * f.cpt * 2 * ns);
   const int64_t rrounds = (row_tasks + blocks * rteams - 1) / (blocks * rteams);
   const int64_t rb = (d.nx / 8 + f.row_team - 1) / f.row_team;  // butterflies per thread
   const int64_t cb = (ns / 8 + f.col_team - 1) / f.col_team;
@@ -569,17 +716,18 @@ FusedShape fused_shape(const pf_spectral_s* s, int sms) {
 }
 
 template <int MODEL>
-const void* fused_kernel_ptr() {
-  return reinterpret_cast<const void*>(&spectral_fused_kernel<MODEL>);
+const void* fused_kernel_ptr(bool d3) {
+  return d3 ? reinterpret_cast<const void*>(&spectral_fused_kernel<MODEL, true>)
+            : reinterpret_cast<const void*>(&spectral_fused_kernel<MODEL, false>);
 }
 
-const void* kernel_for(int model) {
-  if (model == PF_MODEL_AC) return fused_kernel_ptr<PF_MODEL_AC>();
-  if (model == PF_MODEL_CH) return fused_kernel_ptr<PF_MODEL_CH>();
-  return fused_kernel_ptr<PF_MODEL_C>();
+const void* kernel_for(int model, bool d3) {
+  if (model == PF_MODEL_AC) return fused_kernel_ptr<PF_MODEL_AC>(d3);
+  if (model == PF_MODEL_CH) return fused_kernel_ptr<PF_MODEL_CH>(d3);
+  return fused_kernel_ptr<PF_MODEL_C>(d3);
 }
 
-unsigned long long g_attr_mask[3] = {0, 0, 0};
+unsigned long long g_attr_mask[6] = {};
 
 }  // namespace
 
@@ -630,8 +778,9 @@ int spectral_fused_prepare(pf_spectral_s* s) {
   int sms = 0, optin = 0;
   if (int rc = device_limits(&sms, &optin)) return rc;
   const FusedShape f = fused_shape(s, sms);
-  const int mi = s->model == PF_MODEL_AC ? 0 : (s->model == PF_MODEL_CH ? 1 : 2);
-  const void* kern = kernel_for(s->model);
+  const bool d3 = s->dim == 3;
+  const int mi = 2 * (s->model == PF_MODEL_AC ? 0 : (s->model == PF_MODEL_CH ? 1 : 2)) + d3;
+  const void* kern = kernel_for(s->model, d3);
   int dev = 0;
   PF_CUDA_TRY(cudaGetDevice(&dev));
   // the limit is per kernel and device: set it once, to the device's opt-in maximum
@@ -688,7 +837,7 @@ int spectral_fused_run(pf_spectral_s* s, int64_t n_steps) {
   a.bar = s->d_bar;
   a.budget = kWaitBudgetCycles;
   void* args[] = {&a};
-  PF_CUDA_TRY(cudaLaunchCooperativeKernel(kernel_for(s->model), dim3(s->fused_blocks),
+  PF_CUDA_TRY(cudaLaunchCooperativeKernel(kernel_for(s->model, s->dim == 3), dim3(s->fused_blocks),
                                           dim3(s->fused_threads), args, s->fused_smem,
                                           s->stream));
   return PF_OK;
