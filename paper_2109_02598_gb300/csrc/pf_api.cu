@@ -238,16 +238,18 @@ int launch_depth(const pf_grid_s* g, int tile, int k) {
 
 // The tile and depth that run a 2D grid with the standard stencil where nothing was asked for
 // (us a step, against the 128x16 tiles at depth 1 that pf_get_tuning names; the same bits):
-//   up to 2^21 sites 32x32 tiles at the model's greatest depth (GS 128^2 0.78/2.38, 512^2
-//     1.05/2.52, 1502x1111 3.8/6.2; AC 512^2 0.76/2.11; Model B 512^2 1.57/2.55; Model C 512^2
-//     1.89/3.02);
-//   above, strips at that depth, 64 columns for two fields and 128 for one (2048^2 GS 6.2/11.5,
-//     AC 3.9/7.3, Model B 7.6/10.7, Model C 12.0/15.3; at 1502x1111 32x32 tiles are still level:
-//     GS 3.8/3.65, AC 2.25/2.36, Model B 4.7/4.65, Model C 6.8/7.0).
+//   up to 3 2^18 sites 32x32 tiles at the model's greatest depth (GS 128^2 0.78/2.38, 512^2
+//     1.06/2.51; AC 512^2 0.76/2.12; Model B 512^2 1.56/2.56; Model C 512^2 1.89/3.01);
+//   above, strips of 128 columns at that depth (2048^2 GS 4.8/11.5, AC 3.3/7.3, Model B 6.0/10.8,
+//     Model C 8.6/15.3; against the 32x32 tiles: 900x640 GS 1.94/1.63, AC 1.49/1.07, Model B
+//     2.80/2.25, Model C 3.48/2.87; 1024x777 1.95/2.22, 1.48/1.40, 2.78/2.88, 3.48/4.08);
+//   Model C above 3 2^21 sites, strips of 64 (of 128, twelve warps fit an SM, too few once the
+//     fields leave the L2 cache: 2500^2 14.8 us with either, 3000^2 18.9 against 21.9).
 void plan2d(const pf_grid_s* g, int* tile, int* depth) {
   const bool r1 = g->model == PF_MODEL_AC || g->model == PF_MODEL_GS;
-  const bool big = (int64_t)g->nx * g->ny > (int64_t)1 << 21;
-  *tile = big ? kTileStrips2D + (g->nf == 2 ? 1 : 0) : 2;
+  const int64_t n = (int64_t)g->nx * g->ny;
+  const bool narrow = g->model == PF_MODEL_C && n > (int64_t)3 << 21;
+  *tile = n > (int64_t)3 << 18 ? kTileStrips2D + (narrow ? 1 : 0) : 2;
   *depth = r1 ? 4 : 2;
 }
 

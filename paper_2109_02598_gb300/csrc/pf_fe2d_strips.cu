@@ -66,51 +66,30 @@ namespace {
 constexpr int kStripWarps = 1;
 constexpr int kStripThreads = 32 * kStripWarps;
 
-// A lane's C values of one row. xin (the same in every lane of the warp): every lane's
-// columns lie inside the row, so each takes one vector load (gx is a multiple of C and rows
-// start 16-byte aligned); otherwise every lane takes C periodic scalar loads, so the warp
-// never splits between the two paths.
+// A lane's C values of a row, and back: one access of C floats (x is a multiple of C and rows
+// start 16-byte aligned).
 template <int C>
-__device__ __forceinline__ void load_lane(const float* __restrict__ row, int gx, int nx,
-                                          bool xin, float (&v)[C]) {
-  if (xin) {
-    if constexpr (C == 4) {
-      const float4 q = __ldg(reinterpret_cast<const float4*>(row + gx));
-      v[0] = q.x;
-      v[1] = q.y;
-      v[2] = q.z;
-      v[3] = q.w;
-    } else if constexpr (C == 2) {
-      const float2 q = __ldg(reinterpret_cast<const float2*>(row + gx));
-      v[0] = q.x;
-      v[1] = q.y;
-    } else {
-      v[0] = __ldg(row + gx);
-    }
+__device__ __forceinline__ void load_vec(const float* __restrict__ p, float (&v)[C]) {
+  if constexpr (C == 4) {
+    const float4 q = __ldg(reinterpret_cast<const float4*>(p));
+    v[0] = q.x;
+    v[1] = q.y;
+    v[2] = q.z;
+    v[3] = q.w;
   } else {
-#pragma unroll
-    for (int j = 0; j < C; ++j) v[j] = __ldg(row + wrap_index(gx + j, nx));
+    static_assert(C == 2, "lanes of two or four columns");
+    const float2 q = __ldg(reinterpret_cast<const float2*>(p));
+    v[0] = q.x;
+    v[1] = q.y;
   }
 }
 
-// Store a lane's C values; xout (the same in every lane of the warp): every storing lane's
-// columns lie inside the row, else each column is stored only if it does.
 template <int C>
-__device__ __forceinline__ void store_lane(float* row, int gx, int nx, bool xout,
-                                           const float (&v)[C]) {
-  if (xout) {
-    if constexpr (C == 4) {
-      *reinterpret_cast<float4*>(row + gx) = make_float4(v[0], v[1], v[2], v[3]);
-    } else if constexpr (C == 2) {
-      *reinterpret_cast<float2*>(row + gx) = make_float2(v[0], v[1]);
-    } else {
-      row[gx] = v[0];
-    }
-  } else {
-#pragma unroll
-    for (int j = 0; j < C; ++j)
-      if (gx + j < nx) row[gx + j] = v[j];
-  }
+__device__ __forceinline__ void store_vec(float* p, const float (&v)[C]) {
+  if constexpr (C == 4)
+    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+  else
+    *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
 }
 
 // Packed FP32 pairs (one instruction updates two sites, each lane's result the scalar
@@ -180,7 +159,15 @@ __device__ __forceinline__ void lap_lane(const float (&u)[C], const float (&c)[C
   }
 }
 
-template <int MODEL, int K, int C, int ST = PF_ST_STD>
+// RAG: the row length is no multiple of C. Otherwise a lane's columns, wrapped once into the row,
+// are C consecutive floats wherever the strip lies, and every load and store is a vector one; with
+// RAG only those of a strip that lies inside the row are, and the lanes of the others take their
+// columns one by one, at offsets wrapped once per task. (A launch ends with its slowest tasks, and
+// those were the strips at the row's ends, as long as they wrapped every column in every row. Us a
+// step, before and now, 128 columns: 2048^2 Gray-Scott 8.2 -> 4.8, Allen-Cahn 3.9 -> 3.3, Model B
+// 7.6 -> 6.0, Model C 13.1 -> 8.8; 1499 x 1501 5.7 -> 3.6, 2.8 -> 2.7, 5.4 -> 4.9, 8.9 -> 6.3; 64
+// columns: 2048^2 Gray-Scott 6.3 -> 5.3, Model C 12.1 -> 10.0.)
+template <int MODEL, int K, int C, bool RAG, int ST = PF_ST_STD>
 struct StripRun {
   static_assert(ST == PF_ST_STD || ModelTraits<MODEL>::R == 1,
                 "the 9-point stencil runs on the radius-1 models");
@@ -195,8 +182,27 @@ struct StripRun {
   FieldPtrs in;
   FieldOut out;
   int nx, ny, y0, hy, gx;
+  int xw[RAG ? C : 1];  // RAG: the lane's columns, wrapped
   int64_t pitch;
   bool st_lane, xin, xout;
+
+  __device__ __forceinline__ void load_row(const float* __restrict__ row, float (&v)[C]) const {
+    if (!RAG || xin) {
+      load_vec<C>(row + gx, v);
+    } else {
+#pragma unroll
+      for (int j = 0; j < C; ++j) v[j] = __ldg(row + xw[RAG ? j : 0]);
+    }
+  }
+  __device__ __forceinline__ void store_row(float* row, const float (&v)[C]) const {
+    if (!RAG || xout) {
+      store_vec<C>(row + gx, v);
+    } else {
+#pragma unroll
+      for (int j = 0; j < C; ++j)
+        if (gx + j < nx) row[gx + j] = v[j];
+    }
+  }
 
   // Level s (1..K) at an iteration of phase P; its new row goes to o.
   template <int P, int s>
@@ -310,7 +316,7 @@ struct StripRun {
       if (st_lane && (!G || t >= T0)) {
         const int64_t row = (int64_t)(y0 + t - T0) * pitch;
 #pragma unroll
-        for (int f = 0; f < NF; ++f) store_lane<C>(out.f[f] + row, gx, nx, xout, o[f]);
+        for (int f = 0; f < NF; ++f) store_row(out.f[f] + row, o[f]);
       }
     }
     inner_levels<P, G, K - 1>(t, m);
@@ -318,7 +324,7 @@ struct StripRun {
     if (!G || t < rows_in()) {
       const int64_t row = (int64_t)wrap_index(y0 - R * K + t, ny) * pitch;
 #pragma unroll
-      for (int f = 0; f < NF; ++f) load_lane<C>(in.f[f] + row, gx, nx, xin, w[0][f][P]);
+      for (int f = 0; f < NF; ++f) load_row(in.f[f] + row, w[0][f][P]);
     }
   }
 
@@ -337,10 +343,17 @@ struct StripRun {
     const int lane = threadIdx.x & 31;
     gx = x0 - S::HXP + C * lane;
     st_lane = lane >= S::HXP / C && lane < (S::HXP + wo + C - 1) / C;
-    // strips that reach past either end of the row (every strip of a narrow grid or batch
-    // instance) take the periodic paths with the whole warp
-    xin = __all_sync(0xffffffffu, gx >= 0 && gx + C <= nx);
-    xout = __all_sync(0xffffffffu, !st_lane || gx + C <= nx);
+    if constexpr (RAG) {
+      // (strips that reach past either end of the row take the columns one by one with the whole
+      // warp)
+#pragma unroll
+      for (int j = 0; j < C; ++j) xw[j] = wrap_index(gx + j, nx);
+      xin = __all_sync(0xffffffffu, gx >= 0 && gx + C <= nx);
+      xout = __all_sync(0xffffffffu, !st_lane || gx + C <= nx);
+    } else {
+      st_lane = st_lane && gx < nx;
+      gx = wrap_index(gx, nx);
+    }
     const int t_main = rows_in();  // the input rows end here
     int t = 0;
     for (; t < T0; t += 3) {  // start-up: levels begin one after another
@@ -363,7 +376,7 @@ struct StripRun {
 
 // One warp per task: strips of WO output columns by rows of hy (the last row of tasks is
 // shorter); consecutive warps take neighbouring strips of the same rows.
-template <int MODEL, int K, int C, int ST>
+template <int MODEL, int K, int C, bool RAG, int ST>
 __global__ void __launch_bounds__(kStripThreads, (StripCfg<MODEL, K, C>::MINW / kStripWarps))
     fe2d_strip_kernel(FieldPtrs in, FieldOut out, Geom g, ModelParams m, int hy, int tasks_x,
                       int ntasks) {
@@ -373,7 +386,7 @@ __global__ void __launch_bounds__(kStripThreads, (StripCfg<MODEL, K, C>::MINW / 
   const int ty = task / tasks_x;
   const int tx = task - ty * tasks_x;
   const int y0 = ty * hy;
-  StripRun<MODEL, K, C, ST> r;
+  StripRun<MODEL, K, C, RAG, ST> r;
   r.run(in, out, g.nx, g.ny, g.pitch, tx * S::WO, S::WO, y0, min(hy, g.ny - y0), m);
 }
 
@@ -395,19 +408,24 @@ __global__ void __launch_bounds__(kStripThreads, (StripCfg<PF_MODEL_GS, K, C>::M
   in.f[1] = in_base + I.off + plane;
   out.f[0] = out_base + I.off;
   out.f[1] = out_base + I.off + plane;
-  StripRun<PF_MODEL_GS, K, C> r;
-  r.run(in, out, I.nx, I.ny, I.pitch, t.x0, t.wo, t.y0, t.hy, I.m);
+  if (I.nx % C == 0) {
+    StripRun<PF_MODEL_GS, K, C, false> r;
+    r.run(in, out, I.nx, I.ny, I.pitch, t.x0, t.wo, t.y0, t.hy, I.m);
+  } else {
+    StripRun<PF_MODEL_GS, K, C, true> r;
+    r.run(in, out, I.nx, I.ny, I.pitch, t.x0, t.wo, t.y0, t.hy, I.m);
+  }
 }
 
 // Rows per task: the height that makes the launch shortest by waves * (rows + T0) * (100 + w), w
 // the warps per SM of a wave. A task takes T0 iterations beside its rows, and an iteration is
-// mostly latency: its time grows with the resident warps only as 100 + w (fitted to 2200 timed
-// launches, all four models, depths 2 and 4, both widths, 256^2 to 4096^2; its choice is within
-// 5 % of the best height timed on nine of ten). So a wave is filled with the lowest tasks that
-// still fit it, and grids of many rows take a few waves. The rule before (one wave unless that
-// makes tasks of fewer than 4 T0 rows, then that height) left a 1502 x 1111 grid with four warps
-// per SM: Gray-Scott, 64 columns, k = 4: 7.4 -> 3.45 us a step (the tiled kernel 3.8), 2048^2
-// 8.6 -> 6.2; Allen-Cahn 4096^2 at 128 columns 11.4 -> 10.5, Model B 4096^2 20.1 -> 18.2.
+// half latency: its time grows with the resident warps only as 40 + w (timed over 16 heights, all
+// four models at their greatest depth, both widths, 512^2 to 4096^2: its choice is within 2 % of
+// the best height on the mean and 8 % at worst). So a wave is filled with the lowest tasks that
+// still fit it, and grids of many rows take a few waves. One wave unless that makes tasks of fewer
+// than 4 T0 rows, then that height, left a 1502 x 1111 grid with four warps per SM: Gray-Scott, 64
+// columns, k = 4: 7.4 us a step, now 3.0; Allen-Cahn 4096^2 at 128 columns 11.4, now 10.1; Model B
+// 4096^2 20.1, now 17.5.
 constexpr int kStripMinRows = 4;
 int strip_rows(int tasks_x, int ny, int resident_warps, int sms, int t0) {
   int best = ny;
@@ -420,7 +438,7 @@ int strip_rows(int tasks_x, int ny, int resident_warps, int sms, int t0) {
     hy = hy < ny ? hy : ny;
     const long long n = (long long)tasks_x * ((ny + hy - 1) / hy);
     const double w = (double)(n < resident_warps ? n : resident_warps) / sms;
-    const double c = (double)((n + resident_warps - 1) / resident_warps) * (hy + t0) * (100.0 + w);
+    const double c = (double)((n + resident_warps - 1) / resident_warps) * (hy + t0) * (40.0 + w);
     if (cost < 0 || c < cost) {
       cost = c;
       best = hy;
@@ -430,11 +448,11 @@ int strip_rows(int tasks_x, int ny, int resident_warps, int sms, int t0) {
   return cost < 0 ? (ny < 4 * t0 ? ny : 4 * t0) : best;
 }
 
-template <int MODEL, int K, int C, int ST>
+template <int MODEL, int K, int C, bool RAG, int ST>
 cudaError_t launch_strip(const Geom& g, FieldPtrs in, FieldOut out, const ModelParams& m,
                          cudaStream_t s) {
   using S = StripCfg<MODEL, K, C>;
-  using Run = StripRun<MODEL, K, C, ST>;
+  using Run = StripRun<MODEL, K, C, RAG, ST>;
   static int resident[64] = {}, sms_of[64] = {};  // resident warps of this kernel, SMs
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -442,7 +460,7 @@ cudaError_t launch_strip(const Geom& g, FieldPtrs in, FieldOut out, const ModelP
   if (dev >= 64) return cudaErrorInvalidDevice;
   if (resident[dev] == 0) {
     int b = 0, sms = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fe2d_strip_kernel<MODEL, K, C, ST>,
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fe2d_strip_kernel<MODEL, K, C, RAG, ST>,
                                                       kStripThreads, 0);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
@@ -453,18 +471,25 @@ cudaError_t launch_strip(const Geom& g, FieldPtrs in, FieldOut out, const ModelP
   const int hy = strip_rows(tasks_x, g.ny, resident[dev], sms_of[dev], Run::T0);
   const int ntasks = tasks_x * ((g.ny + hy - 1) / hy);
   const int blocks = (ntasks + kStripWarps - 1) / kStripWarps;
-  fe2d_strip_kernel<MODEL, K, C, ST><<<blocks, kStripThreads, 0, s>>>(in, out, g, m, hy,
+  fe2d_strip_kernel<MODEL, K, C, RAG, ST><<<blocks, kStripThreads, 0, s>>>(in, out, g, m, hy,
                                                                       tasks_x, ntasks);
   return cudaGetLastError();
+}
+
+template <int MODEL, int K, int C, int ST>
+cudaError_t launch_strip_rag(const Geom& g, FieldPtrs in, FieldOut out, const ModelParams& m,
+                             cudaStream_t s) {
+  return g.nx % C == 0 ? launch_strip<MODEL, K, C, false, ST>(g, in, out, m, s)
+                       : launch_strip<MODEL, K, C, true, ST>(g, in, out, m, s);
 }
 
 template <int MODEL, int C, int ST>
 cudaError_t launch_strip_k(int k, const Geom& g, FieldPtrs in, FieldOut out,
                            const ModelParams& m, cudaStream_t s) {
-  if (k == 1) return launch_strip<MODEL, 1, C, ST>(g, in, out, m, s);
-  if (k == 2) return launch_strip<MODEL, 2, C, ST>(g, in, out, m, s);
+  if (k == 1) return launch_strip_rag<MODEL, 1, C, ST>(g, in, out, m, s);
+  if (k == 2) return launch_strip_rag<MODEL, 2, C, ST>(g, in, out, m, s);
   if constexpr (ModelTraits<MODEL>::R == 1) {
-    if (k == 4) return launch_strip<MODEL, 4, C, ST>(g, in, out, m, s);
+    if (k == 4) return launch_strip_rag<MODEL, 4, C, ST>(g, in, out, m, s);
   }
   return cudaErrorInvalidValue;
 }
