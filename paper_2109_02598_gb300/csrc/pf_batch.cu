@@ -102,7 +102,11 @@ static int kslot(int k) { return k == 4 ? 2 : k == 2 ? 1 : 0; }
 // 48 rows on 2432 resident warps ran 46 % slower than 2415 tasks of 60 rows). Each
 // candidate height's list is played through that dispatch on the resident warps, with a
 // task costing its iterations (rows + the levels' start-up), and the shortest makespan wins
-// (the taller height on a tie).
+// (the taller height on a tie); an iteration is half latency and takes 40 + w, w the warps per SM
+// (pf_fe2d_strips.cu). Heights below the floor only where the list fits two waves of warps: they
+// fill the chip for batches of a few million sites and less (2.9 million in 64 instances, 64
+// columns, k = 4: 5.7 -> 5.2 us a step, 0.46 million in 20: 5.0 -> 2.6), and longer lists would
+// take the host long to play through.
 static std::vector<int> strip_bounds(int nx, int w) {
   const int s = (nx + w - 1) / w;
   std::vector<int> b(s + 1);
@@ -114,6 +118,13 @@ static std::vector<int> strip_bounds(int nx, int w) {
 static double strip_makespan(const pf_batch_s* b, const std::vector<int>& order,
                              const std::vector<int>& nstrips, int hy, int k, int resident,
                              std::vector<double>& slots) {
+  int64_t tasks = 0;
+  int tallest = 0;
+  for (int i : order) {
+    tasks += (int64_t)nstrips[i] * ((b->ny[i] + hy - 1) / hy);
+    tallest = std::max(tallest, (int)std::min<int64_t>(hy, b->ny[i]));
+  }
+  if (tasks <= resident) return tallest + 3.0 * k;  // a warp each
   slots.assign((size_t)resident, 0.0);
   std::make_heap(slots.begin(), slots.end(), std::greater<double>());
   double span = 0;
@@ -154,12 +165,19 @@ static cudaError_t batch_strips(pf_batch_s* b, int t, int k) {
   // play through cheaply (a list of a few million tasks is past every tail effect anyway)
   const int resident = batch_gs2d_strips_resident(k, c);
   const int floor_rows = strip_task_rows(PF_MODEL_GS, k);
-  int hy = 0;
+  int hy = 0, dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
   double best = 0;
   std::vector<double> slots;
-  for (int h = floor_rows; h <= 192; h += 4) {
-    if (strip_rows_total / h > (int64_t)1 << 22 && h < 192) continue;
-    const double span = strip_makespan(b, order, nstrips, h, k, resident, slots);
+  for (int h = 4; h <= 192; h += 4) {
+    const int64_t tasks = strip_rows_total / h;
+    if (tasks > (int64_t)1 << 22 && h < 192) continue;
+    if (h < floor_rows && tasks > 2 * (int64_t)resident) continue;
+    const double w = (double)std::min<int64_t>(tasks, resident) / std::max(sms, 1);
+    const double span =
+        strip_makespan(b, order, nstrips, h, k, resident, slots) * (40.0 + w);
     if (hy == 0 || span <= best) {
       best = span;
       hy = h;
@@ -177,7 +195,7 @@ static cudaError_t batch_strips(pf_batch_s* b, int t, int k) {
       }
   }
   if (list.size() > (size_t)INT32_MAX) return cudaErrorInvalidValue;
-  cudaError_t e = cudaMalloc(&b->d_strips[slot], sizeof(BatchStrip) * list.size());
+  e = cudaMalloc(&b->d_strips[slot], sizeof(BatchStrip) * list.size());
   if (e != cudaSuccess) return e;
   e = cudaMemcpy(b->d_strips[slot], list.data(), sizeof(BatchStrip) * list.size(),
                  cudaMemcpyHostToDevice);
@@ -364,25 +382,57 @@ int pf_batch_autotune(pf_batch_t b, int probe_launches, int* tile_x, int* tile_y
   cudaEvent_t e0, e1;
   PF_CUDA_TRY(cudaEventCreate(&e0));
   PF_CUDA_TRY(cudaEventCreate(&e1));
+  // Candidates run as a replayed graph of launches that go back and forth between the two buffers,
+  // as a run does (launched one by one, short launches of a small batch cost the host's time and
+  // the deeper ones won too often), and the state is put back from a copy. Without the memory for
+  // one, every launch reads the state and writes the other buffer.
+  const int n_l = probe_launches > 8 ? probe_launches : 8;
+  const size_t bytes = sizeof(float) * (size_t)b->total_floats;
+  float* saved = nullptr;
+  cudaError_t e = cudaMalloc(&saved, bytes);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    saved = nullptr;
+    e = cudaSuccess;
+  } else {
+    e = cudaMemcpyAsync(saved, b->base[b->cur], bytes, cudaMemcpyDeviceToDevice, b->stream);
+  }
   float best = INFINITY;
   int bt = b->tile, bk = b->k;
   static const int ks[3] = {1, 2, 4};
-  cudaError_t e = cudaSuccess;
   for (int ti = 0; ti < kNumTiles2D + 2 && e == cudaSuccess; ++ti) {
     // the tiles, then the strip kernel with 128- and 64-column strips
     const int t = ti < kNumTiles2D ? ti : kTileStrips2D + (ti - kNumTiles2D);
     for (int ki = 0; ki < 3 && e == cudaSuccess; ++ki) {
       const int k = ks[ki];
-      e = batch_launch(b, t, k, b->cur, b->stream);  // warm-up (state unchanged)
-      if (e == cudaSuccess) e = cudaEventRecord(e0, b->stream);
-      for (int i = 0; i < probe_launches && e == cudaSuccess; ++i)
-        e = batch_launch(b, t, k, b->cur, b->stream);
-      if (e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
-      if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-      float ms = 0;
-      if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-      if (e == cudaSuccess && ms / (probe_launches * k) < best) {
-        best = ms / (probe_launches * k);
+      // the work list, outside the capture
+      e = t >= kTileStrips2D ? batch_strips(b, t, k) : batch_tiles(b, t);
+      if (e == cudaSuccess)
+        e = cudaStreamBeginCapture(b->capture, cudaStreamCaptureModeThreadLocal);
+      if (e != cudaSuccess) break;
+      for (int i = 0; i < n_l && e == cudaSuccess; ++i)
+        e = batch_launch(b, t, k, saved != nullptr && (i & 1) ? 1 - b->cur : b->cur, b->capture);
+      cudaGraph_t graph = nullptr;
+      cudaGraphExec_t probe = nullptr;
+      const cudaError_t e2 = cudaStreamEndCapture(b->capture, &graph);
+      if (e == cudaSuccess) e = e2;
+      if (e == cudaSuccess) e = cudaGraphInstantiate(&probe, graph, 0);
+      if (graph) cudaGraphDestroy(graph);
+      float ms = INFINITY;
+      // a first run, and a second where the first comes near the best so far
+      for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {
+        if (rep > 0 && ms > 1.5f * best * n_l * k) break;
+        e = cudaEventRecord(e0, b->stream);
+        if (e == cudaSuccess) e = cudaGraphLaunch(probe, b->stream);
+        if (e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
+        if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+        float t_ms = 0;
+        if (e == cudaSuccess) e = cudaEventElapsedTime(&t_ms, e0, e1);
+        if (t_ms < ms) ms = t_ms;
+      }
+      if (probe) cudaGraphExecDestroy(probe);
+      if (e == cudaSuccess && ms / (n_l * k) < best) {
+        best = ms / (n_l * k);
         bt = t;
         bk = k;
       }
@@ -390,6 +440,13 @@ int pf_batch_autotune(pf_batch_t b, int probe_launches, int* tile_x, int* tile_y
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
+  if (saved != nullptr) {
+    const cudaError_t er = cudaMemcpyAsync(b->base[b->cur], saved, bytes,
+                                           cudaMemcpyDeviceToDevice, b->stream);
+    cudaStreamSynchronize(b->stream);
+    cudaFree(saved);
+    if (e == cudaSuccess) e = er;
+  }
   if (e != cudaSuccess) return cuda_fail(e, "pf_batch_autotune");
   b->tile = bt;
   b->k = bk;
