@@ -256,8 +256,8 @@ void plan2d(const pf_grid_s* g, int* tile, int* depth) {
 // The tile and depth pf_step runs: the tuning in effect, except where it is the library's own
 // choice (nothing asked for) and the stencil the standard one. Then a kernel that passes the one
 // pf_get_tuning names takes its place, with the same bits: plan2d's, and in 3D the general tile's
-// for the depth-1 TMA tiles (256^3 GS 572 against 369 GLUPS, AC 979/716, Model B 520/393, Model C
-// 317/165; 64^3 GS 117/60, Model B 74/38).
+// for the depth-1 TMA tiles (256^3 GS 585 against 369 GLUPS, AC 1015/716, Model B 536/393, Model C
+// 328/165; 64^3 GS 130/60, Model B 87/38).
 void run_plan(const pf_grid_s* g, int* tile, int* depth) {
   const bool untuned = g->stencil == PF_ST_STD && g->model != PF_MODEL_RD && g->req_tile < 0 &&
                        g->req_k == 0;

@@ -16,10 +16,10 @@
 //
 // Bound by latency at small sizes (a CTA takes only some ten planes a launch, behind a
 // prologue) and by issue at large ones. Two CTAs per SM (one of 640 threads waits at its barrier
-// with nothing else to run: 27-point 160^3 209 GLUPS against 285); three of 256 leave the species
-// too few registers. GLUPS against the kernels it replaces, 160^3 and 256^3: Gray-Scott 27-point
-// 158 -> 285 and 160 -> 372, 19-point 167 -> 298 and 166 -> 380; Allen-Cahn 27-point 265 -> 440
-// and 297 -> 602; three species 116 -> 166 and 119 -> 184 (136 x 144 x 160: 108 -> 153).
+// with nothing else to run: 27-point 160^3 209 GLUPS, then 285 with two); three of 256 leave the
+// species too few registers. GLUPS against the kernels it replaces, 160^3: Gray-Scott 27-point 158
+// -> 302, 19-point 167 -> 312; Allen-Cahn 27-point 265 -> 485; three species 116 -> 186 (136 x 144
+// x 160: 108 -> 176). Ragged rows (161^3): 255, 278, 392 and 153.
 #include "pf_fe3d_stream.cuh"
 #include "pf_grid.h"
 #include "pf_rd.cuh"
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(U::NT, U::CTAS)
   const bool live = tid < R * G;  // the last warp's spare threads repeat the last group
   const int t_ = live ? tid : R * G - 1;
   const int r = t_ / G, q = t_ - r * G;
-  const GroupPos t(G, q);
+  const GroupPos t(G, q, RAGGED > 0 && pl.lpad == 0 ? g.nx : 4 * G);
   const int oi = (r + 1) * t.rw + 4 * q;  // own group in an input plane
 
   const int ncols = pl.S * ((g.ny + TY - 1) / TY);
@@ -205,7 +205,6 @@ __global__ void __launch_bounds__(U::NT, U::CTAS)
     // where this thread stores
     const int gy = y0 + r, gx = x0 - pl.lpad + 4 * q;
     const bool store = live && r < TY && gy < g.ny && gx >= x0 && gx < x1;
-    const bool whole = gx + 3 < x1;
     int64_t off = (int64_t)zfirst * g.plane + (int64_t)gy * g.pitch + gx;
     const int64_t off_step = dir > 0 ? g.plane : -g.plane;
 
@@ -232,19 +231,7 @@ __global__ void __launch_bounds__(U::NT, U::CTAS)
       s0 = s1;
       s1 = s2;
       if (++s2 == NS) s2 = 0;
-      if (store) {
-        if (whole) {
-#pragma unroll
-          for (int f = 0; f < NF; ++f) *reinterpret_cast<float4*>(out.f[f] + off) = res[f];
-        } else {
-#pragma unroll
-          for (int f = 0; f < NF; ++f) {
-            out.f[f][off] = res[f].x;
-            if (gx + 1 < x1) out.f[f][off + 1] = res[f].y;
-            if (gx + 2 < x1) out.f[f][off + 2] = res[f].z;
-          }
-        }
-      }
+      if (store) store_group<NF, RAGGED>(out, off, res, gx, x1);
       off += off_step;
     };
     for (int j = 0; j < n; j += U::PHASES) {

@@ -10,15 +10,18 @@ namespace pf {
 
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 
-// A thread's group in a row-major plane of rows of rw floats.
+// A thread's group in a row-major plane of rows of rw floats. cols: the columns after which the row
+// repeats. Whole rows: nx, and a last group of nx % 4 columns holds the first columns behind them,
+// periodic images that every level computes like the columns they repeat (their right neighbour
+// is the column after the last image); strips: any, their outermost columns are not used.
 struct GroupPos {
   int rw;       // floats per row: four per group
   int dm, dp;   // offsets of the group's x-neighbours from its first float
   bool nl, nr;  // take them from shared memory (a warp's or a row's end)
-  __device__ __forceinline__ GroupPos(int G, int q) {
+  __device__ __forceinline__ GroupPos(int G, int q, int cols) {
     rw = 4 * G;
-    dm = q == 0 ? 4 * G - 1 : -1;
-    dp = q == G - 1 ? 4 - 4 * G : 4;
+    dm = q == 0 ? cols - 1 : -1;
+    dp = q == G - 1 ? 4 - cols : 4;
     nl = (threadIdx.x & 31) == 0 || q == 0;
     nr = (threadIdx.x & 31) == 31 || q == G - 1;
   }
@@ -38,9 +41,9 @@ struct GroupPos {
 // floats, fields IN_FIELD apart. With R rows of threads (at least T / 2 + H), a thread copies its
 // group of row r and of row R + r where there is one, from a pointer that moves on with the plane
 // (the fields lie at constant distances).
-// RAGGED > 0 (nx % 4 != 0): groups that are not four consecutive columns of the grid (the ends of
-// the rows) come as 4-byte copies of the columns within H of the strip; 1: at most one a thread,
-// 2: several (short rows). Instantiations of their own: on aligned rows the state and the tests
+// RAGGED > 0 (nx % 4 != 0): groups that are not four consecutive columns of the grid come as 4-byte
+// copies: a whole row's last group, of a strip the columns within H of it at the ends of the rows;
+// 1: at most one a thread, 2: several (short rows). Instantiations of their own: on aligned rows the state and the tests
 // alone cost every warp 46 of 221 instructions a plane (one step of Gray-Scott), and the loop of
 // 2 costs the others 4 to 10 %.
 template <int NF, int H, int IN_FIELD, int RAGGED>
@@ -51,7 +54,7 @@ struct PlaneCopy {
   int64_t step, wrap;   // to the next plane, and past the grid's last (or first) one
   bool has_a, has_b, warp_b;
   // the 4-byte copies: columns a row, left ones, first right one
-  int nsc, nl, fr, items, sdst, x0, y0, T, rw;
+  int nsc, nl, fr, items, sdst, xs, y0, T, rw;
   const float* ps;
 
   __device__ __forceinline__ const float* scalar_item(const FieldPtrs& in, const Geom& g, int i,
@@ -63,7 +66,7 @@ struct PlaneCopy {
 #pragma unroll
     for (int j = 1; j < NF; ++j)
       if (f == j) base = in.f[j];
-    dst = f * IN_FIELD + row * rw + (cx - (x0 - 4));
+    dst = f * IN_FIELD + row * rw + (cx - xs);
     return base + ((int64_t)zin * g.plane + (int64_t)wrap_index(y0 - H + row, g.ny) * g.pitch +
                    wrap_index(cx, g.nx));
   }
@@ -91,14 +94,14 @@ struct PlaneCopy {
     db = (int64_t)(yb - ya) * g.pitch;
     pa = in.f[0] + o;
     if constexpr (RAGGED > 0) {
-      x0 = x0_;
+      xs = x0_ - lpad;
       y0 = y0_;
       T = T_;
-      // H columns left of the first strip, and from the grid's last whole group to H past the
-      // strip's last column
-      nl = x0 == 0 ? H : 0;
-      fr = max(g.nx & ~3, x0 - 4);
-      nsc = nl + max(0, x1 + H - fr);
+      // strips: H columns left of the first one, and from the grid's last whole group to H past
+      // the strip's last column
+      nl = lpad > 0 && x0_ == 0 ? H : 0;
+      fr = max(g.nx & ~3, xs);
+      nsc = lpad > 0 ? nl + max(0, x1 + H - fr) : 4;
       items = NF * (T + 2 * H) * nsc;
       sdst = 0;
       ps = nullptr;
@@ -139,6 +142,23 @@ struct PlaneCopy {
       if (ps != nullptr) ps += s;
   }
 };
+
+// Store a thread's group of output columns gx .. gx + 3, those from x1 on as zeros: strips are a
+// multiple of 4 wide, so they are the places behind the row's end, which stay zero that way (one
+// vector store for every group: 4 to 6 % faster on ragged rows than column by column at their ends).
+template <int NF, int RAGGED>
+__device__ __forceinline__ void store_group(const FieldOut& out, int64_t off, float4 (&v)[NF],
+                                            int gx, int x1) {
+#pragma unroll
+  for (int f = 0; f < NF; ++f) {
+    if constexpr (RAGGED > 0) {
+      if (gx + 1 >= x1) v[f].y = 0.f;
+      if (gx + 2 >= x1) v[f].z = 0.f;
+      if (gx + 3 >= x1) v[f].w = 0.f;
+    }
+    *reinterpret_cast<float4*>(out.f[f] + off) = v[f];
+  }
+}
 
 // A CTA's segments (column tile, z-range, direction) of the schedule.
 struct SegmentWalk {
@@ -191,27 +211,29 @@ struct SegmentWalk {
 
 // The PlaneCopy form for a tile: whether its 4-byte copies fit one a thread.
 inline int copy_form(const Geom& g, const StreamTiles& p, int nf, int H, int threads) {
-  return g.nx % 4 == 0 ? 0 : nf * (p.TY + 2 * H) * (2 * H + 3) <= threads ? 1 : 2;
+  const int row = p.lpad > 0 ? 2 * H + 3 : 4;  // copies a row (at most)
+  return g.nx % 4 == 0 ? 0 : nf * (p.TY + 2 * H) * row <= threads ? 1 : 2;
 }
 
 // Tiles and work split of a grid for a kernel of at most nt threads, row-halo H, whose threads
-// cover T = TY + trim rows. Rows of at most 4 maxg columns whole, longer (or ragged) ones in
-// equal strips; the tile height that makes the launch shortest by span * (c0 + warps): the
+// cover T = TY + trim rows. Rows of at most 4 maxg columns whole, longer ones in
+// equal strips (ragged rows too: as strips with a halo group on either side and seven 4-byte copies
+// a row they took 3 to 25 % longer, the longer the shorter the row); the tile height that makes the launch shortest by span * (c0 + warps): the
 // longest CTA's plane count times a plane's time, linear in the CTA's warps above a fixed part
 // for the barrier and the latencies behind it.
 inline StreamPlan stream_plan(const Geom& g, long long sms, int nt, int maxg, int H, int trim,
                               int c0) {
   StreamPlan pl{};
   StreamTiles& p = pl.tiles;
-  if (g.nx % 4 == 0 && g.nx <= 4 * maxg) {
-    p.G = g.nx / 4;
+  if (g.nx <= 4 * maxg) {
+    p.G = (g.nx + 3) / 4;
     p.S = 1;
     p.w = g.nx;
   } else {
     const int wmax = 4 * maxg - 8;
     p.lpad = 4;
     p.S = (g.nx + wmax - 1) / wmax;
-    p.w = p.S == 1 ? g.nx : ((g.nx + p.S - 1) / p.S + 3) / 4 * 4;
+    p.w = ((g.nx + p.S - 1) / p.S + 3) / 4 * 4;
     p.S = (g.nx + p.w - 1) / p.w;
     p.G = (4 + p.w + H + 3) / 4;  // the halo group, w columns, and H more columns
   }

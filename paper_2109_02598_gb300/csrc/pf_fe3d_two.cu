@@ -17,18 +17,19 @@
 // output plane j - 2 from level-1 planes j - 2, j - 1, j (again the z-neighbours in registers);
 // one CTA barrier per plane. x-neighbours come from the neighbouring lanes by shuffle, and at a
 // warp's or a row's end from shared memory.
-//   Full rows (nx a multiple of 4, at most 256): G = nx / 4, the row wraps in shared memory.
-//   Strips (all other nx): one halo group on the left, enough on the right for two columns,
+//   Whole rows (nx at most 256): G = nx / 4, rounded up; the row wraps in shared memory, and a
+//     last group of nx % 4 columns is filled up with periodic images of the first ones.
+//   Strips (longer rows): one halo group on the left, enough on the right for two columns,
 //     staged at periodic columns; the level-1 values of a strip's outermost columns are wrong
-//     and reach only columns that the strip does not store. Groups that are not four
-//     consecutive columns of the grid (the ends of a row of nx % 4 != 0 columns) come as
-//     4-byte copies, one or two per thread, of the columns the levels read.
+//     and reach only columns that the strip does not store.
+//   Groups that are not four consecutive columns of the grid (the ends of a row of nx % 4 != 0
+//     columns) come as 4-byte copies of the columns the levels read.
 //
 // What bounds it (two time steps of Gray-Scott, 256^3, 640 threads, one CTA per SM): issue and
 // the latencies behind the plane barrier; a plane takes 0.37 us + 0.035 us per warp. GLUPS
 // against the general kernels it replaces (32x16 tiles, 4-byte copies or one plane in flight):
-// GS 210x179x150 386 / 191, 256^3 572 / 200; AC 210x179x150 648 / 301, 256^3 979 / 376; Model B
-// 335 / 102 and 520 / 134; Model C 213 / 88 and 317 / 110 (TMA tiles, 256^3: 369, 716, 393,
+// GS 210x179x150 416 / 191, 256^3 585 / 200; AC 210x179x150 732 / 301, 256^3 1015 / 376; Model B
+// 382 / 102 and 536 / 134; Model C 232 / 88 and 328 / 110 (TMA tiles, 256^3: 369, 716, 393,
 // 165). NS = 5 planes leave three in flight over a plane's 1.1 us (4 and 6 measured the same).
 // 640 threads: with 768 (80 registers) GS 256^3 gains 3 %, but AC, Models B and C lose 1 to
 // 10 %; two CTAs of 320 threads per SM lose 17 % there (shorter tiles, more halo) and gain 2 to
@@ -152,7 +153,7 @@ __global__ void __launch_bounds__(kTwoThreads, 1)
   const bool live = tid < (TY + 2) * G;  // the last warp's spare threads repeat the last group
   const int t_ = live ? tid : (TY + 2) * G - 1;
   const int r = t_ / G, q = t_ - r * G;
-  const GroupPos t(G, q);
+  const GroupPos t(G, q, RAGGED > 0 && pl.lpad == 0 ? g.nx : 4 * G);
   const int o1 = r * t.rw + 4 * q;  // own group in a level-1 plane; in an input plane o1 + rw
   const int ym2 = r > 0 ? -t.rw : 0, yp2 = r < TY + 1 ? t.rw : 0;  // rows level 2 may read
   const bool inner = r >= 1 && r <= TY;
@@ -177,7 +178,6 @@ __global__ void __launch_bounds__(kTwoThreads, 1)
     // where this thread stores: its output row and columns
     const int gy = y0 + r - 1, gx = x0 - pl.lpad + 4 * q;
     const bool store = live && inner && gy < g.ny && gx >= x0 && gx < x1;
-    const bool whole = gx + 3 < x1;
     int64_t off = (int64_t)zfirst * g.plane + (int64_t)gy * g.pitch + gx;
     const int64_t off_step = dir > 0 ? g.plane : -g.plane;
 
@@ -213,19 +213,7 @@ __global__ void __launch_bounds__(kTwoThreads, 1)
       if (j >= 2 && warp2) {
         float4 res[NF];
         zs.template level2<P>(l1r, ym2, yp2, t, m, res);
-        if (store) {
-          if (whole) {
-#pragma unroll
-            for (int f = 0; f < NF; ++f) *reinterpret_cast<float4*>(out.f[f] + off) = res[f];
-          } else {
-#pragma unroll
-            for (int f = 0; f < NF; ++f) {
-              out.f[f][off] = res[f].x;
-              if (gx + 1 < x1) out.f[f][off + 1] = res[f].y;
-              if (gx + 2 < x1) out.f[f][off + 2] = res[f].z;
-            }
-          }
-        }
+        if (store) store_group<NF, RAGGED>(out, off, res, gx, x1);
       }
       if (j >= 2) off += off_step;
       if constexpr (MODEL == PF_MODEL_C) zs.lpsi = lpsi_next;

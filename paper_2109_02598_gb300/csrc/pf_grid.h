@@ -73,7 +73,7 @@ constexpr int kTb2Items = 0, kTb2Balanced = 1, kTb2Rows = 2;
 struct StreamTiles {
   int G;      // groups of four columns per row
   int TY;     // output rows per tile
-  int lpad;   // staged columns left of the strip: 0 (full periodic rows) or 4
+  int lpad;   // staged columns left of the strip: 0 (whole periodic rows) or 4
   int S, w;   // strips and output columns per strip (the last may be narrower)
 };
 
