@@ -74,7 +74,7 @@ __device__ __forceinline__ double warp_sum_d(double v) {
 // Bound by the latency of its chain (staging, LEN - 1 forward and LEN reverse stages, each behind
 // a barrier: about 8 us for four steps on a 64^2 grid, 12 at 512^2) and by shared memory on large
 // grids. The reverse pass of 400 steps, against one launch per step with the states recomputed on
-// a second stream: 512^2 2.09 -> 1.20 ms, 128^2 1.27 -> 0.80, 1024^2 4.7 -> 3.4, 2048^2 14.4 ->
+// a second stream: 512^2 2.09 -> 1.15 ms, 128^2 1.27 -> 0.75, 1024^2 4.7 -> 3.4, 2048^2 14.4 ->
 // 12.3. 64 x 32 tiles (less halo, one CTA per SM): the same at 512^2, 20 to 45 % slower on smaller
 // and larger grids.
 template <int LEN>
@@ -119,9 +119,9 @@ __global__ void __launch_bounds__(AdjBlock<LEN>::NT)
     for (int i = tid; i < (TY + 2 * h) * gpr; i += NT) {
       const int r = i / gpr, q = i - r * gpr - hp / 4;
       const int64_t row = (int64_t)wrap_index(y0 - h + r, g.ny) * g.pitch;
-      const int gx = x0 + 4 * q;
+      const int gx = wrap_index(x0 + 4 * q, g.nx);
       float* d = dst + B::at(r - h, q);
-      if (gx >= 0 && gx + 3 < g.nx) {
+      if (gx + 3 < g.nx && gx % 4 == 0) {
         cp_async16(d, in.f[0] + row + gx);
         cp_async16(d + PL, in.f[1] + row + gx);
       } else {
@@ -302,8 +302,8 @@ cudaError_t launch_gs_block(dim3 grid, const FieldPtrs& x, const FieldPtrs& lam,
 //
 // Bound by latency on small grids and by shared memory on large ones, as the Gray-Scott blocks.
 // Reverse pass of 400 steps, against one launch per step with the states recomputed on a second
-// stream: Model A 64^2 1.07 -> 0.61 ms, 512^2 1.42 -> 0.78, 2048^2 7.9 -> 5.8; Model B 64^2
-// 1.28 -> 0.99, 512^2 2.09 -> 1.25, 2048^2 11.4 -> 9.0. 256 threads and four CTAs per SM: with a
+// stream: Model A 64^2 1.07 -> 0.55 ms, 512^2 1.42 -> 0.72, 2048^2 7.9 -> 5.8; Model B 64^2
+// 1.28 -> 0.91, 512^2 2.09 -> 1.16, 2048^2 11.4 -> 8.9. 256 threads and four CTAs per SM: with a
 // thread for every group of the widest region instead (544 and 416) 512^2 takes 0.93 and 1.53,
 // 2048^2 6.2 and 10.1.
 template <int MODEL, int LEN>
@@ -349,8 +349,8 @@ __global__ void __launch_bounds__(kNT2, 4)
   auto stage = [&](const float* in, int h, float* dst) {
     region(h, [&](int p, int r, int q) {
       const float* row = in + (int64_t)wrap_index(y0 + r, g.ny) * g.pitch;
-      const int gx = x0 + 4 * q;
-      if (gx >= 0 && gx + 3 < g.nx) {
+      const int gx = wrap_index(x0 + 4 * q, g.nx);
+      if (gx + 3 < g.nx && gx % 4 == 0) {
         cp_async16(dst + p, row + gx);
       } else {
 #pragma unroll

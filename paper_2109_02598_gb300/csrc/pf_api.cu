@@ -238,8 +238,8 @@ int launch_depth(const pf_grid_s* g, int tile, int k) {
 
 // The tile and depth that run a 2D grid with the standard stencil where nothing was asked for
 // (us a step, against the 128x16 tiles at depth 1 that pf_get_tuning names; the same bits):
-//   up to 3 2^18 sites 32x32 tiles at the model's greatest depth (GS 128^2 0.78/2.38, 512^2
-//     1.06/2.51; AC 512^2 0.76/2.12; Model B 512^2 1.56/2.56; Model C 512^2 1.89/3.01);
+//   up to 3 2^18 sites 32x32 tiles at the model's greatest depth (GS 128^2 0.74/2.38, 512^2
+//     1.05/2.51; AC 512^2 0.72/2.12; Model B 512^2 1.50/2.56; Model C 512^2 1.85/3.01);
 //   above, strips of 128 columns at that depth (2048^2 GS 4.8/11.5, AC 3.3/7.3, Model B 6.0/10.8,
 //     Model C 8.6/15.3; against the 32x32 tiles: 900x640 GS 1.94/1.63, AC 1.49/1.07, Model B
 //     2.80/2.25, Model C 3.48/2.87; 1024x777 1.95/2.22, 1.48/1.40, 2.78/2.88, 3.48/4.08);

@@ -10,8 +10,8 @@
 namespace pf {
 
 // Copy the rows of every field at plane offset zoff into dst (rows ws floats apart, fields pl
-// floats apart): a 16-byte copy where a group of four columns lies inside the row, else four
-// periodic 4-byte copies. Issues the copies and returns: the caller commits or waits.
+// floats apart): a 16-byte copy where a group of four columns, wrapped, is four consecutive ones
+// on a 16-byte boundary, else four periodic 4-byte copies. Issues the copies and returns: the caller commits or waits.
 template <int NF>
 __device__ __forceinline__ void stage_rows4(const FieldPtrs& in, const Geom& g, int x0, int y0,
                                             int64_t zoff, int ws, int ht, int pl, float* dst,
@@ -20,10 +20,10 @@ __device__ __forceinline__ void stage_rows4(const FieldPtrs& in, const Geom& g, 
   for (int i = threadIdx.x; i < ht * ch4; i += nthreads) {
     const int r = i / ch4, j = i - r * ch4;
     const int gy = wrap_index(y0 - 1 + r, g.ny);
-    const int gx = x0 - 4 + 4 * j;
+    const int gx = wrap_index(x0 - 4 + 4 * j, g.nx);
     const int64_t row = zoff + (int64_t)gy * g.pitch;
     float* d = dst + r * ws + 4 * j;
-    if (gx >= 0 && gx + 3 < g.nx) {
+    if (gx + 3 < g.nx && gx % 4 == 0) {
 #pragma unroll
       for (int f = 0; f < NF; ++f) cp_async16(d + f * pl, in.f[f] + row + gx);
     } else {
