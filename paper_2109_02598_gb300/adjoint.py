@@ -2,8 +2,8 @@
 
 ``GrayScottAdjoint`` and ``PhaseFieldAdjoint`` are ``torch.autograd.Function`` wrappers over
 the library's adjoint entry points (``pf_adj_forward`` / ``pf_adj_backward`` in
-include/pfgpu.h): the forward pass advances the initial fields by n steps with sqrt(N)
-checkpointing, the backward pass runs the hand-written adjoint kernels and returns the
+include/pfgpu.h): the forward pass advances the initial fields by n steps with
+checkpoints, the backward pass runs the hand-written adjoint kernels and returns the
 gradient with respect to the initial fields and the model coefficients -- Gray-Scott
 (Du, Dv, F, k), Model A (c1, c2), Model B (c1, c2, mobility M).  Argument marshalling only;
 all arithmetic runs in libpfgpu's kernels.
