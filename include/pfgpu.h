@@ -217,7 +217,8 @@ int pf_set_stencil(pf_grid_t g, int stencil);
 #define PF_TILE_STRIPS (-2) /* tile_y of the strip kernel (with tile_x = 128 or 64) */
 int pf_set_tuning(pf_grid_t g, int tile_x, int tile_y, int k_steps);
 
-/* The tuning in effect (after defaults are resolved). */
+/* The tuning in effect (after defaults are resolved). Where none was asked for, pf_step runs
+ * another kernel in place of the default tile wherever one is faster, with the same bits. */
 int pf_get_tuning(pf_grid_t g, int* tile_x, int* tile_y, int* k_steps);
 
 /* Time every supported (tile, k) for this grid and model (CUDA events), keep the fastest
@@ -225,7 +226,9 @@ int pf_get_tuning(pf_grid_t g, int* tile_x, int* tile_y, int* k_steps);
  * (as pf_step runs them), the cluster and band kernels as one launch of 16 k probe_launches
  * steps. A cluster or band candidate whose CTAs the device cannot host at once (the launch
  * reports it) is skipped.
- * The state is not changed: probe launches read the current buffer and write the spare one.
+ * The state is not changed: probe launches go back and forth between the two buffers, as a run
+ * does, and the state is put back from a copy (without the device memory for one they read the
+ * current buffer and write the spare one).
  * Errors: PF_ERR_STATE (no model), PF_ERR_CUDA. */
 int pf_autotune(pf_grid_t g, int probe_launches, int* tile_x, int* tile_y, int* k_steps);
 
@@ -275,14 +278,14 @@ int pf_batch_read_field(pf_batch_t b, int inst, int field, float* dst, int on_de
  * kernel) and temporal depth k in {1, 2, 4} for every instance; 0 keeps the current value.
  * With the strip kernel each instance's width is split evenly over the fewest strips of 128
  * (or 64) columns that cover it, their output boundaries multiples of 4, and cut into tasks
- * of one height for the whole batch (at least 6 k rows), chosen by playing the task list
+ * of one height for the whole batch (at least 4 rows), chosen by playing the task list
  * through the device's in-order dispatch onto its resident warps. Other tile_x values with
  * PF_TILE_STRIPS return PF_ERR_INVALID_ARG. */
 int pf_batch_set_tuning(pf_batch_t b, int tile_x, int tile_y, int k_steps);
 int pf_batch_get_tuning(pf_batch_t b, int* tile_x, int* tile_y, int* k_steps);
 
-/* Time every (tile, k) on this batch (probe launches read the current state and write the
- * spare copy, so the state is unchanged) and keep the fastest. */
+/* Time every (tile, k) on this batch, as pf_autotune does (the state is unchanged), and keep the
+ * fastest. */
 int pf_batch_autotune(pf_batch_t b, int probe_launches, int* tile_x, int* tile_y,
                       int* k_steps);
 

@@ -83,3 +83,22 @@ def test_untuned_grids_are_bitwise_the_tiles(pf, model, shape):
     x0 = fields(model, shape)
     for a, b in zip(run(pf, model, x0, None, (7,)), run(pf, model, x0, (128, 16, 1), (7,))):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("calls", [(13,), (1, 2, 3, 7), (4, 9)])
+def test_untuned_batch_is_bitwise_depth_one(pf, calls):
+    def batch(tuning):
+        b = pf.Batch([dict(nx=nx, ny=13 + i, Du=0.2, Dv=0.1, F=0.04, k=0.06)
+                      for i, nx in enumerate(WIDTHS)], 0.5)
+        for i, nx in enumerate(WIDTHS):
+            for f, a in enumerate(fields("gs", (13 + i, nx))):
+                b.write(i, f, a)
+        if tuning:
+            b.set_tuning(*tuning)
+        for n in calls:
+            b.run(n)
+        out = [b.read(i, f) for i in range(len(WIDTHS)) for f in (0, 1)]
+        b.close()
+        return out
+
+    assert all(np.array_equal(a, b) for a, b in zip(batch(None), batch((64, 16, 1))))
