@@ -325,7 +325,8 @@ int pf_adj_forward(pf_grid_t g, int64_t n_steps, int64_t ckpt_interval);
  * Recomputes each segment from its checkpoint with the forward kernel (bitwise the same
  * states), then applies lambda^n = lambda^{n+1} + dt J(x^n)^T lambda^{n+1} per step;
  * parameter terms are summed in FP64 in a fixed order. The grid's state is not changed.
- * Synchronizes the stream. Errors: PF_ERR_STATE (no forward pass), PF_ERR_INVALID_ARG,
+ * Synchronizes the stream. Errors: PF_ERR_STATE (no forward pass with the grid's present
+ * model), PF_ERR_INVALID_ARG,
  * PF_ERR_CUDA. */
 int pf_adj_backward(pf_grid_t g, const float* dLdu_N, const float* dLdv_N, int on_device,
                     float* dLdu0, float* dLdv0, double* dtheta);

@@ -705,7 +705,8 @@ int pf_adj_forward(pf_grid_t g, int64_t n_steps, int64_t ckpt_interval) {
   int64_t C = ckpt_interval > 0 ? ckpt_interval : all ? B : root;
   if (C > n_steps) C = n_steps;
   int64_t n_ckpt = (n_steps + C - 1) / C;
-  if (a.n_ckpt != n_ckpt || a.interval != C) {
+  // (seg's size depends on the model's block length, and a grid's model may change)
+  if (a.n_ckpt != n_ckpt || a.interval != C || a.block != B) {
     // (re)allocate for this schedule; a recorded pass or graph of the old one is void
     a.ready = 0;
     if (g->adj_exec) cudaGraphExecDestroy(g->adj_exec);
@@ -727,6 +728,7 @@ int pf_adj_forward(pf_grid_t g, int64_t n_steps, int64_t ckpt_interval) {
     if (C > B) PF_CUDA_TRY(cudaMalloc(&a.seg, state * ((C + B - 1) / B - 1)));
     a.n_ckpt = n_ckpt;
     a.interval = C;
+    a.block = B;
   }
   if (a.lam == nullptr) {  // lambda twice, the gradient slots of every CTA and the four sums
     const dim3 grid = adj_grid(g);
@@ -751,6 +753,7 @@ int pf_adj_forward(pf_grid_t g, int64_t n_steps, int64_t ckpt_interval) {
   for (int i = 0; i < 4; ++i) a.coeffs[i] = g->coeffs[i];
   a.dt = g->dt;
   a.n_steps = n_steps;
+  a.model = g->model;
   a.ready = 1;
   return PF_OK;
 }
@@ -763,6 +766,11 @@ int pf_adj_backward(pf_grid_t g, const float* dLdu_N, const float* dLdv_N, int o
   AdjointState& a = g->adj;
   if (!a.ready) {
     set_error("pf_adj_backward: no recorded forward pass (call pf_adj_forward first)");
+    return PF_ERR_STATE;
+  }
+  if (a.model != g->model) {  // the states, and what is kept of them, are another model's
+    set_error("pf_adj_backward: the recorded forward pass is of another model (call "
+              "pf_adj_forward after pf_set_model)");
     return PF_ERR_STATE;
   }
   if (dLdu_N == nullptr || (g->nf == 2 && dLdv_N == nullptr))
