@@ -200,6 +200,7 @@ constexpr int kReduceBlocks = 512;
 cudaError_t launch_reduce(int what, const Geom& g, const float* field, double c1, double c2,
                           double h, double* d_partials, double* d_out, cudaStream_t s,
                           const int* d_err = nullptr, int* err_out = nullptr);
+cudaError_t reduce_load_kernels();  // every kernel launch_reduce can choose, on the current device
 // Model C free energy of (psi, m) with coefficients c[0..4] = c1..c5.
 cudaError_t launch_reduce_energy_c(const Geom& g, const float* psi, const float* m,
                                    const double* c, double h, double* d_partials,

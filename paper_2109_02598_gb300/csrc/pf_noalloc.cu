@@ -4,8 +4,9 @@
 // Some callers cannot call cudaMalloc: a host framework that has already reserved all of
 // the device's memory for its own allocator (so any allocation from this library would
 // fail or fragment its pool), or a latency-critical loop where cudaMalloc's implicit
-// device-wide synchronisation is not acceptable.  This entry point runs the same two
-// reduction kernels as pf_reduce, on a field the caller owns, writing the result to a
+// device-wide synchronisation is not acceptable.  This entry point runs the same
+// reduction kernels as pf_reduce (chosen by the quantity, the number of sites and the field's
+// alignment), on a field the caller owns, writing the result to a
 // device double the caller owns; the only other memory it touches is a fixed scratch
 // array of kReduceBlocks (512) FP64 partial sums (4 KiB) defined below, which exists on
 // every GPU that loads the library until the process exits.
@@ -14,13 +15,15 @@
 // for the symbol; its device address is fetched once per device with
 // cudaGetSymbolAddress (with that device current) on the first call made on that device,
 // and cached.  Make that first call before any stream capture.  Under CUDA's lazy module
-// loading (the default) that first call is also where the library's modules are loaded on
-// the device, which allocates device memory for their code and for this array and may
-// synchronise; a warm-up call before the caller's allocator takes the device avoids that.
+// loading (the default) that first call is also where this array and every kernel that any
+// later call can choose are loaded on the device, which allocates device memory for them and
+// may synchronise; a warm-up call before the caller's allocator takes the device, on a field
+// of any size and alignment, avoids that.
 // The cached address belongs to the device's primary context: after cudaDeviceReset it no
 // longer exists, so this entry point must not be called again in that process.
 //
-// Every call on a device shares the one array.  Each call writes all 512 partials before
+// Every call on a device shares the one array.  Each call writes the partials it reads (one
+// per block of its first kernel, at most 512; none where one block does all) before
 // reading any of them, so no stale contents from the previous call are used and nothing
 // needs clearing; but two calls whose kernels overlap on the GPU (e.g. on two streams
 // without ordering) race on the array and may return wrong sums.
@@ -51,6 +54,8 @@ int scratch_for_current_device(double** out) {
     void* p = nullptr;
     e = cudaGetSymbolAddress(&p, g_noalloc_partials);
     if (e != cudaSuccess) return pf::cuda_fail(e, "cudaGetSymbolAddress(g_noalloc_partials)");
+    e = pf::reduce_load_kernels();
+    if (e != cudaSuccess) return pf::cuda_fail(e, "loading the reduction kernels");
     g_scratch[dev] = static_cast<double*>(p);
   }
   *out = g_scratch[dev];

@@ -477,6 +477,24 @@ cudaError_t launch(const RedArgs& a, const Geom& g, cudaStream_t s) {
 
 }  // namespace
 
+// Loads every kernel launch_reduce can choose (under lazy loading a kernel's first launch loads
+// it, which may allocate and synchronise, and is not allowed while a stream is captured).
+cudaError_t reduce_load_kernels() {
+  const void* kernels[] = {reinterpret_cast<const void*>(reduce_kernel<kMass, true, false>),
+                           reinterpret_cast<const void*>(reduce_kernel<kMass, false, false>),
+                           reinterpret_cast<const void*>(reduce_kernel<kEnergy, true, false>),
+                           reinterpret_cast<const void*>(reduce_kernel<kEnergy, false, false>),
+                           reinterpret_cast<const void*>(reduce_kernel<kEnergy, true, true>),
+                           reinterpret_cast<const void*>(reduce_kernel<kEnergy, false, true>),
+                           reinterpret_cast<const void*>(reduce_final_kernel)};
+  for (const void* k : kernels) {
+    cudaFuncAttributes a;
+    const cudaError_t e = cudaFuncGetAttributes(&a, k);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 cudaError_t launch_reduce(int what, const Geom& g, const float* field, double c1, double c2,
                           double h, double* d_partials, double* d_out, cudaStream_t s,
                           const int* d_err, int* err_out) {
