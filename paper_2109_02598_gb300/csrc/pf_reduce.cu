@@ -7,9 +7,10 @@
 // Arithmetic. This GPU's FP64 pipe does two operations per clock and SM against 128 in FP32,
 // so an FP64 sum of an FP32 field is bound by it (two operations and conversions per site for
 // the mass, twenty for the 3D energy). The sums run in FP32 without its rounding instead:
-//   * differences, squares and fourth powers as unevaluated pairs hi + lo (the error-free
-//     sum and product of Knuth and Dekker; fma for the product's error), good to 2^-47 a site
-//     without a bias, so 2^-55 of the sum of 2^16 sites (smaller grids: FP64 throughout);
+//   * differences, squares and fourth powers as unevaluated sums of three words (the error-free
+//     sum and product of Knuth and Dekker; fma for the product's error), good to 2^-70 a site,
+//     below FP64's 2^-53 site by site (with the third word left out, 2^-47: not made up for
+//     where an energy lies in a few sites of a flat field);
 //   * added into three-word accumulators by cascaded error-free sums, whose error, about
 //     2^-72 of the sum, is below FP64's;
 //   * on packed pairs of sites (add.rn.f32x2 and so on), one thread's words becoming one
@@ -26,8 +27,9 @@
 //
 // Bound by issue (energies) and by latency at the CTAs' registers. A call with its
 // synchronisation, before (FP64 sums; 64 of 256 threads busy on 256-wide rows; the result and
-// the error word by two copies) -> now: mass 256^3 115 -> 37 us, 2048^2 43 -> 28, 128^2 29 -> 18;
-// energy 256^3 659 -> 105 us, 2048^2 155 -> 37, 128^2 29 -> 20; Model C 128^3 361 -> 48. Errors
+// the error word by two copies) -> now: mass 256^3 115 -> 35 us, 2048^2 43 -> 27, 128^2 29 -> 17;
+// energy 256^3 659 -> 119 us, 2048^2 155 -> 38, 128^2 29 -> 18; Model C 128^3 361 -> 50 (the third
+// words of squares and products are 10 to 16 % of these: 103, 34 and 46 without). Errors
 // against 128-bit sums over 20 shapes and seven kinds of values (noise, smooth, 1e-9 to 3e6,
 // mixed magnitudes) stay those of the FP64 sums: 4e-18 to 2e-17 on average for the mass, 5e-17
 // to 1.4e-16 for the energies.
@@ -43,8 +45,9 @@ constexpr int kNTR = 256;        // threads of a CTA of the two-kernel form
 constexpr int kOneCta = 512;     // threads of the one-CTA form
 constexpr int kNTS = 64;         // threads of a CTA of the FP64 form
 
-// Energies of fewer sites are summed in FP64: at 2^16 sites the pairs' error per site, averaged
-// over them, has fallen to 2^-55 of the sum.
+// Energies of fewer sites are summed in FP64: many small CTAs of short FP64 work finish before the
+// few that the words' sums would fill (a call on 128^2: 18 us against 29, Model C 21 against 49;
+// from 40^3 on the times are the same).
 constexpr int64_t kFp64Sites = 1 << 16;
 
 constexpr int kMass = 0, kEnergy = 1, kEnergyC = 2;
@@ -105,17 +108,30 @@ __device__ __forceinline__ float2 two_sum(float2 a, float2 b, float2& e) {
   e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
   return s;
 }
-// h + l = a^2 exactly; for a pair (ah, al), h + l = ah^2 + 2 ah al to 2^-48. The rest, al^2, is
-// always positive and mostly under half of l's last place: added to l it would be lost every
-// time (a bias of -1e-15 of the sum, measured), so callers add it to an accumulator's last word.
-__device__ __forceinline__ float2 square2(float2 a, float2& l) {
-  const float2 h = __fmul2_rn(a, a);
-  l = __ffma2_rn(a, a, neg2(h));
+// h + l = a b exactly.
+__device__ __forceinline__ float2 product2(float2 a, float2 b, float2& l) {
+  const float2 h = __fmul2_rn(a, b);
+  l = __ffma2_rn(a, b, neg2(h));
   return h;
 }
-__device__ __forceinline__ float2 square2(float2 ah, float2 al, float2& l) {
+__device__ __forceinline__ float2 square2(float2 a, float2& l) { return product2(a, a, l); }
+// h + l + r = (ah + al) b to 2^-72 for a pair (ah, al): al b meets the rounding of ah b in l, and
+// what both leave goes to r, which callers add to an accumulator's last word.
+__device__ __forceinline__ float2 product2(float2 ah, float2 al, float2 b, float2& l, float2& r) {
+  float2 e, pe;
+  const float2 h = product2(ah, b, l);
+  const float2 p = product2(al, b, pe);
+  l = two_sum(l, p, e);
+  r = add2(e, pe);
+  return h;
+}
+// h + l + r = (ah + al)^2 to 2^-72.
+__device__ __forceinline__ float2 square2(float2 ah, float2 al, float2& l, float2& r) {
+  float2 e, pe;
   const float2 h = square2(ah, l);
-  l = __ffma2_rn(add2(ah, ah), al, l);
+  const float2 p = product2(add2(ah, ah), al, pe);
+  l = two_sum(l, p, e);
+  r = __ffma2_rn(al, al, add2(e, pe));
   return h;
 }
 
@@ -139,7 +155,6 @@ struct Sum3 {  // a0 + a1 + a2, one sum per half of the pair
     add(h, l);
     a2 = add2(a2, l2);
   }
-  __device__ __forceinline__ void add_square(float2 x) { a2 = __ffma2_rn(x, x, a2); }
   __device__ __forceinline__ double value() const {
     return (((double)a2.x + (double)a2.y) + ((double)a1.x + (double)a1.y)) +
            ((double)a0.x + (double)a0.y);
@@ -218,8 +233,7 @@ __device__ __forceinline__ float rows_max(const Rows<R>& c) {
   return m;
 }
 
-// |grad|^2 h^2 of two sites (columns 2 q, 2 q + 1 of row r) as hi + lo + lo2 (lo's roundings are
-// kept too: field values on a lattice of floats round it one way more often than the other), from the differences
+// |grad|^2 h^2 of two sites (columns 2 q, 2 q + 1 of row r) as hi + lo + lo2, from the differences
 // to the right, the next row and (3D) the next plane
 template <int R>
 __device__ __forceinline__ float2 grad2(const Rows<R>& c, int r, int q, bool three, float2& lo,
@@ -228,16 +242,15 @@ __device__ __forceinline__ float2 grad2(const Rows<R>& c, int r, int q, bool thr
   const float2 p = q == 0 ? make_float2(v.x, v.y) : make_float2(v.z, v.w);
   const float2 px = q == 0 ? make_float2(v.y, v.z) : make_float2(v.w, c.after[r]);
   const float2 py = q == 0 ? make_float2(y.x, y.y) : make_float2(y.z, y.w);
-  float2 dl, l, e, r1, r2;
+  float2 dl, l, l2, e, r1, r2;
   float2 d = two_sum(px, neg2(p), dl);
-  float2 s = square2(d, dl, lo);
-  lo2 = __fmul2_rn(dl, dl);
+  float2 s = square2(d, dl, lo, lo2);
   auto more = [&](const float2& pn) {
     d = two_sum(pn, neg2(p), dl);
-    s = two_sum(s, square2(d, dl, l), e);
+    s = two_sum(s, square2(d, dl, l, l2), e);
     lo = two_sum(lo, l, r1);
     lo = two_sum(lo, e, r2);
-    lo2 = __ffma2_rn(dl, dl, add2(lo2, add2(r1, r2)));
+    lo2 = add2(add2(lo2, l2), add2(r1, r2));
   };
   more(py);
   if (three) more(q == 0 ? make_float2(z.x, z.y) : make_float2(z.z, z.w));
@@ -327,7 +340,7 @@ __global__ void __launch_bounds__(FP64 ? kNTS : kOneCta) reduce_kernel(const Red
           if (r >= nr) break;
 #pragma unroll
           for (int i = 0; i < 2; ++i) {
-            float2 lo, lo2, l2, l4;
+            float2 lo, lo2, l2, l4, r4;
             float2 hi = grad2(p, r, i, three, lo, lo2);
             float2 pv = i == 0 ? make_float2(p.v[r].x, p.v[r].y) : make_float2(p.v[r].z, p.v[r].w);
             if (n < 4) {
@@ -339,9 +352,8 @@ __global__ void __launch_bounds__(FP64 ? kNTS : kOneCta) reduce_kernel(const Red
             sg.add(hi, lo, lo2);
             const float2 p2 = square2(pv, l2);
             s2.add(p2, l2);
-            const float2 p4 = square2(p2, l2, l4);
-            s4.add(p4, l4);
-            s4.add_square(l2);
+            const float2 p4 = square2(p2, l2, l4, r4);
+            s4.add(p4, l4, r4);
             if constexpr (WHAT == kEnergyC) {
               hi = grad2(q, r, i, three, lo, lo2);
               float2 qv = i == 0 ? make_float2(q.v[r].x, q.v[r].y) : make_float2(q.v[r].z, q.v[r].w);
@@ -355,13 +367,11 @@ __global__ void __launch_bounds__(FP64 ? kNTS : kOneCta) reduce_kernel(const Red
               float2 m2, m4;
               const float2 q2 = square2(qv, m2);
               t2.add(q2, m2);
-              const float2 q4 = square2(q2, m2, m4);
-              t4.add(q4, m4);
-              t4.add_square(m2);
-              // psi^2 m = (p2 + l2) q: the product's error, and l2 q
-              const float2 x2 = __fmul2_rn(p2, qv);
-              const float2 xl = __ffma2_rn(l2, qv, __ffma2_rn(p2, qv, neg2(x2)));
-              sx.add(x2, xl);
+              const float2 q4 = square2(q2, m2, m4, r4);
+              t4.add(q4, m4, r4);
+              float2 xl;  // psi^2 m
+              const float2 x2 = product2(p2, l2, qv, xl, r4);
+              sx.add(x2, xl, r4);
             }
           }
         }
