@@ -307,8 +307,9 @@ int pf_batch_info(pf_batch_t b, int64_t* sites, int64_t* bytes_per_copy);
  * state (2D grid; Gray-Scott, Allen-Cahn or Cahn-Hilliard model) by n_steps forward-Euler
  * steps exactly like
  * pf_step, storing the state every ckpt_interval steps. 0 leaves the interval C to the library:
- * where they fit 4 GiB of device memory the states the reverse pass starts its launches from
- * (every 4th, for Model B every 2nd), else C = ceil(sqrt(n_steps)), i.e.
+ * the states the reverse pass starts its launches from (every 4th, for Model B every 2nd) where
+ * they fit, with those the device's other grids store this way, 4 GiB, and a sixteenth of the
+ * memory that is free; else C = ceil(sqrt(n_steps)), i.e.
  * sqrt(N) checkpointing of the time loop of Sec. 2.4.1. The gradients do not depend on C.
  * Allocates the checkpoints (ceil(N/C) states), a segment's states between them and the adjoint
  * buffers on first use.

@@ -25,6 +25,7 @@
 // fit, else the segment's are recomputed from its checkpoint with the forward kernel
 // (C ~ sqrt(N)). Parameter-gradient partials are summed per CTA in FP64 (each CTA owns one slot,
 // so the order is fixed and the result deterministic) and added up in a fixed order at the end.
+#include <atomic>
 #include <cmath>
 
 #include "pf_fe2d_tile.cuh"
@@ -35,8 +36,12 @@ namespace pf {
 
 namespace {
 
-// Bytes of stored states up to which the forward pass keeps every block's first one.
-constexpr double kAllStates = 4.0 * (1 << 30);
+// The forward pass keeps every block's first state where they fit, with those that the device's
+// other handles keep this way, kAllStates bytes, and one part in kFreeParts of the memory that is
+// free: a program may hold many handles (an autograd node is one each), and its other allocations
+// do not wait for ours.
+constexpr int64_t kAllStates = (int64_t)4 << 30;
+constexpr int kFreeParts = 16;
 
 constexpr int kATX = 64, kATY = 16;  // adjoint tile
 
@@ -580,8 +585,39 @@ int check_gs2d(pf_grid_s* g) {
 
 }  // namespace
 
+// Bytes that the live handles of a device hold in states stored by the library's choice.
+static std::atomic<int64_t> g_stored[64];
+
+// Count `need` bytes of this handle's checkpoints (in place of what it held) against the limits
+// above; false, and nothing changed, where they do not fit.
+static bool hold_states(pf_grid_s* g, double need) {
+  AdjointState& a = g->adj;
+  if (g->device < 0 || g->device >= 64 || need > (double)kAllStates) return false;
+  size_t free_bytes = 0, total = 0;
+  if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  const int64_t want = (int64_t)need;
+  if (want > ((int64_t)free_bytes + a.held) / kFreeParts) return false;
+  std::atomic<int64_t>& sum = g_stored[g->device];
+  int64_t now = sum.load();
+  do {
+    if (now - a.held + want > kAllStates) return false;
+  } while (!sum.compare_exchange_weak(now, now - a.held + want));
+  a.held = want;
+  return true;
+}
+
+static void drop_states(pf_grid_s* g) {
+  AdjointState& a = g->adj;
+  if (a.held > 0) g_stored[g->device] -= a.held;
+  a.held = 0;
+}
+
 void adjoint_release(pf_grid_s* g) {
   AdjointState& a = g->adj;
+  drop_states(g);
   if (a.ckpt) cudaFree(a.ckpt);
   if (a.seg) cudaFree(a.seg);
   if (a.lam) cudaFree(a.lam);
@@ -698,10 +734,21 @@ int pf_adj_forward(pf_grid_t g, int64_t n_steps, int64_t ckpt_interval) {
   AdjointState& a = g->adj;
   const size_t state = sizeof(float) * g->nf * g->field_elems;
   const int B = block_len(g->model);
-  // The library's choice: every block's first state where they fit kAllStates bytes (nothing to
+  if (a.lam == nullptr) {  // lambda twice, the gradient slots of every CTA and the four sums
+    const dim3 grid = adj_grid(g);
+    const int64_t nctas = (int64_t)grid.x * grid.y;
+    const size_t lam = (2 * state + 255) / 256 * 256;
+    PF_CUDA_TRY(cudaMalloc(&a.lam, lam + sizeof(double) * (4 * nctas + 4)));
+    PF_CUDA_TRY(cudaMemsetAsync(a.lam, 0, 2 * state, g->stream));
+    a.gpart = reinterpret_cast<double*>(reinterpret_cast<char*>(a.lam) + lam);
+    a.gout = a.gpart + 4 * nctas;
+  }
+  // The library's choice: every block's first state where they fit (hold_states; nothing to
   // recompute between blocks then), else sqrt(N) checkpoints.
   const int64_t root = (int64_t)std::ceil(std::sqrt((double)n_steps));
-  const bool all = (double)((n_steps + B - 1) / B) * (double)state <= kAllStates;
+  const bool all = ckpt_interval == 0 &&
+                   hold_states(g, (double)((n_steps + B - 1) / B) * (double)state);
+  if (!all) drop_states(g);
   int64_t C = ckpt_interval > 0 ? ckpt_interval : all ? B : root;
   if (C > n_steps) C = n_steps;
   int64_t n_ckpt = (n_steps + C - 1) / C;
@@ -720,6 +767,7 @@ int pf_adj_forward(pf_grid_t g, int64_t n_steps, int64_t ckpt_interval) {
     cudaError_t e = cudaMalloc(&a.ckpt, state * n_ckpt);
     if (e != cudaSuccess && ckpt_interval == 0 && C < root) {
       cudaGetLastError();  // no room for all of them
+      drop_states(g);
       C = root < n_steps ? root : n_steps;
       n_ckpt = (n_steps + C - 1) / C;
       e = cudaMalloc(&a.ckpt, state * n_ckpt);
@@ -729,15 +777,6 @@ int pf_adj_forward(pf_grid_t g, int64_t n_steps, int64_t ckpt_interval) {
     a.n_ckpt = n_ckpt;
     a.interval = C;
     a.block = B;
-  }
-  if (a.lam == nullptr) {  // lambda twice, the gradient slots of every CTA and the four sums
-    const dim3 grid = adj_grid(g);
-    const int64_t nctas = (int64_t)grid.x * grid.y;
-    const size_t lam = (2 * state + 255) / 256 * 256;
-    PF_CUDA_TRY(cudaMalloc(&a.lam, lam + sizeof(double) * (4 * nctas + 4)));
-    PF_CUDA_TRY(cudaMemsetAsync(a.lam, 0, 2 * state, g->stream));
-    a.gpart = reinterpret_cast<double*>(reinterpret_cast<char*>(a.lam) + lam);
-    a.gout = a.gpart + 4 * nctas;
   }
   // (a grid buffer's fields lie one after the other, as a checkpoint's)
   PF_CUDA_TRY(cudaMemcpyAsync(ckpt_field(g, 0, 0), g->buf[g->cur][0], state,
