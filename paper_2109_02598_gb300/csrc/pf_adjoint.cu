@@ -744,12 +744,21 @@ int pf_adj_forward(pf_grid_t g, int64_t n_steps, int64_t ckpt_interval) {
     a.gout = a.gpart + 4 * nctas;
   }
   // The library's choice: every block's first state where they fit (hold_states; nothing to
-  // recompute between blocks then), else sqrt(N) checkpoints.
+  // recompute between blocks then), else sqrt(N) checkpoints. A request that was answered before
+  // keeps its schedule: asked for anew in every pass of a training loop, a refused choice would
+  // have the buffers freed and allocated again each time, and the reverse pass's graph with them.
   const int64_t root = (int64_t)std::ceil(std::sqrt((double)n_steps));
-  const bool all = ckpt_interval == 0 &&
-                   hold_states(g, (double)((n_steps + B - 1) / B) * (double)state);
-  if (!all) drop_states(g);
-  int64_t C = ckpt_interval > 0 ? ckpt_interval : all ? B : root;
+  const bool answered = a.n_ckpt > 0 && a.block == B && a.asked_steps == n_steps &&
+                        a.asked_interval == ckpt_interval;
+  int64_t C = ckpt_interval > 0 ? ckpt_interval : root;
+  if (answered) {
+    C = a.interval;
+  } else if (ckpt_interval == 0 &&
+             hold_states(g, (double)((n_steps + B - 1) / B) * (double)state)) {
+    C = B;
+  } else {
+    drop_states(g);
+  }
   if (C > n_steps) C = n_steps;
   int64_t n_ckpt = (n_steps + C - 1) / C;
   // (seg's size depends on the model's block length, and a grid's model may change)
@@ -778,6 +787,8 @@ int pf_adj_forward(pf_grid_t g, int64_t n_steps, int64_t ckpt_interval) {
     a.interval = C;
     a.block = B;
   }
+  a.asked_steps = n_steps;
+  a.asked_interval = ckpt_interval;
   // (a grid buffer's fields lie one after the other, as a checkpoint's)
   PF_CUDA_TRY(cudaMemcpyAsync(ckpt_field(g, 0, 0), g->buf[g->cur][0], state,
                               cudaMemcpyDeviceToDevice, g->stream));

@@ -92,6 +92,7 @@ struct AdjointState {
   int64_t interval = 0;      // checkpoint interval C
   int64_t n_ckpt = 0;        // checkpoints stored (states 0, C, 2C, ...)
   int block = 0;             // steps per reverse launch that seg was sized for
+  int64_t asked_steps = 0, asked_interval = -1;  // the request that this schedule answers
   int64_t held = 0;          // bytes of ckpt that count against the device's limit (hold_states)
   int model = -1;            // the recorded forward pass's model
   float* ckpt = nullptr;     // n_ckpt * nf * field_elems floats

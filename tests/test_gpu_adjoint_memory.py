@@ -55,3 +55,17 @@ def test_stored_states_are_bounded_over_handles(pf):
     assert forward(pf, c, x) >= 100 * STATE
     b.close()
     c.close()
+
+
+def test_a_repeated_request_keeps_its_schedule(pf):
+    x, lam, (a, b, c) = setup(pf)
+    forward(pf, a, x)
+    assert forward(pf, b, x) <= 30 * STATE
+    a.close()  # there would be room for b's now
+    for _ in range(3):
+        assert forward(pf, b, x) == 0
+        pf.adjoint_backward(b, *lam)
+    assert forward(pf, b, x, STEPS - 100) > 40 * STATE  # another request: chosen anew
+    assert forward(pf, b, x, STEPS - 100) == 0
+    b.close()
+    c.close()
