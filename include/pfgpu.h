@@ -221,6 +221,11 @@ int pf_set_tuning(pf_grid_t g, int tile_x, int tile_y, int k_steps);
  * another kernel in place of the default tile wherever one is faster, with the same bits. */
 int pf_get_tuning(pf_grid_t g, int* tile_x, int* tile_y, int* k_steps);
 
+/* *untuned = 1 where no tuning is asked for (pf_step chooses its kernels), else 0. To keep a grid's
+ * tuning for later, store (0, 0, 0) for an untuned one: set explicitly, the default that
+ * pf_get_tuning names would run as such. */
+int pf_is_untuned(pf_grid_t g, int* untuned);
+
 /* Time every supported (tile, k) for this grid and model (CUDA events), keep the fastest
  * and report it: tiled kernels as a replayed CUDA graph of max(probe_launches, 8) launches
  * (as pf_step runs them), the cluster and band kernels as one launch of 16 k probe_launches

@@ -73,6 +73,7 @@ SIGNATURES = {
     "pf_set_stencil": (ctypes.c_int, [_vp, ctypes.c_int]),
     "pf_set_tuning": (ctypes.c_int, [_vp, ctypes.c_int, ctypes.c_int, ctypes.c_int]),
     "pf_get_tuning": (ctypes.c_int, [_vp, _c_int_p, _c_int_p, _c_int_p]),
+    "pf_is_untuned": (ctypes.c_int, [_vp, _c_int_p]),
     "pf_autotune": (ctypes.c_int, [_vp, ctypes.c_int, _c_int_p, _c_int_p, _c_int_p]),
     "pf_synchronize": (ctypes.c_int, [_vp]),
     "pf_field_view": (ctypes.c_int, [_vp, ctypes.c_int, ctypes.POINTER(_vp), _c_int64_p,

@@ -844,6 +844,13 @@ int pf_get_tuning(pf_grid_t g, int* tile_x, int* tile_y, int* k_steps) {
   return PF_OK;
 }
 
+int pf_is_untuned(pf_grid_t g, int* untuned) {
+  if (int rc = check_grid(g)) return rc;
+  if (untuned == nullptr) return invalid("untuned is NULL");
+  *untuned = g->req_tile < 0 && g->req_k == 0;
+  return PF_OK;
+}
+
 int pf_autotune(pf_grid_t g, int probe_launches, int* tile_x, int* tile_y, int* k_steps) {
   NvtxRange nvtx_("pf_autotune");
   if (int rc = check_grid(g)) return rc;

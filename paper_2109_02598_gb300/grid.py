@@ -238,11 +238,15 @@ class Grid:
     # ---------------------------------------------------------------- checkpoints
     def save(self, path: str, extra: dict | None = None):
         """Write a checkpoint: the fields and what is needed to continue the run (model,
-        coefficients, dt, h, stencil, tuning, steps taken). `extra`: JSON-serialisable
+        coefficients, dt, h, stencil, tuning, steps taken; an untuned grid's tuning is (0, 0, 0),
+        which leaves the restored one untuned). `extra`: JSON-serialisable
         values stored alongside."""
+        untuned = ctypes.c_int()
+        check(self._lib.pf_is_untuned(self._h, ctypes.byref(untuned)))
         meta = {"shape": list(self.shape), "h": self.h, "model": self.model,
                 "coeffs": list(self.coeffs) if self.coeffs is not None else None,
-                "dt": self.dt, "stencil": self.stencil, "tuning": list(self.tuning),
+                "dt": self.dt, "stencil": self.stencil,
+                "tuning": [0, 0, 0] if untuned.value else list(self.tuning),
                 "steps": self.steps_done, "extra": extra or {}}
         checkpoint.save_state(path, meta, self.read_fields())
         return self
