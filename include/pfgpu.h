@@ -288,6 +288,7 @@ int pf_batch_read_field(pf_batch_t b, int inst, int field, float* dst, int on_de
  * PF_TILE_STRIPS return PF_ERR_INVALID_ARG. */
 int pf_batch_set_tuning(pf_batch_t b, int tile_x, int tile_y, int k_steps);
 int pf_batch_get_tuning(pf_batch_t b, int* tile_x, int* tile_y, int* k_steps);
+int pf_batch_is_untuned(pf_batch_t b, int* untuned); /* as pf_is_untuned */
 
 /* Time every (tile, k) on this batch, as pf_autotune does (the state is unchanged), and keep the
  * fastest. */

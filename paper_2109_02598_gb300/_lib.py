@@ -85,6 +85,7 @@ SIGNATURES = {
     "pf_batch_read_field": (ctypes.c_int, [_vp, ctypes.c_int, ctypes.c_int, _vp, ctypes.c_int]),
     "pf_batch_set_tuning": (ctypes.c_int, [_vp, ctypes.c_int, ctypes.c_int, ctypes.c_int]),
     "pf_batch_get_tuning": (ctypes.c_int, [_vp, _c_int_p, _c_int_p, _c_int_p]),
+    "pf_batch_is_untuned": (ctypes.c_int, [_vp, _c_int_p]),
     "pf_batch_autotune": (ctypes.c_int, [_vp, ctypes.c_int, _c_int_p, _c_int_p, _c_int_p]),
     "pf_batch_run": (ctypes.c_int, [_vp, ctypes.c_int64]),
     "pf_batch_synchronize": (ctypes.c_int, [_vp]),

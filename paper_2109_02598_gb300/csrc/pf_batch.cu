@@ -362,7 +362,8 @@ int pf_batch_set_tuning(pf_batch_t b, int tile_x, int tile_y, int k_steps) {
   if (!fe2d_supported(PF_MODEL_GS, k)) return invalid("unsupported temporal depth %d", k);
   b->tile = t;
   b->k = k;
-  b->tuned = true;
+  // (all zero keeps what there is, and an untuned batch untuned)
+  b->tuned = b->tuned || tile_x != 0 || tile_y != 0 || k_steps != 0;
   return PF_OK;
 }
 
@@ -373,6 +374,13 @@ int pf_batch_get_tuning(pf_batch_t b, int* tile_x, int* tile_y, int* k_steps) {
   if (tile_x) *tile_x = tx;
   if (tile_y) *tile_y = ty;
   if (k_steps) *k_steps = b->k;
+  return PF_OK;
+}
+
+int pf_batch_is_untuned(pf_batch_t b, int* untuned) {
+  if (int rc = check_batch(b)) return rc;
+  if (untuned == nullptr) return invalid("untuned is NULL");
+  *untuned = !b->tuned;
   return PF_OK;
 }
 

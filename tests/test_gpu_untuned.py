@@ -1,6 +1,8 @@
 """A grid or batch without a tuning of the caller's stays so: through a checkpoint, where a restored run
 is to take the kernels (and bits) of the one it resumes, and through a call that keeps the present
 values."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -23,9 +25,9 @@ def pf():
 
 
 def untuned(g):
-    import ctypes
     v = ctypes.c_int(-1)
-    assert g._lib.pf_is_untuned(g.handle, ctypes.byref(v)) == 0
+    ask = g._lib.pf_batch_is_untuned if hasattr(g, "shapes") else g._lib.pf_is_untuned
+    assert ask(g._h, ctypes.byref(v)) == 0
     return bool(v.value)
 
 
@@ -58,3 +60,30 @@ def test_checkpoints_keep_a_grid_untuned(pf, tmp_path, model, shape, tuning):
     assert untuned(h)
     h.close()
     g.close()
+
+
+def test_batch_keeps_its_values(pf):
+    rng = np.random.default_rng(6)
+    shapes = [(40, 52), (33, 70)]
+    x = [[(0.2 + 0.3 * rng.random(s)).astype(np.float32) for _ in range(2)] for s in shapes]
+
+    def run(b):
+        for i in range(2):
+            for f in range(2):
+                b.write(i, f, x[i][f])
+        b.run(11)
+        return [b.read(i, f) for i in range(2) for f in range(2)]
+
+    specs = [dict(nx=s[1], ny=s[0], Du=0.2, Dv=0.1, F=0.04, k=0.06) for s in shapes]
+    b = pf.Batch(specs, 0.5)
+    assert untuned(b)
+    want, named = run(b), b.tuning
+    b.set_tuning(0, 0, 0)
+    assert untuned(b) and b.tuning == named
+    assert all(np.array_equal(p, q) for p, q in zip(want, run(b)))
+    b.set_tuning(*named)  # asked for: runs what it names
+    assert not untuned(b)
+    b.set_tuning(0, 0, 0)
+    assert not untuned(b) and b.tuning == named
+    assert all(np.array_equal(p, q) for p, q in zip(want, run(b)))
+    b.close()
