@@ -711,7 +711,7 @@ static int forward_segments(pf_grid_s* g, int64_t n_steps, int64_t C, int64_t n_
       if (!to_ckpt) last = 1 - last;
       for (int f = 0; f < g->nf; ++f)
         out.f[f] = to_ckpt ? ckpt_field(g, s + 1, f) : g->buf[last][f];
-      PF_CUDA_TRY(launch_2d(g, tile, k, in, out, g->params, g->stream));
+      PF_CUDA_TRY(launch_2d(g, plan_tile(g, tile, k), k, in, out, g->params, g->stream));
       for (int f = 0; f < g->nf; ++f) in.f[f] = out.f[f];
     }
   }

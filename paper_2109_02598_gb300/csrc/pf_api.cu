@@ -245,27 +245,61 @@ int launch_depth(const pf_grid_s* g, int tile, int k) {
 //     2.80/2.25, Model C 3.48/2.87; 1024x777 1.95/2.22, 1.48/1.40, 2.78/2.88, 3.48/4.08);
 //   Model C above 3 2^21 sites, strips of 64 (of 128, twelve warps fit an SM, too few once the
 //     fields leave the L2 cache: 2500^2 14.8 us with either, 3000^2 18.9 against 21.9).
+// The sites are those of whole tile rows: a grid of few rows pays 32 of them in the tiles, and only
+// its own in strips (4 x 65536, tiles, strips and 128x16: GS 2.2/1.3/3.2, AC 2.0/1.1/2.7, Model B
+// 4.4/1.9/3.6, Model C 5.0/2.2/3.9; 1 x 262144 6.5/1.6/7.3, 6.2/1.2/5.7, 13.8/2.2/8.3, 16.6/3.5/9.2).
 void plan2d(const pf_grid_s* g, int* tile, int* depth) {
   const bool r1 = g->model == PF_MODEL_AC || g->model == PF_MODEL_GS;
-  const int64_t n = (int64_t)g->nx * g->ny;
+  const int64_t n = (int64_t)g->nx * g->ny, whole = (int64_t)g->nx * ((g->ny + 31) / 32 * 32);
   const bool narrow = g->model == PF_MODEL_C && n > (int64_t)3 << 21;
-  *tile = n > (int64_t)3 << 18 ? kTileStrips2D + (narrow ? 1 : 0) : 2;
+  *tile = whole > (int64_t)3 << 18 ? kTileStrips2D + (narrow ? 1 : 0) : 2;
   *depth = r1 ? 4 : 2;
+}
+
+static bool runs_untuned(const pf_grid_s* g) {
+  return g->stencil == PF_ST_STD && g->model != PF_MODEL_RD && g->req_tile < 0 && g->req_k == 0;
 }
 
 // The tile and depth pf_step runs: the tuning in effect, except where it is the library's own
 // choice (nothing asked for) and the stencil the standard one. Then a kernel that passes the one
 // pf_get_tuning names takes its place, with the same bits: plan2d's, and in 3D the general tile's
 // for the depth-1 TMA tiles (256^3 GS 585 against 369 GLUPS, AC 1015/716, Model B 536/393, Model C
-// 328/165; 64^3 GS 130/60, Model B 87/38).
+// 328/165; 64^3 GS 130/60, Model B 87/38; rows of 320 to 1024 columns 1.2 to 1.5 times the TMA
+// tiles' rate, Model C 768 x 256 x 128 twice). Not for a few large planes: the general kernel streams
+// four more of them, from memory where a plane is large (us a step, 1024^2 in 1, 2, 4 planes: AC
+// 6.5/5.0, 7.5/6.5, 9.7/9.4, GS 9.8/8.1, 11.9/11.4, 16.1/17.5, Model B 12.5/11.5, 14.3/14.1,
+// 18.6/19.9; 2048^2 in 2, 5, 8: AC 26/19, 44/35, 57/49, GS 45/38, 71/70, 96/99, Model B 51/46, 85/77,
+// 110/108; but 768 x 512 in one 3.2/3.4, 4.4/4.7, 5.9/6.4; Model C is faster on the general tile
+// throughout).
 void run_plan(const pf_grid_s* g, int* tile, int* depth) {
-  const bool untuned = g->stencil == PF_ST_STD && g->model != PF_MODEL_RD && g->req_tile < 0 &&
-                       g->req_k == 0;
+  const bool untuned = runs_untuned(g);
+  const int64_t plane = (int64_t)g->nx * g->ny;
+  const int few = g->model == PF_MODEL_AC ? 4 : 2;  // planes of 2^20 sites, more of larger ones
+  const bool planes = g->model != PF_MODEL_C && plane > 1 << 19 &&
+                      (g->nz <= few || ((int64_t)g->nz << 20) <= few * plane);
   *tile = g->tile;
   int k = g->k;
-  if (untuned && g->dim == 3) *tile = 0;
+  if (untuned && g->dim == 3 && !planes) *tile = 0;
   if (untuned && g->dim == 2) plan2d(g, tile, &k);
   *depth = launch_depth(g, *tile, k);
+}
+
+// A plan's single steps (a call of one step, or what is left over from its depth) of an untuned grid:
+// in 2D on strips, Allen-Cahn and Gray-Scott beyond 96 MB of old and new state, which no longer
+// meet in the L2 cache, on the named tiles (128x16 against strips: GS 2500^2 18.4/18.5 us, 2900^2
+// 24.8/27.3, 4096^2 46.9/52.4; AC 3300^2 18.5/17.5, 3700^2 21.2/25.2, 4096^2 26.5/32.6; Model B's
+// strips stay ahead, 4096^2 36.9/33.4), and Model C on strips of 128 columns (4096^2 53.3, of 64
+// 63.9, tiles 55.4); in 3D, Allen-Cahn and Gray-Scott of more than 2^24 sites (rows of more than 256
+// columns: 3 2^22) on the named tiles (TMA tiles against the one-level kernel: GS 384^3 144/178,
+// 768 x 256 x 128 68/79, 256^2 x 512 88/92, but 256^3 48/46 and 512 x 128^2 29/24; AC 384^3 78/89).
+int plan_tile(const pf_grid_s* g, int tile, int k) {
+  if (k != 1 || !runs_untuned(g)) return tile;
+  const bool r1 = g->model == PF_MODEL_AC || g->model == PF_MODEL_GS;
+  const int64_t n = (int64_t)g->nx * g->ny * g->nz;
+  if (g->dim == 3) return r1 && n > (g->nx <= 256 ? 1 << 24 : 3 << 22) ? g->tile : tile;
+  if (tile < kTileStrips2D) return tile;
+  if (g->model == PF_MODEL_C) return kTileStrips2D;
+  return r1 && 8 * g->nf * n > (int64_t)96 << 20 ? g->tile : tile;
 }
 
 int sync_device_error(pf_grid_s* g);
@@ -365,7 +399,7 @@ static int record_step_graph(pf_grid_s* g, int tile, int depth, int64_t n,
   while (left > 0 && e == cudaSuccess) {
     int k = depth;
     while (k > left) k >>= 1;
-    e = launch_step(g, tile, k, src, 1 - src, g->capture);
+    e = launch_step(g, plan_tile(g, tile, k), k, src, 1 - src, g->capture);
     src = 1 - src;
     left -= k;
     ++launches;
@@ -669,7 +703,7 @@ int pf_step(pf_grid_t g, int64_t n_steps) {
   while (left > 0) {
     int k = depth;
     while (k > left) k >>= 1;  // k in {4, 2, 1}
-    PF_CUDA_TRY(launch_step(g, tile, k, g->cur, 1 - g->cur, g->stream));
+    PF_CUDA_TRY(launch_step(g, plan_tile(g, tile, k), k, g->cur, 1 - g->cur, g->stream));
     g->cur = 1 - g->cur;
     left -= k;
   }

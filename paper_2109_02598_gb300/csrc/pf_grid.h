@@ -184,6 +184,8 @@ cudaError_t launch_2d(const pf_grid_s* g, int tile, int k, const FieldPtrs& in,
 // The tile and depth of an untuned 2D grid with the standard stencil, and those pf_step runs
 void plan2d(const pf_grid_s* g, int* tile, int* depth);
 void run_plan(const pf_grid_s* g, int* tile, int* depth);
+// The tile of a launch of k steps of that plan
+int plan_tile(const pf_grid_s* g, int tile, int k);
 
 // ---- 3D TMA kernels (AC, GS; Models B and C in pf_fe3d_tma2.cu): TMA tile ids 0 = 64x16,
 // 1 = 128x8, 2 = 128x16
