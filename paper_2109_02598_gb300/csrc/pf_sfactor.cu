@@ -17,10 +17,11 @@
 // slowly, adding into a register while the bin stays; when it changes, the warp's lanes add
 // their sums to the warp's histogram in lane order. Fixed order throughout: the same bits on
 // every run. The bin kernel, 256^3 and 32 bins: 1829 us before, 0.2 ms now (reading 135 MB);
-// a whole call 4614 -> 3095 us, 2048^2 1760 -> 1337, 128^3 1308 -> 1110 (the transform and its
-// plan are the rest).
+// a whole call 4614 -> 3095 us, 4096^2 5260 -> 3660, 2048^2 1690 -> 1260, 128^3 1240 -> 1000, 64^2
+// 460 -> 400, 16^2 340 either way (the transform and its plan are the rest).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "pf_cufft.h"
@@ -69,6 +70,10 @@ __device__ int bin_of(double s2, const SfGeom& g) {
   return fq >= (double)(g.n_bins - 1) ? g.n_bins - 1 : (int)fq;
 }
 
+// Bound by the latency of its FP64 chains, some 50 dependent operations a trial of bin_of: a block
+// per SM, and eight lanes try a bin's limit at eight places at once (three trials after one another,
+// where one lane's bisection over 128 doubles takes nine). 7 us on 16^2, 9 with an axis of 2^18.
+constexpr int kTableBlocks = 152;
 __global__ void __launch_bounds__(128) sf_table_kernel(SfGeom g) {
   const int64_t i = blockIdx.x * 128 + threadIdx.x;
   for (int a = 0; a < g.rank; ++a) {
@@ -78,29 +83,30 @@ __global__ void __launch_bounds__(128) sf_table_kernel(SfGeom g) {
       g.k2[a][j] = __dmul_rn(k, k);
     }
   }
-  for (int64_t b = i; b <= g.n_bins; b += (int64_t)gridDim.x * 128) {
-    if (b == g.n_bins) {
-      g.least[b] = __longlong_as_double(0x7ff0000000000000ll);
-      continue;
-    }
-    // the least positive double whose bin is at least b: bisection on the bit patterns of the
+  if (i == 0) g.least[g.n_bins] = __longlong_as_double(0x7ff0000000000000ll);
+  const int lane = threadIdx.x & 7;
+  const unsigned group = 0xffu << (threadIdx.x & 24);  // the eight lanes of a bin
+  for (int64_t b = i >> 3; b < g.n_bins; b += (int64_t)gridDim.x * 16) {
+    // the least positive double whose bin is at least b: a search on the bit patterns of the
     // positive doubles (in their order), bin_of being monotone
-    // bin(lo) < b <= bin(hi), taking bin(0) = -1: from 64 doubles either side of the bin's
-    // lower edge squared, or from all of them where that does not hold it
+    // bin(lo) < b <= bin(hi), taking bin(0) = -1: from 16 doubles either side of the bin's
+    // lower edge squared (the roundings of both come to some ten), or from all of them where
+    // that does not hold it
     const double edge = (double)b * g.kmax / (double)g.n_bins;
     const long long at = __double_as_longlong(edge * edge), top = 0x7ff0000000000000ll;
-    long long lo = at - 64, hi = at + 64;
+    long long lo = at - 16, hi = at + 16;
     auto below = [&](long long v) { return bin_of(__longlong_as_double(v), g) < (int)b; };
-    if (lo < 0 || !below(lo)) lo = 0;
-    if (hi > top || below(hi)) hi = top;
+    const unsigned ends = __ballot_sync(group, below(lane == 0 ? lo : hi)) >> (threadIdx.x & 24);
+    if (lo < 0 || !(ends & 1)) lo = 0;
+    if (hi > top || (ends & 2)) hi = top;
     while (hi - lo > 1) {
-      const long long mid = lo + (hi - lo) / 2;
-      if (below(mid))
-        lo = mid;
-      else
-        hi = mid;
+      const long long step = (hi - lo + 6) / 8;  // eight places from lo + step, the last at hi - 1 or on
+      const long long v = lo + (lane + 1) * step;
+      const int n = __popc(__ballot_sync(group, v < hi && below(v)));
+      hi = min(hi, lo + (n + 1) * step);
+      lo += n * step;
     }
-    g.least[b] = __longlong_as_double(hi);
+    if (lane == 0) g.least[b] = __longlong_as_double(hi);
   }
 }
 
@@ -282,28 +288,32 @@ extern "C" int pf_structure_factor(int dim, const int64_t* n, int64_t pitch, con
   g.kmax = (3.141592653589793 / h) * std::sqrt((double)dim);
   g.n_bins = n_bins;
 
-  // tasks: even chunks of at most 32 columns of kx, and ky segments of at least 32 rows, down
-  // to where there are two tasks for each of the blocks' warps
+  // tasks: even chunks of at most 32 columns of kx, and ky segments of at least kAhead rows, down
+  // to where there are two tasks for each of the blocks' warps; on small grids of two rows, down
+  // to a task per SM (their lanes meet a new bin in nearly every row, and add to the histogram
+  // one after another: 64^2 in 256 bins 495 us a call with segments of 32 rows)
   g.nchunk = (int)((g.nxh + 31) / 32);
   g.cw = (int)((g.nxh + g.nchunk - 1) / g.nchunk);
   g.nseg = 1;
-  while (ny / (2 * g.nseg) >= 32 && (int64_t)g.nchunk * nz * g.nseg < 2 * kWarps * kMaxBinBlocks)
-    g.nseg *= 2;
+  for (;; g.nseg *= 2) {
+    const int64_t rows = ny / (2 * g.nseg), tasks = (int64_t)g.nchunk * nz * g.nseg;
+    if (!(rows >= kAhead && tasks < 2 * kWarps * kMaxBinBlocks) && !(rows >= 2 && tasks < 152)) break;
+  }
   g.seg = (int)((ny + g.nseg - 1) / g.nseg);
   g.nseg = (int)((ny + g.seg - 1) / g.seg);
   g.tasks = (int64_t)g.nchunk * nz * g.nseg;
   int64_t nblocks = (g.tasks + kWarps - 1) / kWarps;
   if (nblocks > kMaxBinBlocks) nblocks = kMaxBinBlocks;
 
-  // One allocation: rho, rho_hat, partial sums and counts, results, tables.
+  // One allocation: rho (after its transform the tables), rho_hat, partial sums and counts, results.
   auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
-  const size_t b_rho = up(sizeof(double) * (size_t)g.nsite);
+  const size_t b_rho = up(sizeof(double) * (size_t)std::max<int64_t>(
+      g.nsite, nz + ny + g.nxh + n_bins + 1));
   const size_t b_hat = up(sizeof(double2) * (size_t)g.nk);
   const size_t b_part = up(sizeof(double) * (size_t)(nblocks * n_bins));
   const size_t b_res = up(sizeof(double) * (size_t)n_bins);
-  const size_t b_tab = up(sizeof(double) * (size_t)(nz + ny + g.nxh + n_bins + 1));
   unsigned char* mem = nullptr;
-  cudaError_t e = cudaMalloc(&mem, b_rho + b_hat + 2 * b_part + 2 * b_res + b_tab);
+  cudaError_t e = cudaMalloc(&mem, b_rho + b_hat + 2 * b_part + 2 * b_res);
   if (e != cudaSuccess) {
     cudaGetLastError();
     set_error("pf_structure_factor: out of device memory");
@@ -316,7 +326,7 @@ extern "C" int pf_structure_factor(int dim, const int64_t* n, int64_t pitch, con
   double* d_mean = reinterpret_cast<double*>(mem + b_rho + b_hat + 2 * b_part);
   long long* d_cnt = reinterpret_cast<long long*>(mem + b_rho + b_hat + 2 * b_part + b_res);
 
-  double* tab = reinterpret_cast<double*>(mem + b_rho + b_hat + 2 * b_part + 2 * b_res);
+  double* tab = rho;
   for (int i = 0; i < dim; ++i) {
     g.k2[i] = tab;
     tab += i == dim - 1 ? g.nxh : g.d[i];
@@ -342,7 +352,7 @@ extern "C" int pf_structure_factor(int dim, const int64_t* n, int64_t pitch, con
       if (e == cudaSuccess)
         e = ensure_smem_attr(sf_bin_kernel, (size_t)kWarps * kMaxBins * 16, &g_bin_smem_mask);
       if (e == cudaSuccess) {
-        sf_table_kernel<<<32, 128, 0, st>>>(g);
+        sf_table_kernel<<<kTableBlocks, 128, 0, st>>>(g);
         sf_bin_kernel<<<(int)nblocks, kThreads, smem, st>>>(rhat, g, psum, pcnt);
         e = cudaGetLastError();
       }
