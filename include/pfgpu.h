@@ -317,7 +317,8 @@ int pf_batch_info(pf_batch_t b, int64_t* sites, int64_t* bytes_per_copy);
  * they fit, with those the device's other grids store this way, 4 GiB, and a sixteenth of the
  * memory that is free; else C = ceil(sqrt(n_steps)), i.e.
  * sqrt(N) checkpointing of the time loop of Sec. 2.4.1. The gradients do not depend on C.
- * Allocates the checkpoints (ceil(N/C) states), a segment's states between them and the adjoint
+ * Allocates the checkpoints (ceil(N/C) states), a segment's states between them (at an interval of
+ * the caller's two segments', where they fit) and the adjoint
  * buffers on first use.
  * Errors: PF_ERR_STATE (no Gray-Scott model), PF_ERR_INVALID_ARG (3D grid, n < 1),
  * PF_ERR_OOM, PF_ERR_CUDA. */

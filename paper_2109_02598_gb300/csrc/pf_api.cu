@@ -505,6 +505,7 @@ void pf_destroy(pf_grid_t g) {
   pf::fe2d_bands_release(g);
   drop_graphs(g);
   if (g->capture) cudaStreamDestroy(g->capture);
+  if (g->branch) cudaStreamDestroy(g->branch);
   if (g->base) cudaFree(g->base);
   if (g->red_host) cudaFreeHost(g->red_host);
   g->magic = 0;

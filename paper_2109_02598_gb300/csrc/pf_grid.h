@@ -97,7 +97,8 @@ struct AdjointState {
   int model = -1;            // the recorded forward pass's model
   float* ckpt = nullptr;     // n_ckpt * nf * field_elems floats
   float* seg = nullptr;      // a segment's recomputed states: the first of each block of
-                             // reverse steps but the segment's own first
+                             // reverse steps but the segment's own first; twice (seg_bufs) at
+  int seg_bufs = 0;          // an interval of the caller's, where there is the memory for it
   float* lam = nullptr;      // 2 * nf * field_elems floats: adjoint ping-pong; and behind them
   double* gpart = nullptr;   //   per-CTA parameter-gradient partials (4 per CTA)
   double* gout = nullptr;    //   and the 4 final sums
@@ -157,6 +158,7 @@ struct pf_grid_s {
   // CUDA-graph cache of pf_step: a few recorded launch sequences, keyed by
   // (steps, tile, k, starting buffer), least recently used replaced first
   cudaStream_t capture = nullptr;  // private stream used only to record graphs
+  cudaStream_t branch = nullptr;   // second branch of the adjoint's reverse pass
   struct StepGraph {
     cudaGraphExec_t exec = nullptr;
     int64_t steps = -1;
