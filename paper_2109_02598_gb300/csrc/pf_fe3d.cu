@@ -17,19 +17,20 @@ constexpr int kNT3 = 256;
 template <int MODEL, int TX, int TY>
 struct Cfg3 {
   static constexpr int NF = ModelTraits<MODEL>::NF;
-  static constexpr int R = ModelTraits<MODEL>::R;
+  static constexpr int R = 2;
+  static_assert(ModelTraits<MODEL>::R == R, "Models B and C");
   // phi planes (halo R)
   static constexpr int W = TX + 2 * R;
   static constexpr int HT = TY + 2 * R;
   static constexpr int PL = W * HT;
-  // mu planes (Model B only, halo 1)
+  // mu planes (halo 1)
   static constexpr int W1 = TX + 2;
   static constexpr int HT1 = TY + 2;
   static constexpr int PL1 = W1 * HT1;
   // ring of phi planes: three (z-1, z, z+1), four for Model C, whose psi needs plane z-1
   // while plane z+2 is already staged for the chemical potential of m
   static constexpr int NPH = (MODEL == PF_MODEL_C) ? 4 : 3;
-  static constexpr int SMEM_FLOATS = NPH * NF * PL + (R == 2 ? 3 * PL1 : 0);
+  static constexpr int SMEM_FLOATS = NPH * NF * PL + 3 * PL1;
 };
 
 // Stage plane z (periodic) of every field into ring slot `slot`: 4-byte cp.async copies (the
@@ -52,31 +53,27 @@ __device__ __forceinline__ void load_plane3d(const FieldPtrs& in, const Geom& g,
 }
 
 // 3D Laplacian at position p of a staged plane c (row width W) with the planes b below and
-// a above: 7-point (ST = PF_ST_STD), isotropic 19-point (faces and edges, PF_ST_ISO) or
-// isotropic 27-point (faces, edges and corners, PF_ST_ISO27).
+// a above: isotropic 19-point (faces and edges, PF_ST_ISO) or isotropic 27-point (faces, edges
+// and corners, PF_ST_ISO27).
 template <int ST>
 __device__ __forceinline__ float lap3d_planes(const float* b, const float* c, const float* a,
                                               int p, int W, float scale) {
-  if constexpr (ST == PF_ST_STD) {
-    return lap3d(c[p], c[p - 1], c[p + 1], c[p - W], c[p + W], b[p], a[p], scale);
+  const float faces = __fadd_rn(__fadd_rn(__fadd_rn(c[p - 1], c[p + 1]),
+                                          __fadd_rn(c[p - W], c[p + W])),
+                                __fadd_rn(b[p], a[p]));
+  const float exy = __fadd_rn(__fadd_rn(c[p - W - 1], c[p - W + 1]),
+                              __fadd_rn(c[p + W - 1], c[p + W + 1]));
+  const float eb = __fadd_rn(__fadd_rn(b[p - 1], b[p + 1]), __fadd_rn(b[p - W], b[p + W]));
+  const float ea = __fadd_rn(__fadd_rn(a[p - 1], a[p + 1]), __fadd_rn(a[p - W], a[p + W]));
+  const float edges = __fadd_rn(exy, __fadd_rn(eb, ea));
+  if constexpr (ST == PF_ST_ISO) {
+    return lap3d_iso(c[p], faces, edges, scale);
   } else {
-    const float faces = __fadd_rn(__fadd_rn(__fadd_rn(c[p - 1], c[p + 1]),
-                                            __fadd_rn(c[p - W], c[p + W])),
-                                  __fadd_rn(b[p], a[p]));
-    const float exy = __fadd_rn(__fadd_rn(c[p - W - 1], c[p - W + 1]),
-                                __fadd_rn(c[p + W - 1], c[p + W + 1]));
-    const float eb = __fadd_rn(__fadd_rn(b[p - 1], b[p + 1]), __fadd_rn(b[p - W], b[p + W]));
-    const float ea = __fadd_rn(__fadd_rn(a[p - 1], a[p + 1]), __fadd_rn(a[p - W], a[p + W]));
-    const float edges = __fadd_rn(exy, __fadd_rn(eb, ea));
-    if constexpr (ST == PF_ST_ISO) {
-      return lap3d_iso(c[p], faces, edges, scale);
-    } else {
-      const float cb = __fadd_rn(__fadd_rn(b[p - W - 1], b[p - W + 1]),
-                                 __fadd_rn(b[p + W - 1], b[p + W + 1]));
-      const float ca = __fadd_rn(__fadd_rn(a[p - W - 1], a[p - W + 1]),
-                                 __fadd_rn(a[p + W - 1], a[p + W + 1]));
-      return lap3d_iso27(c[p], faces, edges, __fadd_rn(cb, ca), scale);
-    }
+    const float cb = __fadd_rn(__fadd_rn(b[p - W - 1], b[p - W + 1]),
+                               __fadd_rn(b[p + W - 1], b[p + W + 1]));
+    const float ca = __fadd_rn(__fadd_rn(a[p - W - 1], a[p - W + 1]),
+                               __fadd_rn(a[p + W - 1], a[p + W + 1]));
+    return lap3d_iso27(c[p], faces, edges, __fadd_rn(cb, ca), scale);
   }
 }
 
