@@ -156,8 +156,9 @@ int pf_read_field_host_async(pf_grid_t g, int field, float* dst);
  * PF_ERR_CUDA. */
 int pf_step(pf_grid_t g, int64_t n_steps);
 
-/* Deterministic reduction of the current state into *out (see PF_REDUCE_*): warp
- * shuffles to per-block partial sums in FP64, then one fixed-order FP64 sum.
+/* Deterministic reduction of the current state into *out (see PF_REDUCE_*), to FP64 accuracy site
+ * by site: error-free FP32 sums per thread (energies of fewer than 2^16 sites: FP64), then FP64 sums
+ * in a fixed order.
  *   PF_REDUCE_MASS    h^d sum_x phi_x of field `field` (the conserved quantity of Model B,
  *                     Sec. 3, and of Model C's m);
  *   PF_REDUCE_ENERGY  the discrete free energy (the paper does not write one out; the reading
@@ -315,8 +316,9 @@ int pf_batch_info(pf_batch_t b, int64_t* sites, int64_t* bytes_per_copy);
  * pf_step, storing the state every ckpt_interval steps. 0 leaves the interval C to the library:
  * the states the reverse pass starts its launches from (every 4th, for Model B every 2nd) where
  * they fit, with those the device's other grids store this way, 4 GiB, and a sixteenth of the
- * memory that is free; else C = ceil(sqrt(n_steps)), i.e.
- * sqrt(N) checkpointing of the time loop of Sec. 2.4.1. The gradients do not depend on C.
+ * memory that is free (asked again with the same arguments, a grid keeps its schedule); else
+ * C = ceil(sqrt(n_steps)), i.e. sqrt(N) checkpointing of the time loop of Sec. 2.4.1. The
+ * gradients do not depend on C.
  * Allocates the checkpoints (ceil(N/C) states), a segment's states between them (at an interval of
  * the caller's two segments', where they fit) and the adjoint
  * buffers on first use.

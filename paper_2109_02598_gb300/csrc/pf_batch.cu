@@ -162,8 +162,9 @@ static cudaError_t batch_strips(pf_batch_s* b, int t, int k) {
     nstrips[i] = (int)((b->nx[i] + w - 1) / w);
     strip_rows_total += (int64_t)nstrips[i] * b->ny[i];
   }
-  // candidate heights: from the floor up, skipping those whose lists would be too long to
-  // play through cheaply (a list of a few million tasks is past every tail effect anyway)
+  // candidate heights: from 4 rows where the list fits two waves of warps, else from the floor,
+  // skipping those whose lists would be too long to play through cheaply (a list of a few million
+  // tasks is past every tail effect anyway)
   const int resident = batch_gs2d_strips_resident(k, c);
   const int floor_rows = strip_task_rows(PF_MODEL_GS, k);
   int hy = 0, dev = 0, sms = 0;

@@ -417,7 +417,7 @@ __global__ void __launch_bounds__(kStripThreads, (StripCfg<PF_MODEL_GS, K, C>::M
   }
 }
 
-// Rows per task: the height that makes the launch shortest by waves * (rows + T0) * (100 + w), w
+// Rows per task: the height that makes the launch shortest by waves * (rows + T0) * (40 + w), w
 // the warps per SM of a wave. A task takes T0 iterations beside its rows, and an iteration is
 // half latency: its time grows with the resident warps only as 40 + w (timed over 16 heights, all
 // four models at their greatest depth, both widths, 512^2 to 4096^2: its choice is within 2 % of
@@ -543,7 +543,8 @@ int strip_out_cols(int model, int k, int c) {
   return 0;
 }
 
-// The shortest batch task considered: twice the levels' start-up.
+// The shortest batch task considered where the list is longer than two waves of warps: twice the
+// levels' start-up.
 int strip_task_rows(int model, int k) {
   const int r = (model == PF_MODEL_CH || model == PF_MODEL_C) ? 2 : 1;
   return 2 * (2 * r + 1) * k;

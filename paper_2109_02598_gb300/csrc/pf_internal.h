@@ -183,7 +183,7 @@ struct BatchStrip {
   short hy, wo;
 };
 int strip_out_cols(int model, int k, int c);  // output columns of a strip of 32 c columns
-int strip_task_rows(int model, int k);        // fewest rows per batch strip task
+int strip_task_rows(int model, int k);        // fewest rows of a batch strip task of long lists
 int batch_gs2d_strips_resident(int k, int c);  // warps of the batch strip kernel on the device
 cudaError_t launch_batch_gs2d_strips(int c, int k, const BatchInst* d_insts,
                                      const BatchStrip* d_tasks, int ntasks, const float* in_base,
